@@ -59,7 +59,8 @@ def work_of(wl, C=1):
     """Algorithmic FLOPs / bytes per launch site for one call over C candidates (GEMM = 2MNK;
     causal attention counts the lower triangle including the diagonal; backward attention = 2.5x
     forward; the KL term's two score products = the forward's two products; no dX GEMM). The
-    quantiser reads W (2 B) and writes the fp16 operand (2 B) per weight, per candidate."""
+    preparation reads X and W once (2 B each) and writes their fp16 operands (2 B), W's per candidate
+    (a fit step on a prepared X leaves X out)."""
     s = wl.shape
     N, D, d = wl.batch * wl.seq_len, s.d_out, s.d_model
     attn = 4.0 * wl.batch * s.n_q_heads * s.head_dim * wl.seq_len * (wl.seq_len + 1) / 2
@@ -71,8 +72,7 @@ def work_of(wl, C=1):
         "wgrad_lsq": ("flop", 2.0 * N * D * d),
         "wgrad_store": ("flop", 2.0 * N * D * d),
         "attn_jvp": ("flop", 2.5 * attn * C),
-        "convert_x": ("byte", 4.0 * N * d),
-        "quantize": ("byte", 4.0 * D * d * C),
+        "prep": ("byte", 4.0 * N * d + 2.0 * D * d * (1 + C)),  # X, W -> fp16 operands
         "probe": ("byte", 2.0 * D * d * C),
     }
 
@@ -468,8 +468,7 @@ def wl_table(J, wl, args, dev, pk, st, with_cpu):
     hw = {"proj_gemm": ("flop", w1["proj_gemm"][1] * nbh * (2 + m)),
           "attn_fwd": ("flop", w1["attn_fwd"][1] * nbh),
           "attn_jvp": ("flop", w1["attn_jvp"][1] * nbh * m),
-          "convert_x": ("byte", w1["convert_x"][1] * nbh * 2),
-          "quantize": ("byte", w1["quantize"][1] * nbh * 2),
+          "prep": ("byte", w1["prep"][1] * nbh * 2),
           "probe": ("byte", w1["probe"][1] * nbh * m)}
     hflops = hw["proj_gemm"][1] + hw["attn_fwd"][1] + hw["attn_jvp"][1]
     out["hutchinson"] = {

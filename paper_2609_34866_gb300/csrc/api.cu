@@ -2,6 +2,7 @@
 // Every step of the computation runs in the kernels of this library; there is no host fallback.
 #include <math.h>
 
+#include <algorithm>
 #include <cmath>
 #include <stdlib.h>
 #include <string.h>
@@ -155,13 +156,38 @@ bool is_prepared(const void* ws, const void* x, int32_t B, int32_t T, int32_t d)
   return false;
 }
 
-// X (bf16) -> the workspace's fp16 copy, with the fp16 range check; records it for *_prepared.
-jab_status convert_x_into(const jab_block_desc* desc, int32_t B, int32_t T, const void* X_dev,
-                          void* ws, const Workspace& wp, int* status, int sms, cudaStream_t st) {
-  const int64_t N = (int64_t)B * T;
-  JAB_SITE("convert_x", 1, launch_convert_x(X_dev, static_cast<char*>(ws) + wp.x16,
-                                            N * desc->d_model, status, sms, st));
-  note_prepared(ws, X_dev, B, T, desc->d_model);
+// X in fp16 (unless the workspace holds it: x_prepared), the fp16 operand of every candidate (n_cand
+// = 0: W itself; W_dev null: none) and the RoPE table, in one launch. Records X for *_prepared.
+jab_status prepare_inputs(const jab_block_desc* desc, int32_t B, int32_t T, const void* X_dev,
+                          bool x_prepared, const void* W_dev, int n_cand,
+                          const float* const* scales, const int32_t* bits, void* ws,
+                          const Workspace& wp, int* status, int sms, cudaStream_t st) {
+  char* w = static_cast<char*>(ws);
+  PrepInputs in{};
+  if (!x_prepared) {
+    in.x = X_dev;
+    in.xh = w + wp.x16;
+    in.nx = (int64_t)B * T * desc->d_model;
+  }
+  in.D = (int)block_rows(desc);
+  in.d = desc->d_model;
+  in.G = desc->group_size;
+  if (W_dev != nullptr) {
+    in.w = W_dev;
+    in.w16 = w + wp.w16;
+    in.ncand = n_cand;
+    in.s = scales;
+    in.bits = bits;
+    if (desc->use_rope) {
+      in.cos_t = reinterpret_cast<float*>(w + wp.rope);
+      in.sin_t = in.cos_t + (int64_t)T * (desc->head_dim / 2);
+      in.T = T;
+      in.dh = desc->head_dim;
+      in.theta = desc->rope_theta;
+    }
+  }
+  JAB_SITE("prep", std::max(1, (n_cand + 7) / 8), launch_prep(in, status, sms, st));
+  if (!x_prepared) note_prepared(ws, X_dev, B, T, desc->d_model);
   return JAB_OK;
 }
 
@@ -197,13 +223,12 @@ jab_status jab_reference_forward(const jab_block_desc* desc, int32_t B, int32_t 
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
   const int64_t N = (int64_t)B * T;
-  const int D = (int)block_rows(desc), dm = desc->d_model, dh = desc->head_dim;
+  const int D = (int)block_rows(desc), dh = desc->head_dim;
   float* cos_t = reinterpret_cast<float*>(w + wp.rope);
   float* sin_t = cos_t + (int64_t)T * (dh / 2);
-  if ((s = convert_x_into(desc, B, T, X_dev, ws, wp, status, sms, st)) != JAB_OK) return s;
-  JAB_SITE("quantize", 1, launch_quantize(W_dev, nullptr, D, dm, desc->group_size, 0, w + wp.w16, nullptr, nullptr,
-                          status, sms, st));
-  if (desc->use_rope) JAB_SITE("rope_table", 1, launch_rope_table(T, dh, desc->rope_theta, cos_t, sin_t, st));
+  if ((s = prepare_inputs(desc, B, T, X_dev, false, W_dev, 0, nullptr, nullptr, ws, wp, status, sms,
+                          st)) != JAB_OK)
+    return s;
   if ((s = run_projection(desc, N, T, 1, w + wp.x16, w + wp.w16, w + wp.qkv, cos_t, sin_t, status, st)) !=
       JAB_OK)
     return s;
@@ -249,14 +274,12 @@ static jab_status forward_candidates(const jab_block_desc* desc, int32_t B, int3
   if ((s = device_info(&status, &sms)) != JAB_OK) return s;
   char* w = static_cast<char*>(ws);
   const int64_t N = (int64_t)B * T;
-  const int D = (int)block_rows(desc), dm = desc->d_model, dh = desc->head_dim;
+  const int D = (int)block_rows(desc), dh = desc->head_dim;
   float* cos_t = reinterpret_cast<float*>(w + wp.rope);
   float* sin_t = cos_t + (int64_t)T * (dh / 2);
-  if ((s = convert_x_into(desc, B, T, X_dev, ws, wp, status, sms, st)) != JAB_OK) return s;
-  for (int c = 0; c < n_cand; ++c)
-    JAB_SITE("quantize", 1, launch_quantize(W_dev, scales_host[c], D, dm, desc->group_size, bits_host[c],
-                            w + wp.w16 + (size_t)c * D * dm * 2, nullptr, nullptr, status, sms, st));
-  if (desc->use_rope) JAB_SITE("rope_table", 1, launch_rope_table(T, dh, desc->rope_theta, cos_t, sin_t, st));
+  if ((s = prepare_inputs(desc, B, T, X_dev, false, W_dev, n_cand, scales_host, bits_host, ws, wp,
+                          status, sms, st)) != JAB_OK)
+    return s;
   if ((s = run_projection(desc, N, T, n_cand, w + wp.x16, w + wp.w16, w + wp.qkv, cos_t, sin_t,
                           status, st)) != JAB_OK)
     return s;
@@ -303,13 +326,12 @@ jab_status jab_reference_projection(const jab_block_desc* desc, int32_t B, int32
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
   const int64_t N = (int64_t)B * T;
-  const int D = (int)block_rows(desc), dm = desc->d_model, dh = desc->head_dim;
+  const int D = (int)block_rows(desc), dh = desc->head_dim;
   float* cos_t = reinterpret_cast<float*>(w + wp.rope);
   float* sin_t = cos_t + (int64_t)T * (dh / 2);
-  if ((s = convert_x_into(desc, B, T, X_dev, ws, wp, status, sms, st)) != JAB_OK) return s;
-  JAB_SITE("quantize", 1, launch_quantize(W_dev, nullptr, D, dm, desc->group_size, 0, w + wp.w16,
-                                          nullptr, nullptr, status, sms, st));
-  if (desc->use_rope) JAB_SITE("rope_table", 1, launch_rope_table(T, dh, desc->rope_theta, cos_t, sin_t, st));
+  if ((s = prepare_inputs(desc, B, T, X_dev, false, W_dev, 0, nullptr, nullptr, ws, wp, status, sms,
+                          st)) != JAB_OK)
+    return s;
   return run_projection(desc, N, T, 1, w + wp.x16, w + wp.w16, QKV_ref_dev, cos_t, sin_t, status,
                         st);
 }
@@ -382,10 +404,9 @@ jab_status jab_hutchinson_trace(const jab_block_desc* desc, int32_t B, int32_t T
   double* tmp = reinterpret_cast<double*>(w + wp.scal);
   const int nP = (T + attn_jvp_tc_rows() - 1) / attn_jvp_tc_rows();
   const double n_el = (double)N * desc->n_q_heads * dh;
-  if ((s = convert_x_into(desc, B, T, X_dev, ws, wp, status, sms, st)) != JAB_OK) return s;
-  JAB_SITE("quantize", 1, launch_quantize(W_dev, nullptr, D, dm, desc->group_size, 0, w + wp.w16,
-                                          nullptr, nullptr, status, sms, st));
-  if (desc->use_rope) JAB_SITE("rope_table", 1, launch_rope_table(T, dh, desc->rope_theta, cos_t, sin_t, st));
+  if ((s = prepare_inputs(desc, B, T, X_dev, false, W_dev, 0, nullptr, nullptr, ws, wp, status, sms,
+                          st)) != JAB_OK)
+    return s;
   if ((s = run_projection(desc, N, T, 1, w + wp.x16, w + wp.w16, qkv, cos_t, sin_t, status, st)) !=
       JAB_OK)
     return s;
@@ -496,17 +517,13 @@ static jab_status backward_to_dqkvt(const jab_block_desc* desc, int32_t B, int32
   char* w = static_cast<char*>(ws);
   const int64_t N = (int64_t)B * T;
   const int D = (int)block_rows(desc), dm = desc->d_model, dh = desc->head_dim;
-  const int G = desc->group_size;
   float* cos_t = reinterpret_cast<float*>(w + wp.rope);
   float* sin_t = cos_t + (int64_t)T * (dh / 2);
-  if (x_prepared) {  // the workspace already holds this X in fp16 (jab_prepare_x)
-    if (!is_prepared(ws, X_dev, B, T, dm)) return JAB_ERR_INVALID_ARG;
-  } else if ((s = convert_x_into(desc, B, T, X_dev, ws, wp, status, sms, st)) != JAB_OK) {
+  // with x_prepared the workspace already holds this X in fp16 (jab_prepare_x)
+  if (x_prepared && !is_prepared(ws, X_dev, B, T, dm)) return JAB_ERR_INVALID_ARG;
+  if ((s = prepare_inputs(desc, B, T, X_dev, x_prepared, W_dev, 1, &scales_dev, &bits, ws, wp, status,
+                          sms, st)) != JAB_OK)
     return s;
-  }
-  JAB_SITE("quantize", 1, launch_quantize(W_dev, scales_dev, D, dm, G, bits, w + wp.w16, nullptr, nullptr, status,
-                          sms, st));
-  if (desc->use_rope) JAB_SITE("rope_table", 1, launch_rope_table(T, dh, desc->rope_theta, cos_t, sin_t, st));
   if ((s = run_projection(desc, N, T, 1, w + wp.x16, w + wp.w16, w + wp.qkv, cos_t, sin_t, status, st)) !=
       JAB_OK)
     return s;
@@ -602,7 +619,7 @@ jab_status jab_prepare_x(const jab_block_desc* desc, int32_t B, int32_t T, const
   int* status;
   int sms;
   if ((s = device_info(&status, &sms)) != JAB_OK) return s;
-  return convert_x_into(desc, B, T, X_dev, ws, wp, status, sms,
+  return prepare_inputs(desc, B, T, X_dev, false, nullptr, 0, nullptr, nullptr, ws, wp, status, sms,
                         reinterpret_cast<cudaStream_t>(stream));
 }
 
@@ -695,7 +712,7 @@ jab_status jab_quantize(const jab_block_desc* desc, int32_t bits, const void* W_
   int sms;
   if ((s = device_info(&status, &sms)) != JAB_OK) return s;
   JAB_TRY(launch_quantize(W_dev, scales_dev, (int)block_rows(desc), desc->d_model,
-                          desc->group_size, bits, nullptr, codes_dev, w_hat_dev, status, sms,
+                          desc->group_size, bits, codes_dev, w_hat_dev, status, sms,
                           reinterpret_cast<cudaStream_t>(stream)));
   return JAB_OK;
 }

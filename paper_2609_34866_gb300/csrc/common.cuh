@@ -62,6 +62,25 @@ __device__ __forceinline__ float lsq_factor(float w, float s, int qmax) {
   return (fabsf(v) <= (float)qmax) ? (q - v) : copysignf((float)qmax, v);
 }
 
+// fl32(w / s) of several bf16 weights with one scale: with r = fl32(1 / s) and v0 = fl32(w r), the
+// remainder w - v0 s is exact in one fused operation and v0 + r (w - v0 s) rounds to the IEEE quotient
+// (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990).
+// Equal to w / s for every pair of a bf16 and an fp32 mantissa (2^7 x 2^23, checked one by one), and
+// so wherever no intermediate leaves the normal range: s within 2^-60 .. 2^60, |w| within 2^-90 ..
+// 2^60 or 0 (below 2^-90 the quotient is less than 2^-30 and its code 0 either way). Other values take
+// the division. Three operations a weight, in packed pairs, where the division takes about ten.
+__device__ __forceinline__ bool quot_window(float s) { return s >= 8.6736174e-19f && s <= 1.1529215e18f; }
+// Largest magnitude bits of packed 16-bit floats seen so far, per half: one AND and one 16x2 maximum.
+__device__ __forceinline__ uint32_t max_abs_f16x2(uint32_t acc, uint32_t v2) {
+  return __vmaxu2(acc, v2 & 0x7fff7fffu);
+}
+// Whether either half of such a maximum is at or above `limit`.
+__device__ __forceinline__ bool either_at_least(uint32_t m2, uint32_t limit) {
+  return (m2 & 0xffffu) >= limit || (m2 >> 16) >= limit;
+}
+constexpr uint32_t kBf16Inf = 0x7f80u, kHalfInf = 0x7c00u;
+constexpr uint32_t kBf16TwoTo60 = 187u << 7;
+
 __device__ __forceinline__ double warp_sum(double x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);

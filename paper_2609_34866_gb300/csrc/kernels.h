@@ -26,15 +26,31 @@ struct AttnLaunch {
 };
 
 // prep.cu
-cudaError_t launch_convert_x(const void* x, void* xh, int64_t n, int* status, int sms, cudaStream_t st);
-cudaError_t launch_quantize(const void* w, const float* s, int D, int d, int G, int bits, void* w16,
+// What a projection needs besides W as stored, prepared by one launch: X in fp16 (x null: it is there
+// already), every candidate's fp16 w_hat (ncand = 0: W itself; w null: none) and the RoPE table (cos_t
+// null: none).
+struct PrepInputs {
+  const void* x;
+  void* xh;
+  int64_t nx;  // elements of X
+  const void* w;
+  void* w16;
+  int ncand;
+  const float* const* s;  // host arrays [ncand]
+  const int32_t* bits;
+  int D, d, G;
+  float *cos_t, *sin_t;
+  int T, dh;
+  float theta;
+};
+cudaError_t launch_prep(const PrepInputs& in, int* status, int sms, cudaStream_t st);
+cudaError_t launch_quantize(const void* w, const float* s, int D, int d, int G, int bits,
                             int8_t* codes, float* w_hat32, int* status, int sms, cudaStream_t st);
 // codes a, b: int8 [n], 16-byte aligned; *count (int64, device) = #{i : a[i] != b[i]}
 cudaError_t launch_flip_count(const int8_t* a, const int8_t* b, int64_t n, int64_t* count,
                               int sms, cudaStream_t st);
 cudaError_t launch_init_scales(const void* w, int D, int d, int G, int bits, int mode, float* s_out,
                                cudaStream_t st);
-cudaError_t launch_rope_table(int T, int dh, double theta, float* cos_t, float* sin_t, cudaStream_t st);
 
 // gemm_tc.cu
 cudaError_t launch_proj_gemm_tc(const void* A, const void* Bw, void* C, int64_t M, int Nn, int K,

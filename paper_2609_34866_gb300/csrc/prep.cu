@@ -1,88 +1,260 @@
-// Elementwise and small kernels of the L_JAB path: X conversion, the quantiser (Eq. 2), scale
-// initialisation, the RoPE table. All are HBM-bound: 16-byte vector loads and stores, grids sized
-// in multiples of the SM count.
+// Elementwise and small kernels of the L_JAB path: X conversion, the quantiser (Eq. 2) and the RoPE
+// table in one launch, the quantiser alone, scale initialisation, probes, sums over the weights.
+// 16-byte vector loads and stores, grids sized in multiples of the SM count.
+#include <math.h>
+
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "tc.cuh"
 
 namespace jab {
 
+// Arguments of prep_kernel (a part that is not wanted has no blocks).
+struct PrepArgs {
+  static constexpr int kMaxCand = 8;  // candidates of one launch
+  int nrope, nw, nx;                  // blocks of the RoPE table, the weights and X
+  const uint4* x;
+  uint4* xh;
+  int64_t n8x;
+  const uint4* w;
+  uint4* w16;  // [ncand, D, d] fp16
+  const float* s[kMaxCand];
+  int bits[kMaxCand];
+  int ncand, D, d, G;
+  float *cos_t, *sin_t;
+  int T, half;
+  double freq_pi[64];  // theta^(-j / half) / pi
+  int* status;
+};
+
 // ---------------------------------------------------------------- X: bf16 -> fp16 (+ range check)
-__global__ void convert_x_kernel(const uint4* __restrict__ x, uint4* __restrict__ xh, int64_t n8,
-                                 int* status) {
-  int bad = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    uint4 v = __ldg(x + i);
-    const bf16_t* b = reinterpret_cast<const bf16_t*>(&v);
-    uint4 o;
-    half_t* h = reinterpret_cast<half_t*>(&o);
+// 8 bf16 as fp16; the largest magnitudes before and after, for the finiteness and range checks.
+__device__ __forceinline__ uint4 convert8(const uint4& v, uint32_t& in, uint32_t& out) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  uint4 o;
+  uint32_t* u = reinterpret_cast<uint32_t*>(&o);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float f = __bfloat162float(b[k]);
-      h[k] = __float2half_rn(f);
-      if (!isfinite(f)) bad |= 2;
-      else if (__hisinf(h[k])) bad |= 1;
-    }
-    xh[i] = o;
+  for (int k = 0; k < 4; ++k) {
+    u[k] = tc::pack_half2(__uint_as_float(w[k] << 16), __uint_as_float(w[k] & 0xffff0000u));
+    in = max_abs_f16x2(in, w[k]);
+    out = max_abs_f16x2(out, u[k]);
   }
-  if (bad & 2) report(status, JAB_ERR_NONFINITE);
-  else if (bad & 1) report(status, JAB_ERR_RANGE);
+  return o;
+}
+
+// Block `blk` of `nblk`: four 16-byte loads of a thread in flight at a time.
+__device__ __forceinline__ void convert_x_role(const uint4* __restrict__ x, uint4* __restrict__ xh,
+                                               int64_t n8, int blk, int nblk, int* status) {
+  uint32_t in = 0, out = 0;
+  const int64_t step = (int64_t)nblk * blockDim.x;
+  int64_t i = (int64_t)blk * blockDim.x + threadIdx.x;
+  for (; i + 3 * step < n8; i += 4 * step) {
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = __ldg(x + i + u * step);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) xh[i + u * step] = convert8(v[u], in, out);
+  }
+  for (; i < n8; i += step) xh[i] = convert8(__ldg(x + i), in, out);
+  if (either_at_least(in, kBf16Inf)) report(status, JAB_ERR_NONFINITE);
+  else if (either_at_least(out, kHalfInf)) report(status, JAB_ERR_RANGE);
 }
 
 // ---------------------------------------------------------------- quantiser (Section 2.1, Eq. 2)
-// bits == 0: plain bf16 -> fp16 conversion of W (the teacher's weights).
-__global__ void quantize_kernel(const uint4* __restrict__ w, const float* __restrict__ s, int D,
-                                int d, int G, int bits, uint4* __restrict__ w16,
-                                int8_t* __restrict__ codes, float* __restrict__ w_hat32,
-                                int* status) {
-  const int64_t n8 = (int64_t)D * d / 8;
-  const int qmax = bits > 0 ? qmax_of(bits) : 0;
-  const int ng = d / G;
-  int bad = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    uint4 v = __ldg(w + i);
-    const bf16_t* b = reinterpret_cast<const bf16_t*>(&v);
-    const int64_t e0 = i * 8;
-    const int64_t row = e0 / d;
-    const int col = (int)(e0 - row * d);
-    float out[8];
-    if (bits == 0) {
+// Codes of 8 weights that share a scale, as floats: clip(rint(fl32(w / s))).
+__device__ __forceinline__ void quant_codes8(const uint4& v, float sc, int qmax, float (&q)[8]) {
+  const uint32_t w2[4] = {v.x, v.y, v.z, v.w};
+  const bf16_t* b = reinterpret_cast<const bf16_t*>(&v);
+  uint32_t big = 0;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) out[k] = __bfloat162float(b[k]);
-    } else {
-      float sc = __ldg(s + row * ng + col / G);
-      if (!(sc > 0.f) || !isfinite(sc)) {  // reading: scales must be finite and > 0
-        bad = 1;
-        sc = 1.f;
-      }
-      char cq[8];
+  for (int k = 0; k < 4; ++k) big = max_abs_f16x2(big, w2[k]);
+  if (quot_window(sc) && !either_at_least(big, kBf16TwoTo60)) {
+    const float r = __frcp_rn(sc), qm = (float)qmax;
+    const float2 r2 = make_float2(r, r), ns2 = make_float2(-sc, -sc);
+    const float2 magic = make_float2(12582912.f, 12582912.f);  // 1.5 * 2^23: rounds half to even
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const float q = quant_code(__bfloat162float(b[k]), sc, qmax, nullptr);
-        cq[k] = (char)(int)q;
-        out[k] = __fmul_rn(q, sc);
-      }
-      if (codes) *reinterpret_cast<uint2*>(codes + e0) = *reinterpret_cast<uint2*>(cq);
-      if (w_hat32) {
-        reinterpret_cast<float4*>(w_hat32 + e0)[0] = make_float4(out[0], out[1], out[2], out[3]);
-        reinterpret_cast<float4*>(w_hat32 + e0)[1] = make_float4(out[4], out[5], out[6], out[7]);
-      }
+    for (int k = 0; k < 4; ++k) {
+      const float2 w = make_float2(__uint_as_float(w2[k] << 16), __uint_as_float(w2[k] & 0xffff0000u));
+      const float2 v0 = tc::mul2(w, r2);
+      float2 t = tc::fma2(tc::fma2(v0, ns2, w), r2, v0);
+      t.x = fminf(fmaxf(t.x, -qm), qm);  // qmax is whole: clipping before rounding is the same
+      t.y = fminf(fmaxf(t.y, -qm), qm);
+      const float2 c = tc::sub2(tc::add2(t, magic), magic);
+      q[2 * k] = c.x;
+      q[2 * k + 1] = c.y;
     }
-    if (w16) {
-      uint4 o;
-      half_t* h = reinterpret_cast<half_t*>(&o);
+  } else {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        h[k] = __float2half_rn(out[k]);
-        if (__hisinf(h[k]) || __hisnan(h[k])) bad |= 2;  // not representable as an fp16 operand
+    for (int k = 0; k < 8; ++k) q[k] = quant_code(__bfloat162float(b[k]), sc, qmax, nullptr);
+  }
+}
+
+// The scale of 8-weight chunk i is number i / (G / 8), as G divides the row length. Walks that quotient
+// along a grid-stride loop by additions: an integer division per chunk costs as much as its codes.
+struct GroupWalk {
+  int64_t g;       // quotient
+  int r;           // remainder
+  int64_t dg;      // steps of both
+  int dr, g8;
+  __device__ __forceinline__ GroupWalk(int64_t i, int64_t step, int g8_) : g8(g8_) {
+    g = i / g8;
+    r = (int)(i - g * g8);
+    dg = step / g8;
+    dr = (int)(step - dg * g8);
+  }
+  __device__ __forceinline__ int64_t next() {  // the quotient at i, then on to i + step
+    const int64_t now = g;
+    g += dg;
+    r += dr;
+    if (r >= g8) {
+      r -= g8;
+      ++g;
+    }
+    return now;
+  }
+};
+
+// w_hat = q s of 8 weights as fp16 operands; the largest magnitude, for the range check.
+__device__ __forceinline__ uint4 pack_w16(const float (&f)[8], uint32_t& out) {
+  uint4 o;
+  uint32_t* u = reinterpret_cast<uint32_t*>(&o);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    u[k] = tc::pack_half2(f[2 * k], f[2 * k + 1]);
+    out = max_abs_f16x2(out, u[k]);
+  }
+  return o;
+}
+
+// A scale as the quantiser uses it: finite and > 0 (else flagged, and 1 in its place).
+__device__ __forceinline__ float checked_scale(float sc, int& bad) {
+  if (sc > 0.f && isfinite(sc)) return sc;
+  bad |= 1;
+  return 1.f;
+}
+
+// jab_quantize: int8 codes and / or fp32 w_hat.
+__global__ void __launch_bounds__(256) quantize_kernel(const uint4* __restrict__ w,
+                                                       const float* __restrict__ s, int D, int d,
+                                                       int G, int bits, int8_t* __restrict__ codes,
+                                                       float* __restrict__ w_hat32, int* status) {
+  const int64_t n8 = (int64_t)D * d / 8, step = (int64_t)gridDim.x * blockDim.x;
+  const int qmax = qmax_of(bits);
+  int bad = 0;
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  GroupWalk at(i, step, G / 8);
+  auto put = [&](const uint4& v, float sc, int64_t i) {
+    float q[8];
+    quant_codes8(v, sc, qmax, q);
+    if (codes) {
+      uint32_t c[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        c[h] = (uint32_t)((int)q[4 * h] & 0xff) | (uint32_t)((int)q[4 * h + 1] & 0xff) << 8 |
+               (uint32_t)((int)q[4 * h + 2] & 0xff) << 16 | (uint32_t)(int)q[4 * h + 3] << 24;
+      *reinterpret_cast<uint2*>(codes + i * 8) = make_uint2(c[0], c[1]);
+    }
+    if (w_hat32) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) q[k] = __fmul_rn(q[k], sc);
+      reinterpret_cast<float4*>(w_hat32 + i * 8)[0] = make_float4(q[0], q[1], q[2], q[3]);
+      reinterpret_cast<float4*>(w_hat32 + i * 8)[1] = make_float4(q[4], q[5], q[6], q[7]);
+    }
+  };
+  for (; i + step < n8; i += 2 * step) {
+    const uint4 v0 = __ldg(w + i), v1 = __ldg(w + i + step);
+    const float s0 = __ldg(s + at.next()), s1 = __ldg(s + at.next());
+    put(v0, checked_scale(s0, bad), i);
+    put(v1, checked_scale(s1, bad), i + step);
+  }
+  if (i < n8) put(__ldg(w + i), checked_scale(__ldg(s + at.next()), bad), i);
+  if (bad) report(status, JAB_ERR_NONFINITE);
+}
+
+// Block `blk` of `nblk`: the fp16 operand of every candidate (or of W itself, ncand = 0). W is read
+// once for all candidates; the outputs are what moves.
+__device__ __forceinline__ void quantize_role(const PrepArgs& p, int blk, int nblk) {
+  const int64_t n8 = (int64_t)p.D * p.d / 8, step = (int64_t)nblk * blockDim.x;
+  int bad = 0;
+  uint32_t in = 0, out = 0;
+  int64_t i = (int64_t)blk * blockDim.x + threadIdx.x;
+  if (p.ncand == 0) {
+    for (; i + step < n8; i += 2 * step) {
+      const uint4 v0 = __ldg(p.w + i), v1 = __ldg(p.w + i + step);
+      p.w16[i] = convert8(v0, in, out);
+      p.w16[i + step] = convert8(v1, in, out);
+    }
+    if (i < n8) p.w16[i] = convert8(__ldg(p.w + i), in, out);
+  } else {
+    GroupWalk at(i, step, p.G / 8);
+    auto put = [&](const uint4& v, float sc, int c, int64_t i) {
+      float q[8];
+      sc = checked_scale(sc, bad);
+      quant_codes8(v, sc, qmax_of(p.bits[c]), q);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) q[k] = __fmul_rn(q[k], sc);
+      p.w16[c * n8 + i] = pack_w16(q, out);
+    };
+    for (; i < n8; i += 2 * step) {
+      const bool two = i + step < n8;
+      const uint4 v0 = __ldg(p.w + i);
+      uint4 v1 = make_uint4(0u, 0u, 0u, 0u);
+      if (two) v1 = __ldg(p.w + i + step);
+      const int64_t g0 = at.next(), g1 = two ? at.next() : g0;
+      float s0 = __ldg(p.s[0] + g0), s1 = __ldg(p.s[0] + g1);
+      for (int c = 0; c < p.ncand; ++c) {
+        const int cn = c + 1 < p.ncand ? c + 1 : c;  // the next candidate's scales, ahead
+        const float n0 = __ldg(p.s[cn] + g0), n1 = __ldg(p.s[cn] + g1);
+        put(v0, s0, c, i);
+        if (two) put(v1, s1, c, i + step);
+        s0 = n0;
+        s1 = n1;
       }
-      w16[i] = o;
     }
   }
-  if (bad & 1) report(status, JAB_ERR_NONFINITE);
-  else if (bad & 2) report(status, JAB_ERR_RANGE);
+  if (bad) report(p.status, JAB_ERR_NONFINITE);
+  else if (either_at_least(out, kHalfInf)) report(p.status, JAB_ERR_RANGE);  // not an fp16 operand
+}
+
+// ---------------------------------------------------------------- RoPE table (reading R7)
+// fp64: a pow and a sincos per entry took 48 us for 2048 x 64, as an SM issues an fp64 instruction of a
+// warp in about 16 clocks. The frequencies come with the launch; a thread takes the sincos of its
+// first row and of one step and rotates on through kRopeRun rows (an fp64 rotation adds 1e-16, the
+// table keeps 6e-8); a block has one run of rows only, so that the work spreads over all SMs.
+constexpr int kRopeRun = 16;
+__device__ __forceinline__ void rope_role(const PrepArgs& p, int blk) {
+  const int j = threadIdx.x, t0 = blk * kRopeRun;
+  if (j >= p.half) return;
+  const double f = p.freq_pi[j];  // (the pi forms need no long argument reduction)
+  double sn, cs, sd, cd;
+  sincospi((double)t0 * f, &sn, &cs);
+  sincospi(f, &sd, &cd);
+  const int n = min(kRopeRun, p.T - t0);
+  int64_t i = (int64_t)t0 * p.half + j;
+  for (int k = 0; k < n; ++k, i += p.half) {
+    p.cos_t[i] = (float)cs;
+    p.sin_t[i] = (float)sn;
+    const double c2 = cs * cd - sn * sd;
+    sn = sn * cd + cs * sd;
+    cs = c2;
+  }
+}
+
+// Everything the projection reads that is not there yet, in one launch: blocks [0, nrope) the RoPE
+// table, then nw blocks the weights, then nx blocks X. As launches of their own, and with a 64-bit index
+// division per chunk and a quotient division per weight, they took 38 us for one candidate's 6144 x
+// 4096 weights and 30-85 us for the table (1337-4096 rows), now 31 us together at 1337 rows; for five
+// candidates, 2048 rows and 65536 x 4096 of X 462 us, now 248 us (1.37 GB: 202 us at the copy rate).
+__global__ void __launch_bounds__(256, 4) prep_kernel(const __grid_constant__ PrepArgs p) {
+  const int blk = blockIdx.x;
+  if (blk < p.nrope)
+    rope_role(p, blk);
+  else if (blk < p.nrope + p.nw)
+    quantize_role(p, blk - p.nrope, p.nw);
+  else
+    convert_x_role(p.x, p.xh, p.n8x, blk - p.nrope - p.nw, p.nx, p.status);
 }
 
 // ---------------------------------------------------------------- Rademacher probes (Section 2.4)
@@ -117,7 +289,7 @@ __global__ void rademacher_probe_kernel(uint64_t seed, uint64_t first, int64_t n
 // about two FP64 operations per clock and SM, and five of them per weight bounded the kernel (199 us
 // for 6144 x 4096). So a term is formed as an unevaluated pair of floats: q s - w exactly (product and
 // difference with their rounding errors), its square to about 2^-46 of itself, eight of them added
-// with the errors carried along, and only that sum goes to the fp64 accumulator: 52 us. Weights and
+// with the errors carried along, and only that sum goes to the fp64 accumulator: 42 us. Weights and
 // scale are first multiplied by the power of two that brings the scale to [1, 2) (exact), so that no
 // square under- or overflows; a chunk whose values leave that window takes the fp64 form.
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -127,7 +299,8 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 }
 
 // Sum of (q s - w)^2 over the 8 weights of a chunk.
-__device__ __forceinline__ double qerr_chunk(const bf16_t* b, float sc, int qmax) {
+__device__ __forceinline__ double qerr_chunk(const uint4& v, float sc, int qmax) {
+  const bf16_t* b = reinterpret_cast<const bf16_t*>(&v);
   const int ex = (__float_as_int(sc) >> 23) & 0xff;  // exponent field of the scale
   const float up = __int_as_float((254 - ex) << 23);  // 2^(127 - ex): the scale times this is in [1, 2)
   const float ss = sc * up;
@@ -143,11 +316,11 @@ __device__ __forceinline__ double qerr_chunk(const bf16_t* b, float sc, int qmax
     }
     return acc;
   }
-  float sh = 0.f, sl = 0.f;
+  float sh = 0.f, sl = 0.f, code[8];
+  quant_codes8(v, sc, qmax, code);
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    const float wv = __bfloat162float(b[k]);
-    const float q = quant_code(wv, sc, qmax, nullptr);
+    const float wv = __bfloat162float(b[k]), q = code[k];
     const float ph = __fmul_rn(q, ss), pl = __fmaf_rn(q, ss, -ph);  // q s = ph + pl
     float dh, dl;
     two_sum(ph, -(wv * up), dh, dl);
@@ -171,27 +344,14 @@ __global__ void __launch_bounds__(256) qerr_partial_kernel(const uint4* __restri
   __shared__ double red[8];
   const int64_t n8 = (int64_t)D * d / 8;
   const int qmax = qmax_of(bits);
-  const int ng = d / G, d8 = d / 8, g8 = G / 8;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
   double acc = 0.0;
   int bad = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    uint4 v = __ldg(w + i);
-    int64_t row;
-    int c8;
-    if (n8 <= INT32_MAX) {  // (a 64-bit division costs more than the rest of the addressing)
-      row = (int)i / d8;
-      c8 = (int)i - (int)row * d8;
-    } else {
-      row = i / d8;
-      c8 = (int)(i - row * d8);
-    }
-    float sc = __ldg(s + row * ng + c8 / g8);
-    if (!(sc > 0.f) || !isfinite(sc)) {
-      bad = 1;
-      sc = 1.f;
-    }
-    acc += qerr_chunk(reinterpret_cast<const bf16_t*>(&v), sc, qmax);
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  for (GroupWalk at(i, step, G / 8); i < n8; i += step) {
+    const uint4 v = __ldg(w + i);
+    const float sc = checked_scale(__ldg(s + at.next()), bad);
+    acc += qerr_chunk(v, sc, qmax);
   }
   const double t = block_sum<256>(acc, red);
   if (threadIdx.x == 0) part[blockIdx.x] = t;
@@ -401,21 +561,6 @@ __global__ void __launch_bounds__(256) init_scales_minmse_kernel(const bf16_t* _
   if (live && l16 == 0) s_out[grp] = best >= 0 ? trial_scale(s0, best) : s0;
 }
 
-// ---------------------------------------------------------------- RoPE table (reading R7)
-__global__ void rope_table_kernel(int T, int dh, double theta, float* __restrict__ cos_t,
-                                  float* __restrict__ sin_t) {
-  const int half = dh / 2;
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= (int64_t)T * half) return;
-  const int t = (int)(i / half), j = (int)(i % half);
-  const double inv_freq = pow(theta, -2.0 * (double)j / (double)dh);
-  const double phi = (double)t * inv_freq;
-  double sn, cs;
-  sincos(phi, &sn, &cs);
-  cos_t[i] = (float)cs;
-  sin_t[i] = (float)sn;
-}
-
 // ---------------------------------------------------------------- host launchers
 static int grid_for(int64_t n, int threads, int sms) {
   int64_t g = (n + threads - 1) / threads;
@@ -423,19 +568,62 @@ static int grid_for(int64_t n, int threads, int sms) {
   return (int)(g < cap ? (g < 1 ? 1 : g) : cap);
 }
 
-cudaError_t launch_convert_x(const void* x, void* xh, int64_t n, int* status, int sms,
-                             cudaStream_t st) {
-  const int64_t n8 = n / 8;
-  convert_x_kernel<<<grid_for(n8, 256, sms), 256, 0, st>>>((const uint4*)x, (uint4*)xh, n8, status);
-  return cudaGetLastError();
+cudaError_t launch_prep(const PrepInputs& in, int* status, int sms, cudaStream_t st) {
+  const int64_t n8 = (int64_t)in.D * in.d / 8;
+  for (int c0 = 0; c0 == 0 || c0 < in.ncand; c0 += PrepArgs::kMaxCand) {
+    PrepArgs p{};
+    p.status = status;
+    p.D = in.D;
+    p.d = in.d;
+    p.G = in.G;
+    if (in.w != nullptr) {
+      p.w = static_cast<const uint4*>(in.w);
+      p.w16 = static_cast<uint4*>(in.w16) + c0 * n8;
+      p.ncand = std::min(in.ncand - c0, (int)PrepArgs::kMaxCand);
+      for (int c = 0; c < p.ncand; ++c) {
+        p.s[c] = in.s[c0 + c];
+        p.bits[c] = in.bits[c0 + c];
+      }
+      p.nw = std::min(grid_for(n8, 256, sms), 4 * sms);  // what is resident at once
+    }
+    if (c0 == 0 && in.x != nullptr) {
+      p.x = static_cast<const uint4*>(in.x);
+      p.xh = static_cast<uint4*>(in.xh);
+      p.n8x = in.nx / 8;
+      p.nx = std::min(grid_for((p.n8x + 3) / 4, 256, sms), 4 * sms);
+    }
+    if (c0 == 0 && in.cos_t != nullptr) {
+      p.cos_t = in.cos_t;
+      p.sin_t = in.sin_t;
+      p.T = in.T;
+      p.half = in.dh / 2;
+      // by squares of the first ratio: one pow a call, each frequency a product of at most six powers
+      // (long double: the rounding to double is the only one that counts)
+      long double pw[6];
+      pw[0] = powl((long double)in.theta, -1.0L / p.half);
+      for (int b = 1; b < 6; ++b) pw[b] = pw[b - 1] * pw[b - 1];
+      for (int j = 0; j < p.half; ++j) {
+        long double f = 0.318309886183790671537767526745028724L;  // 1 / pi
+        for (int b = 0; b < 6; ++b)
+          if ((j >> b) & 1) f *= pw[b];
+        p.freq_pi[j] = (double)f;
+      }
+      p.nrope = (in.T + kRopeRun - 1) / kRopeRun;
+    }
+    const int grid = p.nrope + p.nw + p.nx;
+    if (grid == 0) return cudaSuccess;
+    prep_kernel<<<(unsigned)grid, 256, 0, st>>>(p);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_quantize(const void* w, const float* s, int D, int d, int G, int bits,
-                            void* w16, int8_t* codes, float* w_hat32, int* status, int sms,
-                            cudaStream_t st) {
+                            int8_t* codes, float* w_hat32, int* status, int sms, cudaStream_t st) {
   const int64_t n8 = (int64_t)D * d / 8;
-  quantize_kernel<<<grid_for(n8, 256, sms), 256, 0, st>>>(
-      (const uint4*)w, s, D, d, G, bits, (uint4*)w16, codes, w_hat32, status);
+  quantize_kernel<<<grid_for(n8, 256, sms), 256, 0, st>>>((const uint4*)w, s, D, d, G, bits, codes,
+                                                          w_hat32, status);
   return cudaGetLastError();
 }
 
@@ -475,13 +663,6 @@ cudaError_t launch_init_scales(const void* w, int D, int d, int G, int bits, int
   else
     init_scales_minmse_kernel<<<(unsigned)((groups + 15) / 16), 256, 0, st>>>((const bf16_t*)w, groups,
                                                                               G, bits, s_out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_rope_table(int T, int dh, double theta, float* cos_t, float* sin_t,
-                              cudaStream_t st) {
-  const int64_t n = (int64_t)T * (dh / 2);
-  rope_table_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(T, dh, theta, cos_t, sin_t);
   return cudaGetLastError();
 }
 

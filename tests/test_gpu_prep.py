@@ -72,3 +72,48 @@ def test_omega_error_sum_in_pairs(kind, bits):
     want, _ = O.omega_scores(1.0, np64(w), s.cpu().numpy(), bits, G, layers_after=1)
     np.testing.assert_allclose(c1.item(), want, rtol=2.0 ** -46 + 4096 * 2.0 ** -53)
     assert J().jab_get_device_status() == 0
+
+
+@pytest.mark.parametrize("bits", [2, 3, 8])
+@pytest.mark.parametrize("w_mul,s_mul", [(1.0, 1.0), (1e-25, 1e-25), (1e30, 1e30), (1e-30, 1.0)])
+def test_codes_bit_exact_in_and_out_of_the_quotient_window(w_mul, s_mul, bits):
+    """The corrected-reciprocal quotient inside its window, the division outside it, and chunks that mix
+    zeros and both: the codes of the fp32 quotient, ties included (weights on half steps)."""
+    d, G = 256, 64
+    g = torch.Generator().manual_seed(5)
+    s = (torch.rand((256, d // G), generator=g) + 0.5).numpy().astype(np.float32)
+    s[::2] = 0.25                                      # exact ties below
+    w = torch.randint(-9, 10, (256, d), generator=g).float() * 0.125
+    w[:, ::7] = torch.randn((256, (d + 6) // 7), generator=g)
+    w = (w * w_mul).to(torch.bfloat16)
+    s = (s * np.float32(s_mul)).astype(np.float32)
+    desc = J().desc_from_shape(BlockShape(d, 2, 1, 64, False), G)
+    codes = torch.empty(w.shape, dtype=torch.int8, device="cuda")
+    w_hat = torch.empty(w.shape, dtype=torch.float32, device="cuda")
+    J().jab_quantize(desc, bits, w.cuda(), torch.from_numpy(s).cuda(), codes=codes, w_hat=w_hat)
+    oc, ow, _ = O.quantize(np64(w), s, bits, G)
+    np.testing.assert_array_equal(codes.cpu().numpy(), oc)
+    np.testing.assert_array_equal(w_hat.cpu().numpy(), ow.astype(np.float32))
+    assert J().jab_get_device_status() == 0
+
+
+@pytest.mark.parametrize("shape,T", [(BlockShape(256, 4, 1, 64, True, 500.0), 65),
+                                     (BlockShape(512, 4, 2, 128, True, 1e4), 33)])
+def test_ten_candidates_in_one_call_equal_single_calls(shape, T):
+    """More candidates than one preparation launch takes (8): each loss has the bits of a call of its
+    own, with an odd number of rows for the last run of the RoPE table."""
+    from dataclasses import replace
+    from tests.harness import Case
+    from workloads import WORKLOADS
+    c = Case(replace(WORKLOADS["gpt2_smoke"], shape=shape), 2, T, 64)
+    bits = [2, 3, 4, 5, 8, 2, 3, 4, 5, 8]
+    scales = [c.gpu_scales(b) * f for b, f in zip(bits, [1.0] * 5 + [0.7] * 5)]
+    ws = c.workspace(n_cand=10, with_bwd=False)
+    A, _, _ = c.gpu_teacher(ws)
+    loss = torch.empty(10, dtype=torch.float64, device="cuda")
+    J().jab_loss_forward(c.desc, c.B, c.T, c.X, c.W, A, bits, scales, loss, ws)
+    one = torch.empty(1, dtype=torch.float64, device="cuda")
+    for i in range(10):
+        J().jab_loss_forward(c.desc, c.B, c.T, c.X, c.W, A, bits[i:i + 1], scales[i:i + 1], one, ws)
+        assert one.item() == loss[i].item(), i
+    assert J().jab_get_device_status() == 0
