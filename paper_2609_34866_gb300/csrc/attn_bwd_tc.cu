@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
   }
   uint8_t* smem = smem_raw;
   DkdvBars* bars = reinterpret_cast<DkdvBars*>(smem + L::BAR_OFF);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   volatile int* abort = &bars->abort;
 
   const int r = p.Hq / p.Hkv;
@@ -259,10 +259,10 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = bars->tmem_base;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
 
   if (warp == 0) {
-    if (lane == 0) {  // ------------------------------------------------------------- TMA
+    if (tc::elect_one()) {  // ------------------------------------------------------------- TMA
       uint32_t issued = 0, last_par = 0;
       tc::mbar_expect_tx(&bars->kv_full, 2 * BK * DH * 2);
       for (int ch = 0; ch < L::NCH; ++ch) {
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
       }
     }
   } else if (warp == 1 || warp == DKDV_GRAD_WARP) {
-    if (lane == 0) {  // ---------------------- UMMA: S^T, dP^T (warp 1); dV, dK (DKDV_GRAD_WARP)
+    if (tc::elect_one()) {  // ------------------- UMMA: S^T, dP^T (warp 1); dV, dK (DKDV_GRAD_WARP)
       // Two issuing threads, so that the score products of the next block are never held back
       // behind the issue of this block's gradient products, nor the other way round. Every
       // dependency between them goes through a barrier: S^T(j) overwrites P^T(j - 1), so it waits
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
       drain_wait(dr, 0);
     }
   } else if (warp == 2 + DKDV_EW) {
-    if (lane == 0) {  // ------------------------------------------ dS^T tiles to global memory
+    if (tc::elect_one()) {  // ----------------------------------------- dS^T tiles to global memory
       // Tile (sequence b, head h, query block i, key block kb) is row block
       // (b Hq + h) npairs + i (i + 1) / 2 + kb of the dS^T buffer: 128 key rows of 128 queries.
       auto tile_of = [&](int it) {
@@ -692,7 +692,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
   }
   uint8_t* smem = smem_raw;
   TpBars* bars = reinterpret_cast<TpBars*>(smem + L::BAR_OFF);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   volatile int* abort = &bars->abort;
 
   const int r = p.Hq / p.Hkv;
@@ -736,10 +736,10 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = bars->tmem_base;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
 
   if (warp == 0) {
-    if (lane == 0) {  // ------------------------------------------------------------- TMA
+    if (tc::elect_one()) {  // ------------------------------------------------------------- TMA
       uint32_t issued = 0, last_par = 0;
       tc::mbar_expect_tx(&bars->kv_full, 2 * BK * DH * 2);
       for (int ch = 0; ch < L::NCH; ++ch) {
@@ -776,7 +776,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {  // ---------------------------------------------------------------- UMMA
+    if (tc::elect_one()) {  // ---------------------------------------------------------------- UMMA
       constexpr uint32_t ID_S = tc::idesc_f16(false, BK, BQ);
       bool ok = tc::mbar_wait(&bars->kv_full, 0, abort, p.status);
       const uint64_t kt = tc::sdesc_kmajor_sw128(tc::smem_u32(smem + L::KT_OFF));
@@ -810,7 +810,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       drain_wait(&bars->drain, 0);
     }
   } else if (warp == 2 + DKDV_EW) {
-    if (lane == 0) {  // ------------------------------------------------- P^T tiles to global
+    if (tc::elect_one()) {  // ------------------------------------------------- P^T tiles to global
       for (int it = 0; it < n_it; ++it) {
         if (!tc::mbar_wait(&bars->dss_full, it & 1, abort, p.status)) break;
         const int h = g * r + it / per_head, i = kb + it % per_head;
@@ -989,7 +989,7 @@ __global__ void __launch_bounds__(DQ_THREADS, 1)
   }
   uint8_t* smem = smem_raw;
   DqBars* bars = reinterpret_cast<DqBars*>(smem + L::BAR_OFF);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   volatile int* abort = &bars->abort;
 
   const int nqb = (p.T + BQ - 1) / BQ;
@@ -1019,10 +1019,10 @@ __global__ void __launch_bounds__(DQ_THREADS, 1)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = bars->tmem_base;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
 
   if (warp == 0) {
-    if (lane == 0) {  // ---------------------------------------------------------------- TMA
+    if (tc::elect_one()) {  // ---------------------------------------------------------------- TMA
       uint32_t J = 0, iss = 0, par = 0;
       bool ok = true;
       for (int it = 0, tile = sched_tile(0, gridDim.x, blockIdx.x); ok && tile < n_tiles;
@@ -1051,7 +1051,7 @@ __global__ void __launch_bounds__(DQ_THREADS, 1)
           if (iss & (1u << st)) drain_wait(&bars->full[st], (par >> st) & 1);
     }
   } else if (warp == 1) {
-    if (lane == 0) {  // ---------------------------------------------------------------- UMMA
+    if (tc::elect_one()) {  // ---------------------------------------------------------------- UMMA
       // A = dS (M = queries, K = keys) and B = K (N = d_h, K = keys) are both MN-major tiles
       constexpr uint32_t ID_Q = tc::idesc_f16(false, BQ, DH) | (1u << 15) | (1u << 16);
       uint32_t J = 0;

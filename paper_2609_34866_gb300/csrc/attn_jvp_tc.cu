@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
   JvpBars* bars = reinterpret_cast<JvpBars*>(smem + L::BAR_OFF);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   volatile int* abort = &bars->abort;
 
   // CTA order: grouped by (sequence, KV group), so that the CTAs which stream the K blocks
@@ -128,10 +128,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = bars->tmem_base;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
 
   if (warp == 0) {
-    if (lane == 0) {  // ---------------------------------------------------------------- TMA
+    if (tc::elect_one()) {  // ---------------------------------------------------------------- TMA
       const int qcol = h * DH, kcol = (p.Hq + g) * DH, vcol = (p.Hq + p.Hkv + g) * DH;
       uint32_t kd_issued = 0, kd_par = 0;
       bool vd_issued = false, ok = true;
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {  // ---------------------------------------------------------------- UMMA
+    if (tc::elect_one()) {  // ---------------------------------------------------------------- UMMA
       constexpr uint32_t ID_S = tc::idesc_f16(false, BQ, BK);
       constexpr uint32_t ID_Z = tc::idesc_f16(false, BQ, DH) | (1u << 16);  // B = V / dV, MN-major
       bool ok = tc::mbar_wait(&bars->q_full, 0, abort, p.status);

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
   KlBars* bars = reinterpret_cast<KlBars*>(smem + L::BAR_OFF);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   volatile int* abort = &bars->abort;
 
   // CTA order: grouped by (sequence x candidate, KV group), so that the CTAs which stream the K blocks
@@ -161,10 +161,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = bars->tmem_base;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
 
   if (warp == 0) {
-    if (lane == 0) {  // ---------------------------------------------------------------- TMA
+    if (tc::elect_one()) {  // ---------------------------------------------------------------- TMA
       const int qs_col = c * p.D + h * DH, qt_col = h * DH;
       const int ks_col = c * p.D + (p.Hq + g) * DH, kt_col = (p.Hq + g) * DH;
       uint32_t issued = 0, last_par = 0;
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {  // ---------------------------------------------------------------- UMMA
+    if (tc::elect_one()) {  // ---------------------------------------------------------------- UMMA
       constexpr uint32_t ID_S = tc::idesc_f16(false, BQ, BK);
       bool ok = tc::mbar_wait(&bars->q_full, 0, abort, p.status);
       if (ok) {

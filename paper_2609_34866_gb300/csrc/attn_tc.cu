@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(Issue<DH>::kThreads, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
   StackBars* bars = reinterpret_cast<StackBars*>(smem + L::BAR_OFF);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   volatile int* abort = &bars->abort;
   const int units = p.Hq / HPT, BC = p.B * p.C;
   const int nqb = (p.T + RPH - 1) / RPH;
@@ -180,10 +180,10 @@ __global__ void __launch_bounds__(Issue<DH>::kThreads, 1)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = bars->tmem_base;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
 
   if (warp == 0 || warp == 10) {
-    if (lane == 0) {  // ------------------------------------------------ TMA: Q and K (warp 0), V (10)
+    if (tc::elect_one()) {  // --------------------------------------- TMA: Q and K (warp 0), V (10)
       const bool is_v = warp == 10;
       int gi = 0, tc_ = 0;
       uint32_t iss = 0, par = 0, qiss = 0, qpar = 0;
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(Issue<DH>::kThreads, 1)
       }
     }
   } else if (warp == 1 || (Issue<DH>::kSplit && warp == PV_WARP)) {
-    if (lane == 0) {  // ------------------------------------------ UMMA: S (warp 1), P V (PV_WARP)
+    if (tc::elect_one()) {  // ------------------------------------- UMMA: S (warp 1), P V (PV_WARP)
       constexpr uint32_t ID_S = tc::idesc_f16(false, 128, SKB);
       constexpr uint32_t ID_PV = tc::idesc_f16(false, 128, DH) | (1u << 16);  // B = V, MN-major
       int g0 = 0, tc_ = 0;

@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
   Bars2* bars = reinterpret_cast<Bars2*>(smem + STAGES2 * STAGE2_BYTES);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = tc::cluster_ctarank();  // 0: issues the pair's UMMAs
   const bool leader = rank == 0;
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
@@ -310,12 +310,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   tc::fence_after_sync();
   // both CTAs' barriers are initialised and their tensor memory allocated before any signal crosses
   tc::cluster_sync();
-  const uint32_t tmem = bars->tmem_base;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
   const uint32_t full_lead = tc::mapa_shared(tc::smem_u32(&bars->full[0]), 0);
   const uint32_t tempty_lead = tc::mapa_shared(tc::smem_u32(&bars->tempty[0]), 0);
 
   if (warp == 0) {
-    if (lane == 0) {  // ---------------- TMA producer
+    if (tc::elect_one()) {  // ---------------- TMA producer
       int stage = 0;
       uint32_t phase = 0;
       uint32_t issued = 0, last_parity = 0;  // per-stage bitmasks for the exit drain (even CTA)
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           if (issued & (1u << s)) drain_wait(&bars->full[s], (last_parity >> s) & 1);
     }
   } else if (warp == 1) {
-    if (lane == 0 && leader) {  // ---------------- UMMA issuer of the pair
+    if (leader && tc::elect_one()) {  // ---------------- UMMA issuer of the pair
       constexpr uint32_t IDESC = tc::idesc_f16(BF16, BM2, BN) | (B_MN ? (1u << 16) : 0u);
       int stage = 0, it = 0;
       uint32_t phase = 0;

@@ -24,6 +24,24 @@ __device__ __forceinline__ uint64_t globaltimer() {
 // the other roles of the CTA to stop (no kernel can hang the GPU on a barrier that never flips).
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
+// True in one lane of the (converged) warp. The roles of a single thread branch on this rather than
+// on a lane number: the compiler then knows that one thread runs and issues a tcgen05 or TMA
+// instruction, whose operands are uniform registers, as it stands. After `lane == 0` it cannot know, and
+// each such instruction waits for its operands to be made uniform: four K = 16 UMMAs took 400 clocks to
+// issue that way and 120 this way (GB300; the pipe needs 256 for them), more than any attention
+// kernel's products left room for.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok));
+  return ok != 0;
+}
+// The warp's index, known to be the same in all its lanes.
+__device__ __forceinline__ int warp_index() {
+  return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+}
+
 // ------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
