@@ -21,16 +21,16 @@ constexpr int BQ = 128;          // query rows of a tile
 constexpr int EW_WARPS = 8;      // softmax warps
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
-constexpr float kRescaleLog2 = 8.f;  // rescale O only when the row max grows by more than 2^8
+// O is rescaled only when a row's maximum grows by more than 2^12: P then stays below 2^12, far inside
+// fp16, and large scores, which grow by 2^8 in most blocks of a heavy-tailed batch, rescale less often.
+constexpr float kRescaleLog2 = 12.f;
 
 struct FwdParams {
   int T, B, C, Hq, Hkv, D, nqb, nP, lse_pitch;
   float sl2;  // softmax scale * log2(e)
   double* part;
   const float* a_ref;
-  float* a_out;
   float* lse;
-  half_t* d_o;
   float* dvec;
   int* status;
 };
@@ -58,35 +58,38 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
 // softmax warps already work on tile i + 1.
 //   warp 0       TMA: Q tile, K ring (3 stages: a K load is issued once S two blocks back has
 //                completed and must land before S of the block after next)
-//   warp 1       TMEM owner, tcgen05.cp of Q, UMMA issuer (one thread): S, and for d_h = 64 also
-//                P V; for d_h = 128 warp 15 issues P V (two issuers, so that S of the next block
-//                is not held back behind the issue of P V, and vice versa)
+//   warp 1       TMEM owner, tcgen05.cp of Q, UMMA issuer of S (one thread);   warp 15  of P V
 //   warps 2..9   softmax: warp (quarter q, half h) owns the 16 rows at lanes 32 q + 16 h; with the
 //                16x256b TMEM shape four threads share a row (32 of its 128 scores each, two rows per
 //                thread), so row maxima and sums need only warp shuffles. Lazy rescaling as in the
 //                single-head kernel. At the end of a tile the row statistics go to shared memory.
 //   warp 10      TMA: V ring (2 stages), so that K loads never queue behind a V stage that is busy
-//   warps 11..14 epilogue, one TMEM lane quarter each (32x32b shape, one row per thread, 32 columns
-//                at a time): O is staged through shared memory so that A_ref loads and dO / A
-//                stores are coalesced; per-mode outputs and the SSE partials. Each thread
-//                prefetches its row of the next tile's A_ref into L2 a whole tile ahead.
+//   warps 11..14 epilogue, one TMEM lane quarter each (32x32b shape, one row per thread, 32 columns at a
+//                time): A_ref arrives in shared memory by TMA (32 x 32 boxes, two per warp in flight,
+//                its lines brought into L2 a whole tile ahead), dO / A leave by TMA from the same
+//                buffers (rows past T are clipped by the tensor map), so that row sums need no
+//                shuffles and nothing is staged: 4.4k clocks a tile in mode 1 and 8.3k in mode 2 at
+//                d_h = 128, where coalesced loads and stores through a staging tile took 8k and 16k,
+//                more than the main loop (mode 2, 128 x 2048 tokens: 4.95 -> 4.35 ms; 3 x 1337: 75 ->
+//                58 us). With that the softmax warps bound the loop again: about 1450 clocks a block of
+//                reading S, maximum, exponentials and store in a row, against 1024 of tensor work at
+//                d_h = 128 and 640 at 64. Two query tiles in flight per CTA, or two sets of four warps on
+//                alternate blocks, were slower: their chains through P, P V and the running maximum
+//                fall into step (899-961 against 738 us for 4 x 64 x 12 heads of 1024 x 64).
 constexpr int SQ = 64, SKB = 128, SK_ST = 3, SV_ST = 2;
-// d_h = 128: S and P V are issued by two threads (warp 1 and PV_WARP), so that S of the next block
-// never waits behind the issue of the current P V. d_h = 64: one issuer (measured faster there).
-template <int DH> struct Issue {
-  static constexpr bool kSplit = DH == 128;
-  static constexpr int kThreads = kSplit ? 512 : 480;
-};
+constexpr int NUM_THREADS = 512;
+// S and P V are issued by two threads (warp 1 and PV_WARP), so that S of the next block never waits
+// behind the issue of the current P V.
 constexpr int PV_WARP = 15;
 constexpr int EPI_WARPS = 4, EPI_WARP0 = 11;
 
 struct StackBars {
   uint64_t q_full, q_empty, k_full[SK_ST], k_empty[SK_ST], v_full[SV_ST], v_empty[SV_ST];
   uint64_t s_full, s_empty, p_full, pv_done, o_full[2], o_empty[2], st_full[2], st_empty[2];
-  uint64_t drain, drain_pv;
+  uint64_t a_full[EPI_WARPS][2], drain, drain_pv;
   uint32_t tmem_base;
   int abort;
-  double red[2][EPI_WARPS];         // [tile parity][epilogue warp]
+  double red[2][EPI_WARPS];         // [tile parity][TMEM lane quarter]
   float row_m[2][128], row_l[2][128];  // [tile parity][stacked row]: running max (log2), sum
 };
 
@@ -97,9 +100,10 @@ struct StackLayout {
   static constexpr int Q_OFF = 0;
   static constexpr int K_OFF = Q_OFF + TILE;
   static constexpr int V_OFF = K_OFF + SK_ST * TILE;
-  static constexpr int EPI_OFF = V_OFF + SV_ST * TILE;  // per epilogue warp: 32 x 32 fp32
-  static constexpr int BAR_OFF = EPI_OFF + EPI_WARPS * 4096;
-  static constexpr int USED = BAR_OFF + (int)sizeof(StackBars) + 1024;
+  static constexpr int EPI_OFF = V_OFF + SV_ST * TILE;  // per epilogue warp two boxes of 32 x 32 fp32
+  static constexpr int BAR_OFF = EPI_OFF + EPI_WARPS * 2 * 4096;
+  static constexpr int USED = BAR_OFF + (int)sizeof(StackBars);  // base alignment checked in the kernel
+  static_assert(USED <= 227 * 1024, "shared memory budget");
   static constexpr int SMEM = USED > 118 * 1024 ? USED : 118 * 1024;
   static constexpr uint32_t S_COL = 0, O_COL = SKB, Q_COL = SKB + 2 * DH,
                             P_COL = SKB + 2 * DH + DH / 2;
@@ -129,14 +133,19 @@ __device__ __forceinline__ StackTile stack_tile(int k, int units, int Hkv, int n
 // HPT = query heads per tile: 2 stacks 64 rows of two heads of one KV group (even GQA ratio), 1
 // takes 128 rows of one head (any ratio, e.g. GPT-2's separate heads).
 template <int DH, int MODE, int HPT>
-__global__ void __launch_bounds__(Issue<DH>::kThreads, 1)
+__global__ void __launch_bounds__(NUM_THREADS, 1)
     attn_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q,
-                         const __grid_constant__ CUtensorMap tm_kv, const FwdParams p) {
+                         const __grid_constant__ CUtensorMap tm_kv,
+                         const __grid_constant__ CUtensorMap tm_a,
+                         const __grid_constant__ CUtensorMap tm_do, const FwdParams p) {
   using L = StackLayout<DH>;
   constexpr int RPH = 128 / HPT;  // query rows of each head in a tile
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                             ~uintptr_t(1023));
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  if (tc::smem_u32(smem_raw) & 1023u) {  // the swizzled TMA tiles need a 1024-byte aligned base
+    if (threadIdx.x == 0) report(p.status, JAB_ERR_INTERNAL);
+    return;
+  }
+  uint8_t* smem = smem_raw;
   StackBars* bars = reinterpret_cast<StackBars*>(smem + L::BAR_OFF);
   const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   volatile int* abort = &bars->abort;
@@ -166,12 +175,16 @@ __global__ void __launch_bounds__(Issue<DH>::kThreads, 1)
       tc::mbar_init(&bars->st_full[i], EW_WARPS);
       tc::mbar_init(&bars->st_empty[i], EPI_WARPS);
     }
+    for (int w = 0; w < EPI_WARPS; ++w)
+      for (int i = 0; i < 2; ++i) tc::mbar_init(&bars->a_full[w][i], 1);
     tc::mbar_init(&bars->drain, 1);
     tc::mbar_init(&bars->drain_pv, 1);
     bars->abort = 0;
     tc::fence_mbar_init();
     tc::prefetch_tmap(&tm_q);
     tc::prefetch_tmap(&tm_kv);
+    tc::prefetch_tmap(&tm_a);
+    if (MODE == 2) tc::prefetch_tmap(&tm_do);
   }
   if (warp == 1) {
     tc::tmem_alloc(&bars->tmem_base, 512);
@@ -226,7 +239,7 @@ __global__ void __launch_bounds__(Issue<DH>::kThreads, 1)
           if (iss & (1u << st)) drain_wait(&full[st], (par >> st) & 1);
       }
     }
-  } else if (warp == 1 || (Issue<DH>::kSplit && warp == PV_WARP)) {
+  } else if (warp == 1 || warp == PV_WARP) {
     if (tc::elect_one()) {  // ------------------------------------- UMMA: S (warp 1), P V (PV_WARP)
       constexpr uint32_t ID_S = tc::idesc_f16(false, 128, SKB);
       constexpr uint32_t ID_PV = tc::idesc_f16(false, 128, DH) | (1u << 16);  // B = V, MN-major
@@ -298,10 +311,8 @@ __global__ void __launch_bounds__(Issue<DH>::kThreads, 1)
               ok = tc::mbar_wait(&bars->s_empty, gg & 1, abort, p.status) && load_q(tc_ + 1) &&
                    issue_s(gg + 1);
             }
-            if (!Issue<DH>::kSplit) ok = ok && issue_pv(gg, j == 0);
           }
           if (!ok) break;
-          if (!Issue<DH>::kSplit) tc::umma_commit(&bars->o_full[tc_ & 1]);
           g0 += tl.nkb;
           ++tc_;
           k = kn;
@@ -479,171 +490,174 @@ __global__ void __launch_bounds__(Issue<DH>::kThreads, 1)
       if (lane == 0) tc::mbar_arrive(&bars->st_full[sbf]);
     }
   } else if (warp < EPI_WARP0 + EPI_WARPS) {  // ------------------------------------- epilogue
-    // Coalesced pass: the warp's 32 rows x 32 columns of O go through shared memory; lane l then
-    // handles 16 bytes of rows 4 i + l / 8 (i < 8), eight lanes per 128-byte row segment. In mode 2
-    // each lane accumulates its share of D = rowsum(dO * O) for its rows in this layout and the
-    // eight lanes of a row add them at the end of the tile (no second pass through the slots).
+    constexpr int NCH = DH / 32;  // 32-column chunks of a row
     const int quarter = warp & 3;
     const int ew = warp - EPI_WARP0;
     const int row = quarter * 32 + lane;  // stacked row = TMEM lane
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-    float* stg = reinterpret_cast<float*>(smem + L::EPI_OFF + ew * 4096);
-    const int rbase = quarter * 32;
-    const int c4 = lane & 7;
+    uint8_t* buf = smem + L::EPI_OFF + ew * 8192;
+    uint64_t* a_full = bars->a_full[ew];
+    const int y_off = (quarter * 32) & (RPH - 1);  // this warp's rows lie in one head
+    const int h_off = quarter * 32 / RPH;
     int tc_ = 0;
+    int cc = 0;               // chunks done: buffer cc & 1, phase (cc >> 1) & 1
     uint32_t range_bits = 0;  // mode 2: an fp16 dO value out of range (inf) or NaN
-    const int64_t ext_a = (int64_t)p.B * p.T * p.Hq * DH;         // A_ref, A, dO elements
     const int64_t ext_p = (int64_t)p.C * p.B * p.Hq * p.nP;       // loss partials
-    // A_ref row segment (DH fp32) of this thread's stacked row of tile k into L2, one line at a time
+    // This row's A_ref (DH fp32) of tile k into L2, one line at a time.
     auto prefetch_aref = [&](int k) {
       const StackTile tn = stack_tile(k, units, p.Hkv, nqb, p.T, RPH);
       const int tt = tn.qb * RPH + (row & (RPH - 1));
       if (tt >= p.T) return;
       const float* src = p.a_ref + ((int64_t)(tn.bc % p.B) * p.T + tt) * (int64_t)(p.Hq * DH) +
-                         (HPT * tn.hu + row / RPH) * DH;
+                         (HPT * tn.hu + h_off) * DH;
 #pragma unroll
-      for (int l = 0; l < DH / 32; ++l) tc::prefetch_line_l2(src + 32 * l);
+      for (int l = 0; l < NCH; ++l) tc::prefetch_line_l2(src + 32 * l);
     };
+    // The loads of A_ref run two chunks ahead: the next one is chunk lch of tile lt, which is round lit's.
+    int lit = 0, lk = sched_tile(0, gridDim.x, blockIdx.x), lch = 0, issued = 0;
+    StackTile lt = stack_tile(lk < ntiles ? lk : 0, units, p.Hkv, nqb, p.T, RPH);
+    auto load_next = [&] {  // the whole warp
+      if (lk >= ntiles) return;
+      const int i = issued & 1;
+      if (tc::elect_one()) {
+        tc::mbar_expect_tx(&a_full[i], 4096);
+        tc::tma_load_3d(buf + 4096 * i, &tm_a, &a_full[i], (HPT * lt.hu + h_off) * DH + lch * 32,
+                        lt.qb * RPH + y_off, lt.bc % p.B);
+      }
+      ++issued;
+      if (++lch == NCH) {
+        lch = 0;
+        lk = sched_tile(++lit, gridDim.x, blockIdx.x);
+        if (lk < ntiles) lt = stack_tile(lk, units, p.Hkv, nqb, p.T, RPH);
+      }
+    };
+    if (MODE != 0) {
+      load_next();
+      load_next();
+    }
     for (int it = 0, k = sched_tile(0, gridDim.x, blockIdx.x); k < ntiles;
          k = sched_tile(++it, gridDim.x, blockIdx.x), ++tc_) {
       if (*abort) break;
       const StackTile tl = stack_tile(k, units, p.Hkv, nqb, p.T, RPH);
       const int b = tl.bc % p.B, c = tl.bc / p.B;
-      const int h = HPT * tl.hu + row / RPH;
-      const int q0 = tl.qb * RPH;
-      const int t = q0 + (row & (RPH - 1));
-      const int row0 = b * p.T;
-      if (MODE != 0) {  // A_ref of this tile (the first one) and of the next, a whole tile ahead
-        if (it == 0) prefetch_aref(k);
+      const int h = HPT * tl.hu + h_off;
+      const int y0 = tl.qb * RPH + y_off;  // the warp's first query row
+      const int t = y0 + lane;
+      if (MODE != 0) {  // the next tile's A_ref into L2, a whole tile ahead
         const int kn = sched_tile(it + 1, gridDim.x, blockIdx.x);
         if (kn < ntiles) prefetch_aref(kn);
       }
       const int ob = tc_ & 1;
       const uint32_t ph = (tc_ >> 1) & 1;
-      double acc = 0.0;
-      const bool have = tc::mbar_wait(&bars->st_full[ob], ph, abort, p.status) &&
-                        tc::mbar_wait(&bars->o_full[ob], ph, abort, p.status);
+      bool have = tc::mbar_wait(&bars->st_full[ob], ph, abort, p.status) &&
+                  tc::mbar_wait(&bars->o_full[ob], ph, abort, p.status);
       if (have) {
-        const float m = bars->row_m[ob][row], lt = bars->row_l[ob][row];
+        const float m = bars->row_m[ob][row], lt_ = bars->row_l[ob][row];
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&bars->st_empty[ob]);
         tc::fence_after_sync();
-        const float inv_l = __fdiv_rn(1.f, lt);
+        const bool valid = t < p.T;
+        const float inv_l = __fdiv_rn(1.f, lt_);
         float2 sq = make_float2(0.f, 0.f);  // packed partial sum of squares
-        float dpart[8];                     // mode 2: this lane's share of D for rows 4 i + lane / 8
-#pragma unroll
-        for (int i = 0; i < 8; ++i) dpart[i] = 0.f;
-        const float2 il2 = make_float2(inv_l, inv_l);
-        // A_ref rows of this lane in the coalesced layout (loading them a chunk ahead costs more in
-        // register spills than it hides)
-        float4 av[8];
-        auto load_aref = [&](int ch, float4 (&dst)[8]) {
-          const int col = h * DH + ch * 32 + c4 * 4;
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int tt = q0 + ((rbase + 4 * i + (lane >> 3)) & (RPH - 1));
-            const int64_t aoff = ((int64_t)row0 + tt) * (int64_t)(p.Hq * DH) + col;
-            if (tt < p.T && in_bounds(aoff + 3, ext_a, p.status))
-              dst[i] = __ldg(reinterpret_cast<const float4*>(p.a_ref + aoff));
-          }
-        };
-#pragma unroll 1
-        for (int ch = 0; ch < DH / 32; ++ch) {
-          const int col = h * DH + ch * 32 + c4 * 4;
-          if (MODE != 0) load_aref(ch, av);
-          {
-            uint32_t r[32];
+        float2 dd = make_float2(0.f, 0.f);  // mode 2: D = rowsum(dO * O)
+        uint32_t rb = 0;
+        // Chunk ch of the row (columns 32 ch ..), unnormalised in r.
+        auto process = [&](int ch, const uint32_t (&r)[32]) {
+          const int i = cc & 1;
+          uint8_t* bf = buf + 4096 * i;
+          if (MODE != 0 && !tc::mbar_wait(&a_full[i], (cc >> 1) & 1, abort, p.status)) have = false;
+          if (MODE == 0) {  // this buffer's last store (issued by the same elected lane) has been read
+            if (tc::elect_one()) tc::bulk_wait_group_read<1>();
             __syncwarp();
-            tc::tmem_ld32(tmem + lane_base + L::O_COL + ob * DH + ch * 32, r);
-            tc::tmem_ld_wait();
-            if (ch == DH / 32 - 1) {  // O of this buffer is read out: the next-but-one tile may use it
-              tc::fence_before_sync();
-              __syncwarp();
-              if (lane == 0) tc::mbar_arrive(&bars->o_empty[ob]);
-            }
-#pragma unroll
-            for (int v = 0; v < 8; ++v) {
-              const float2 lo = tc::mul2(make_float2(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1])), il2);
-              const float2 hi = tc::mul2(make_float2(__uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3])), il2);
-              *reinterpret_cast<float4*>(stg + lane * 32 + ((v ^ (lane & 7)) << 2)) =
-                  make_float4(lo.x, lo.y, hi.x, hi.y);
-            }
           }
-          __syncwarp();
+          uint32_t dw[16];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int rr = 4 * i + (lane >> 3);
-            const float4 ov = *reinterpret_cast<const float4*>(stg + rr * 32 + ((c4 ^ (rr & 7)) << 2));
-            const int tt = q0 + ((rbase + rr) & (RPH - 1));
-            if (tt >= p.T) continue;
-            const int64_t off = ((int64_t)row0 + tt) * (int64_t)(p.Hq * DH) + col;
-            if (!in_bounds(off + 3, ext_a, p.status)) continue;
+          for (int v = 0; v < 8; ++v) {  // 16-byte unit v of the row (128-byte swizzle)
+            // (scalar products: packed ones would be fused with the difference below, and a student
+            // equal to the teacher must give e = 0)
+            const float2 o01 = make_float2(__fmul_rn(__uint_as_float(r[4 * v]), inv_l),
+                                           __fmul_rn(__uint_as_float(r[4 * v + 1]), inv_l));
+            const float2 o23 = make_float2(__fmul_rn(__uint_as_float(r[4 * v + 2]), inv_l),
+                                           __fmul_rn(__uint_as_float(r[4 * v + 3]), inv_l));
+            float4* at = reinterpret_cast<float4*>(bf + lane * 128 + ((v ^ (lane & 7)) << 4));
             if (MODE == 0) {
-              *reinterpret_cast<float4*>(p.a_out + off) = ov;
-              const float2 v01 = make_float2(ov.x, ov.y), v23 = make_float2(ov.z, ov.w);
-              sq = tc::fma2(v23, v23, tc::fma2(v01, v01, sq));
+              *at = make_float4(o01.x, o01.y, o23.x, o23.y);
+              sq = tc::fma2(o23, o23, tc::fma2(o01, o01, sq));
             } else {
-              const float4 a = av[i];
-              const float2 e01 = tc::sub2(make_float2(ov.x, ov.y), make_float2(a.x, a.y));
-              const float2 e23 = tc::sub2(make_float2(ov.z, ov.w), make_float2(a.z, a.w));
+              const float4 a = *at;
+              const float2 e01 = tc::sub2(o01, make_float2(a.x, a.y));
+              const float2 e23 = tc::sub2(o23, make_float2(a.z, a.w));
               sq = tc::fma2(e23, e23, tc::fma2(e01, e01, sq));
               if (MODE == 2) {
-                const __half2 a01 = __floats2half2_rn(e01.x, e01.y), a23 = __floats2half2_rn(e23.x, e23.y);
-                uint2 u;
-                u.x = *reinterpret_cast<const uint32_t*>(&a01);
-                u.y = *reinterpret_cast<const uint32_t*>(&a23);
-                *reinterpret_cast<uint2*>(p.d_o + off) = u;
-                range_bits |= half2_exp_all_ones(u.x) | half2_exp_all_ones(u.y);
-                // D = rowsum(dO * O) with dO as stored (fp16-rounded)
-                const float2 f01 = __half22float2(a01), f23 = __half22float2(a23);
-                const float2 d2 = tc::fma2(f23, make_float2(ov.z, ov.w),
-                                           tc::mul2(f01, make_float2(ov.x, ov.y)));
-                dpart[i] += d2.x + d2.y;
+                const __half2 h01 = __floats2half2_rn(e01.x, e01.y), h23 = __floats2half2_rn(e23.x, e23.y);
+                dw[2 * v] = *reinterpret_cast<const uint32_t*>(&h01);
+                dw[2 * v + 1] = *reinterpret_cast<const uint32_t*>(&h23);
+                rb = max_abs_f16x2(max_abs_f16x2(rb, dw[2 * v]), dw[2 * v + 1]);
+                // D with dO as stored (fp16-rounded)
+                dd = tc::fma2(__half22float2(h23), o23, tc::fma2(__half22float2(h01), o01, dd));
               }
             }
           }
-          __syncwarp();  // the staging slots are rewritten by the next chunk
-        }
-        if (MODE == 2) {  // the eight lanes of a row (lane / 8 equal) add their shares, fixed tree
+          if (MODE == 2) {
+            __syncwarp();  // every row of A_ref has been read: dO over it, 64-byte rows and swizzle
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            float v = dpart[i];
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
-            v += __shfl_xor_sync(0xffffffffu, v, 2);
-            v += __shfl_xor_sync(0xffffffffu, v, 4);
-            const int rr = 4 * i + (lane >> 3);
-            const int tt = q0 + ((rbase + rr) & (RPH - 1));
-            const int64_t li = ((int64_t)b * p.Hq + h) * p.lse_pitch + tt;
-            if ((lane & 7) == 0 && tt < p.T && in_bounds(li, (int64_t)p.B * p.Hq * p.lse_pitch, p.status))
-              p.dvec[li] = v;
+            for (int v = 0; v < 4; ++v)
+              *reinterpret_cast<uint4*>(bf + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4)) =
+                  make_uint4(dw[4 * v], dw[4 * v + 1], dw[4 * v + 2], dw[4 * v + 3]);
           }
+          if (MODE != 1) tc::fence_proxy_async_smem();
+          __syncwarp();
+          if (MODE != 1) {
+            if (tc::elect_one()) {
+              // rows from T on are outside the tensor map's second dimension: not written
+              if (have && y0 < p.T)
+                tc::tma_store_3d(MODE == 0 ? &tm_a : &tm_do, bf, h * DH + ch * 32,
+                                 y0, b);
+              tc::bulk_commit_group();
+              if (MODE == 2) tc::bulk_wait_group_read<0>();
+            }
+            __syncwarp();
+          }
+          if (MODE != 0 && have) load_next();
+          ++cc;
+        };
+#pragma unroll 1
+        for (int ch = 0; ch < NCH; ++ch) {
+          uint32_t r[32];
+          __syncwarp();
+          tc::tmem_ld32(tmem + lane_base + L::O_COL + ob * DH + ch * 32, r);
+          tc::tmem_ld_wait();
+          if (ch == NCH - 1) {  // O of this buffer is read out: the next-but-one tile may use it
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&bars->o_empty[ob]);
+          }
+          process(ch, r);
         }
-        if (MODE != 1 && p.lse != nullptr && t < p.T &&
-            in_bounds(((int64_t)b * p.Hq + h) * p.lse_pitch + t, (int64_t)p.B * p.Hq * p.lse_pitch,
-                      p.status)) {
-          const int64_t li = ((int64_t)b * p.Hq + h) * p.lse_pitch + t;
-          p.lse[li] = MODE == 2 ? m + log2f(lt) : (m + log2f(lt)) * kLn2;  // mode 2: log2 units
+        if (MODE == 2 && valid) range_bits = max_abs_f16x2(range_bits, rb);
+        const int64_t li = ((int64_t)b * p.Hq + h) * p.lse_pitch + t;
+        if (MODE != 1 && valid && in_bounds(li, (int64_t)p.B * p.Hq * p.lse_pitch, p.status)) {
+          if (MODE == 2) p.dvec[li] = dd.x + dd.y;
+          // mode 2: log2 units
+          if (p.lse != nullptr) p.lse[li] = MODE == 2 ? m + log2f(lt_) : (m + log2f(lt_)) * kLn2;
         }
-        acc = (double)sq.x + (double)sq.y;
+        double acc = valid ? (double)sq.x + (double)sq.y : 0.0;
+        acc = warp_sum(acc);
+        if (lane == 0) bars->red[ob][quarter] = acc;
       }
-      acc = warp_sum(acc);
-      double* red = bars->red[tc_ & 1];  // alternate by tile
-      if (lane == 0) red[ew] = acc;
       tc::named_bar_sync(2, EPI_WARPS * 32);  // every epilogue warp reaches this once per tile
-      if (HPT == 2 && lane == 0 && (quarter & 1) == 0 && have) {
-        // head hd = row >> 6 has lane quarters 2 hd and 2 hd + 1; quarter q is epilogue warp (q + 1) & 3
-        const int hd = row >> 6;
-        const double v = red[(2 * hd + 1) & 3] + red[(2 * hd + 2) & 3];
+      if (lane == 0 && y_off == 0 && have) {  // the first warp of each head adds its warps' sums
+        const double* red = bars->red[ob] + quarter;
         const int64_t pi = (((int64_t)c * p.B + b) * p.Hq + h) * p.nP + tl.qb;
+        const double v = HPT == 2 ? red[0] + red[1] : ((red[0] + red[1]) + red[2]) + red[3];
         if (in_bounds(pi, ext_p, p.status)) p.part[pi] = v;
-      }
-      if (HPT == 1 && lane == 0 && quarter == 0 && have) {  // one head: all four lane quarters
-        const int64_t pi = (((int64_t)c * p.B + b) * p.Hq + h) * p.nP + tl.qb;
-        if (in_bounds(pi, ext_p, p.status)) p.part[pi] = ((red[0] + red[1]) + red[2]) + red[3];
       }
       if (!have) break;
     }
-    if (MODE == 2 && range_bits) report(p.status, JAB_ERR_RANGE);
+    if (MODE != 1 && tc::elect_one()) tc::bulk_wait_group<0>();
+    if (MODE != 0)  // loads that nobody waited for land before shared memory goes
+      for (int i = cc; i < issued; ++i) drain_wait(&a_full[i & 1], (i >> 1) & 1);
+    if (MODE == 2 && either_at_least(range_bits, kHalfInf)) report(p.status, JAB_ERR_RANGE);
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -667,9 +681,25 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
+// [B, T, cols] rows of a caller's or workspace tensor in boxes of 32 columns x 32 rows of one sequence
+// (what lies past T is neither read nor written).
+bool tmap_rows32(CUtensorMap* m, const void* base, bool fp32, uint64_t cols, uint64_t T, uint64_t B) {
+  const uint64_t es = fp32 ? 4 : 2;
+  cuuint64_t dims[3] = {cols, T, B};
+  cuuint64_t strides[2] = {cols * es, cols * es * T};
+  cuuint32_t box[3] = {32, 32, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return encode_fn()(m, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3,
+                     const_cast<void*>(base), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     fp32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 template <int DH, int MODE, int HPT>
-cudaError_t launch_fwd_pair(const CUtensorMap& tq, const CUtensorMap& tkv, const FwdParams& p,
-                            int grid, cudaStream_t st) {
+cudaError_t launch_fwd_pair(const CUtensorMap& tq, const CUtensorMap& tkv, const CUtensorMap& ta,
+                            const CUtensorMap& td, const FwdParams& p, int grid, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(attn_fwd_pair_kernel<DH, MODE, HPT>,
@@ -678,8 +708,8 @@ cudaError_t launch_fwd_pair(const CUtensorMap& tq, const CUtensorMap& tkv, const
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  attn_fwd_pair_kernel<DH, MODE, HPT><<<grid, Issue<DH>::kThreads, StackLayout<DH>::SMEM, st>>>(tq,
-                                                                                      tkv, p);
+  attn_fwd_pair_kernel<DH, MODE, HPT>
+      <<<grid, NUM_THREADS, StackLayout<DH>::SMEM, st>>>(tq, tkv, ta, td, p);
   return cudaGetLastError();
 }
 
@@ -706,9 +736,7 @@ cudaError_t launch_attn_fwd_tc(const AttnLaunch& L, int mode) {
   p.sl2 = L.scale * kLog2e;
   p.part = L.part;
   p.a_ref = L.a_ref;
-  p.a_out = L.a_out;
   p.lse = L.lse;
-  p.d_o = static_cast<half_t*>(L.d_o);
   p.dvec = L.dvec;
   p.status = L.status;
   p.C = L.C;
@@ -716,7 +744,11 @@ cudaError_t launch_attn_fwd_tc(const AttnLaunch& L, int mode) {
   // stacked into a tile); otherwise a tile is 128 rows of one head. Same kernel either way.
   const bool pair = (L.Hq / L.Hkv) % 2 == 0;
   const int rph = pair ? SQ : BQ;
-  CUtensorMap tq, tkv;
+  CUtensorMap tq, tkv, ta, td;
+  const uint64_t cols = (uint64_t)L.Hq * L.dh;
+  if (!tmap_rows32(&ta, mode == 0 ? L.a_out : L.a_ref, true, cols, L.T, L.B)) return cudaErrorInvalidValue;
+  td = ta;
+  if (mode == 2 && !tmap_rows32(&td, L.d_o, false, cols, L.T, L.B)) return cudaErrorInvalidValue;
   cuuint32_t box_q[2] = {64, (cuuint32_t)rph};
   cuuint32_t box_kv[2] = {64, (cuuint32_t)SKB};
   if (fn(&tq, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(L.qkv), dims, strides, box_q,
@@ -735,7 +767,7 @@ cudaError_t launch_attn_fwd_tc(const AttnLaunch& L, int mode) {
   }
   const int64_t ntiles = (int64_t)(L.Hq / (pair ? 2 : 1)) * L.B * L.C * ((L.T + rph - 1) / rph);
   const int grid = (int)std::min<int64_t>(ntiles, sms);
-#define JAB_FWD2(DH_, M_, H_) return launch_fwd_pair<DH_, M_, H_>(tq, tkv, p, grid, L.stream)
+#define JAB_FWD2(DH_, M_, H_) return launch_fwd_pair<DH_, M_, H_>(tq, tkv, ta, td, p, grid, L.stream)
   if (pair) {
     if (L.dh == 128) {
       if (mode == 0) JAB_FWD2(128, 0, 2);
