@@ -8,7 +8,8 @@
 // 128 rows of A, half of the B tile and 128 lanes of the accumulator (details above the kernel).
 //   warp 0      TMA producer: the CTA's 128x64 A tile and 128x64 half of B per stage, 6-stage ring
 //   warp 1      TMEM owner (512 columns, allocated by the pair) and, in the even CTA, UMMA issuer
-//   warps 2..5  epilogue: tcgen05.ld of the CTA's 128 x 256 fp32 accumulator, one lane per thread
+//   warps 2..5  epilogue: tcgen05.ld of the CTA's 128 x 256 fp32 accumulator, one lane per thread;
+//               the projection's fp16 results leave by TMA through two boxes per warp
 // Two accumulators (2 x 256 TMEM columns) let the epilogue of one tile overlap the next mainloop.
 //
 // Epilogues:
@@ -42,7 +43,6 @@ struct GemmParams {
   int num_m, num_n, splits, k_blocks, group_m;
   int* status;
   // projection epilogue
-  half_t* C;
   int D, n_rot, dh, T;
   const float* cos_t;
   const float* sin_t;
@@ -84,12 +84,20 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
   }
 }
 
-__device__ __forceinline__ void epi_rope(const GemmParams& p, uint32_t taddr, int mb, int nb,
-                                         int row) {
+// The projection's 128 rows x 256 columns of one CTA, RoPE applied, to fp16 C. A thread has one row, so
+// storing its registers directly is 16 bytes of 32 different rows per instruction; at K = 768 (12 K
+// blocks) that took 11.5k clocks a tile where the products take 6.1k (65536 x 9216: 735 us, now 526). The
+// warp's 32 rows x 64 columns go through a swizzled box in shared memory and leave by TMA (rows past M
+// are clipped by the tensor map). buf: the warp's two boxes.
+__device__ __forceinline__ void epi_rope(const GemmParams& p, const CUtensorMap* tmC, uint32_t taddr,
+                                         int mb, int nb, int row, uint8_t* buf) {
+  const int lane = row & 31;
   const int64_t m = (int64_t)mb * BM + row;
+  const int64_t y = m - lane;  // the warp's first row
   const bool row_ok = m < p.M;
   const int t = row_ok ? (int)(m % p.T) : 0;
   const int half = p.dh >> 1;
+  uint32_t big = 0;  // largest magnitude bits of the row's fp16 results
 #pragma unroll 1
   for (int pr = 0; pr < BN / 64; ++pr) {
     const int c1 = (p.dh == 128) ? (pr >> 1) * 4 + (pr & 1) : pr * 2;
@@ -134,30 +142,47 @@ __device__ __forceinline__ void epi_rope(const GemmParams& p, uint32_t taddr, in
         }
       }
     }
-    if (row_ok && in_bounds(m * p.Nn + col1 + half + 31, p.M * (int64_t)p.Nn, p.status)) {
-      uint4* d1 = reinterpret_cast<uint4*>(p.C + m * p.Nn + col1);
-      uint4* d2 = reinterpret_cast<uint4*>(p.C + m * p.Nn + col1 + half);
-      uint32_t inf_bits = 0;  // a half with all exponent bits set: inf (out of fp16 range) or NaN
+    // Boxes of 64 columns. d_h = 64: a and b are the halves of one box, the two boxes in turn. d_h = 128:
+    // columns c1 are in the head's first box, c2 in its second; two rounds fill both.
+    const bool wide = p.dh == 128;
+    if (tc::elect_one()) {  // (the same lane that issues the stores) the box has been read
+      if (!wide)
+        tc::bulk_wait_group_read<1>();
+      else if ((pr & 1) == 0)
+        tc::bulk_wait_group_read<0>();
+    }
+    __syncwarp();
+    uint8_t* box_a = buf + (wide ? 0 : (pr & 1) * 4096) + lane * 128;
+    uint8_t* box_b = wide ? box_a + 4096 : box_a;
+    const int ua = wide ? (pr & 1) * 4 : 0, ub = wide ? ua : 4;  // 16-byte units of the box row
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        uint4 u1, u2;
-        __half2* h1 = reinterpret_cast<__half2*>(&u1);
-        __half2* h2 = reinterpret_cast<__half2*>(&u2);
+    for (int v = 0; v < 4; ++v) {
+      uint32_t u1[4], u2[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          h1[e] = __floats2half2_rn(a[v * 8 + 2 * e], a[v * 8 + 2 * e + 1]);
-          h2[e] = __floats2half2_rn(b[v * 8 + 2 * e], b[v * 8 + 2 * e + 1]);
-        }
-        inf_bits |= half2_exp_all_ones(u1.x) | half2_exp_all_ones(u1.y) |
-                    half2_exp_all_ones(u1.z) | half2_exp_all_ones(u1.w) |
-                    half2_exp_all_ones(u2.x) | half2_exp_all_ones(u2.y) |
-                    half2_exp_all_ones(u2.z) | half2_exp_all_ones(u2.w);
-        d1[v] = u1;
-        d2[v] = u2;
+      for (int e = 0; e < 4; ++e) {
+        u1[e] = tc::pack_half2(a[v * 8 + 2 * e], a[v * 8 + 2 * e + 1]);
+        u2[e] = tc::pack_half2(b[v * 8 + 2 * e], b[v * 8 + 2 * e + 1]);
+        big = max_abs_f16x2(max_abs_f16x2(big, u1[e]), u2[e]);
       }
-      if (inf_bits) report(p.status, JAB_ERR_RANGE);
+      *reinterpret_cast<uint4*>(box_a + (((ua + v) ^ (lane & 7)) << 4)) = make_uint4(u1[0], u1[1], u1[2], u1[3]);
+      *reinterpret_cast<uint4*>(box_b + (((ub + v) ^ (lane & 7)) << 4)) = make_uint4(u2[0], u2[1], u2[2], u2[3]);
+    }
+    if (!wide || (pr & 1)) {
+      tc::fence_proxy_async_smem();
+      __syncwarp();
+      if (tc::elect_one()) {
+        if (y < p.M) {
+          const int x0 = wide ? col1 - 32 : col1;
+          tc::tma_store_2d(tmC, buf + (wide ? 0 : (pr & 1) * 4096), x0, (int32_t)y);
+          if (wide) tc::tma_store_2d(tmC, buf + 4096, x0 + 64, (int32_t)y);
+        }
+        tc::bulk_commit_group();
+      }
+      __syncwarp();
     }
   }
+  // a half with all exponent bits set: inf (out of fp16 range) or NaN
+  if (row_ok && either_at_least(big, kHalfInf)) report(p.status, JAB_ERR_RANGE);
 }
 
 // STE weight gradient (App. B: d w_hat / d w = 1, so dL/dW = dL/dw_hat = coef * dQKV^T X): the
@@ -262,23 +287,25 @@ constexpr int BM2 = 2 * BM;                 // rows of A per pair tile
 constexpr int B2_ROWS = BN / 2;             // rows (K-major) or columns (MN-major) of B per CTA
 constexpr int B2_BYTES = B2_ROWS * BK * 2;  // 16 KB
 constexpr int STAGE2_BYTES = A_BYTES + B2_BYTES;
-constexpr int SMEM2_BYTES = STAGES2 * STAGE2_BYTES + 1024 + 256;
+constexpr int EPI2_BYTES = 4 * 2 * 4096;  // two output boxes per epilogue warp
+constexpr int SMEM2_BYTES = STAGES2 * STAGE2_BYTES + EPI2_BYTES + 1024 + 256;
 
 struct Bars2 {
   uint64_t full[STAGES2], empty[STAGES2], tfull[2], tempty[2], drain;
   uint32_t tmem_base;
   int abort;
 };
-static_assert(STAGES2 * STAGE2_BYTES + (int)sizeof(Bars2) <= SMEM2_BYTES - 1024, "shared memory");
+static_assert(STAGES2 * STAGE2_BYTES + EPI2_BYTES + (int)sizeof(Bars2) <= SMEM2_BYTES - 1024, "shared memory");
+static_assert(SMEM2_BYTES <= 227 * 1024, "shared memory budget");
 
 template <int EPI, bool BF16, bool B_MN>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     gemm2_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    const GemmParams p) {
+                    const __grid_constant__ CUtensorMap tmC, const GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
-  Bars2* bars = reinterpret_cast<Bars2*>(smem + STAGES2 * STAGE2_BYTES);
+  Bars2* bars = reinterpret_cast<Bars2*>(smem + STAGES2 * STAGE2_BYTES + EPI2_BYTES);
   const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = tc::cluster_ctarank();  // 0: issues the pair's UMMAs
   const bool leader = rank == 0;
@@ -300,6 +327,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     tc::fence_mbar_init();
     tc::prefetch_tmap(&tmA);
     tc::prefetch_tmap(&tmB);
+    if (EPI == kEpiRope) tc::prefetch_tmap(&tmC);
   }
   if (warp == 1) {
     tc::tmem_alloc2(&bars->tmem_base, TMEM_COLS);
@@ -402,7 +430,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + acc * BN;
       const int mb128 = 2 * mb + (int)rank;  // this CTA's 128-row block
       if (EPI == kEpiRope)
-        epi_rope(p, taddr, mb128, nb, row);  // masks rows past M itself
+        epi_rope(p, &tmC, taddr, mb128, nb, row,  // rows past M are masked there
+                 smem + STAGES2 * STAGE2_BYTES + q * 8192);
       else if ((int64_t)mb128 * BM < p.M) {  // M is a multiple of 128: whole halves are valid or not
         if (EPI == kEpiLsq)
           epi_lsq(p, taddr, mb128, nb, ks, row);
@@ -418,6 +447,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           tc::mbar_arrive_cluster(tempty_lead + acc * 8);
       }
     }
+    if (EPI == kEpiRope && tc::elect_one()) tc::bulk_wait_group<0>();  // the stores have read their boxes
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -471,8 +501,8 @@ int sm_count() {
 
 // CTA-pair launch: clusters of two, one pair per two SMs (as many pairs as fit at once).
 template <int EPI, bool BF16, bool B_MN>
-cudaError_t launch_gemm2(const CUtensorMap& ta, const CUtensorMap& tb, GemmParams& p,
-                         cudaStream_t st) {
+cudaError_t launch_gemm2(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tcm,
+                         GemmParams& p, cudaStream_t st) {
   auto kern = gemm2_tc_kernel<EPI, BF16, B_MN>;
   static bool attr_set = false;
   if (!attr_set) {
@@ -504,7 +534,7 @@ cudaError_t launch_gemm2(const CUtensorMap& ta, const CUtensorMap& tb, GemmParam
   const int64_t total = (int64_t)p.num_m * p.num_n * p.splits;
   const int pairs = (int)std::min<int64_t>(total, std::min(clusters, sms / 2));
   cfg.gridDim = dim3((unsigned)(2 * pairs));
-  return cudaLaunchKernelEx(&cfg, kern, ta, tb, p);
+  return cudaLaunchKernelEx(&cfg, kern, ta, tb, tcm, p);
 }
 
 }  // namespace
@@ -512,8 +542,9 @@ cudaError_t launch_gemm2(const CUtensorMap& ta, const CUtensorMap& tb, GemmParam
 cudaError_t launch_proj_gemm_tc(const void* A, const void* Bw, void* C, int64_t M, int Nn, int K,
                                 int D, int n_rot, int dh, int T, const float* cos_t,
                                 const float* sin_t, int* status, cudaStream_t st) {
-  CUtensorMap ta, tb;
-  if (!make_tmap(&ta, A, false, K, M, K, BM) || !make_tmap(&tb, Bw, false, K, Nn, K, B2_ROWS))
+  CUtensorMap ta, tb, tcm;
+  if (!make_tmap(&ta, A, false, K, M, K, BM) || !make_tmap(&tb, Bw, false, K, Nn, K, B2_ROWS) ||
+      !make_tmap(&tcm, C, false, Nn, M, Nn, 32))
     return cudaErrorInvalidValue;
   GemmParams p{};
   p.M = M;
@@ -525,14 +556,13 @@ cudaError_t launch_proj_gemm_tc(const void* A, const void* Bw, void* C, int64_t 
   p.k_blocks = K / BK;
   p.group_m = 16;  // 16 pair rows = 4096 rows of X and all of W in L2 while the N tiles pass
   p.status = status;
-  p.C = static_cast<half_t*>(C);
   p.D = D;
   p.n_rot = n_rot;
   p.dh = dh;
   p.T = T;
   p.cos_t = cos_t;
   p.sin_t = sin_t;
-  return launch_gemm2<kEpiRope, false, false>(ta, tb, p, st);
+  return launch_gemm2<kEpiRope, false, false>(ta, tb, tcm, p, st);
 }
 
 // Split K so that the units (tile x K range) fill whole waves of the persistent grid: the makespan
@@ -580,7 +610,7 @@ cudaError_t launch_wgrad_lsq_tc(const void* dqkvt, int64_t ldt, const void* x, c
   p.dspart = dspart;
   // every (split, row, group) partial is written once; the splits are summed in order: the scale
   // gradient is bit-identical between calls
-  cudaError_t e = launch_gemm2<kEpiLsq, true, true>(ta, tb, p, st);
+  cudaError_t e = launch_gemm2<kEpiLsq, true, true>(ta, tb, ta, p, st);
   if (e != cudaSuccess) return e;
   return launch_split_sum(dspart, p.splits, (int64_t)D * (d / G), ds, st);
 }
@@ -613,7 +643,7 @@ cudaError_t launch_wgrad_store_tc(const void* dqkvt, int64_t ldt, const void* x,
     e = cudaMemsetAsync(target, 0, (size_t)n_w * sizeof(float), st);
     if (e != cudaSuccess) return e;
   }
-  e = launch_gemm2<kEpiStore, true, true>(ta, tb, p, st);
+  e = launch_gemm2<kEpiStore, true, true>(ta, tb, ta, p, st);
   if (e != cudaSuccess || sqnorm == nullptr) return e;
   return launch_sumsq(target, n_w, red, sqnorm, st);  // fixed order
 }
