@@ -79,7 +79,7 @@ __device__ __forceinline__ bool either_at_least(uint32_t m2, uint32_t limit) {
   return (m2 & 0xffffu) >= limit || (m2 >> 16) >= limit;
 }
 constexpr uint32_t kBf16Inf = 0x7f80u, kHalfInf = 0x7c00u;
-constexpr uint32_t kBf16TwoTo60 = 187u << 7;
+constexpr uint32_t kBf16TwoTo60 = 187u << 7, kBf16TwoToM60 = 67u << 7;
 
 __device__ __forceinline__ double warp_sum(double x) {
 #pragma unroll

@@ -221,6 +221,59 @@ __device__ __forceinline__ void epi_store(const GemmParams& p, uint32_t taddr, i
   }
 }
 
+// Sum over 32 columns of G[o, i] r(w_i, sc) with the LSQ factor of Eq. 13. g: this row's columns of G, w: the
+// 32 bf16 weights. The quotient in packed pairs from a corrected reciprocal where that is the IEEE one
+// (see quot_window), by division elsewhere: with 32 divisions a chunk took 3k clocks, and small
+// batches waited for the epilogue (512 tokens x 2304 x 768: 20.6 us).
+__device__ __forceinline__ float lsq_chunk(const uint32_t (&g)[32], const uint4 (&w)[4], float sc, int qmax) {
+  uint32_t big = 0, small = 0xffffffffu;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const uint32_t x[4] = {w[v].x, w[v].y, w[v].z, w[v].w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const uint32_t m = x[e] & 0x7fff7fffu;
+      big = __vmaxu2(big, m);
+      small = __vminu2(small, m);  // (a zero weight takes the division too)
+    }
+  }
+  const bool fast = quot_window(sc) && !either_at_least(big, kBf16TwoTo60) &&
+                    (small & 0xffffu) >= kBf16TwoToM60 && (small >> 16) >= kBf16TwoToM60;
+  float2 acc = make_float2(0.f, 0.f);
+  if (fast) {
+    const float r = __frcp_rn(sc), qm = (float)qmax;
+    const float2 r2 = make_float2(r, r), ns2 = make_float2(-sc, -sc);
+    const float2 magic = make_float2(12582912.f, 12582912.f);  // 1.5 * 2^23: rounds half to even
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const uint32_t x[4] = {w[v].x, w[v].y, w[v].z, w[v].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 wv = make_float2(__uint_as_float(x[e] << 16), __uint_as_float(x[e] & 0xffff0000u));
+        const float2 v0 = tc::mul2(wv, r2);
+        const float2 q = tc::fma2(tc::fma2(v0, ns2, wv), r2, v0);  // fl32(w / s)
+        // q clipped to +-qmax (whole); inside, its rounding error is the factor, else the bound itself
+        const float2 c = make_float2(fminf(fmaxf(q.x, -qm), qm), fminf(fmaxf(q.y, -qm), qm));
+        const float2 d = tc::sub2(tc::sub2(tc::add2(c, magic), magic), q);
+        const float2 f = make_float2(c.x == q.x ? d.x : c.x, c.y == q.y ? d.y : c.y);
+        const int i = 8 * v + 2 * e;
+        acc = tc::fma2(make_float2(__uint_as_float(g[i]), __uint_as_float(g[i + 1])), f, acc);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const bf16_t* wb = reinterpret_cast<const bf16_t*>(&w[v]);
+#pragma unroll
+      for (int e = 0; e < 8; e += 2) {
+        acc.x = fmaf(__uint_as_float(g[v * 8 + e]), lsq_factor(__bfloat162float(wb[e]), sc, qmax), acc.x);
+        acc.y = fmaf(__uint_as_float(g[v * 8 + e + 1]), lsq_factor(__bfloat162float(wb[e + 1]), sc, qmax), acc.y);
+      }
+    }
+  }
+  return acc.x + acc.y;
+}
+
 __device__ __forceinline__ void epi_lsq(const GemmParams& p, uint32_t taddr, int mb, int nb,
                                         int ks, int row) {
   const int o = mb * BM + row;  // M = D is a multiple of 128: every row is valid
@@ -231,6 +284,22 @@ __device__ __forceinline__ void epi_lsq(const GemmParams& p, uint32_t taddr, int
   const int64_t part_extent = (int64_t)p.splits * p.M * ng;
   float part = 0.f;
   int cur = -1;
+  // The weights and scale of a chunk are loaded while the one before it is summed.
+  uint4 wn[4];
+  float sn = 0.f;
+  auto load = [&](int c) {
+    const int i0 = nb * BN + c * 32;
+    if (c < BN / 32 && i0 < p.Nn && in_bounds((int64_t)o * p.d + i0 + 31, (int64_t)p.M * p.d, p.status) &&
+        in_bounds((int64_t)o * ng + i0 / p.G, (int64_t)p.M * ng, p.status)) {
+      const uint4* wp = reinterpret_cast<const uint4*>(p.w + (int64_t)o * p.d + i0);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) wn[v] = __ldg(wp + v);
+      sn = __ldg(p.s + (int64_t)o * ng + i0 / p.G);
+    }
+  };
+#pragma unroll
+  for (int v = 0; v < 4; ++v) wn[v] = make_uint4(0u, 0u, 0u, 0u);
+  load(0);
 #pragma unroll 1
   for (int c = 0; c < BN / 32; ++c) {
     const int i0 = nb * BN + c * 32;
@@ -238,30 +307,18 @@ __device__ __forceinline__ void epi_lsq(const GemmParams& p, uint32_t taddr, int
     uint32_t r[32];
     __syncwarp();
     tc::tmem_ld32(taddr + c * 32, r);
+    const uint4 w[4] = {wn[0], wn[1], wn[2], wn[3]};
+    const float sc = sn;
+    load(c + 1);
     tc::tmem_ld_wait();
     const int g = i0 / p.G;
-    float acc = 0.f;
-    if (in_bounds((int64_t)o * p.d + i0 + 31, (int64_t)p.M * p.d, p.status) &&
-        in_bounds((int64_t)o * ng + g, (int64_t)p.M * ng, p.status)) {
-      const float sc = __ldg(p.s + (int64_t)o * ng + g);
-      const uint4* wp = reinterpret_cast<const uint4*>(p.w + (int64_t)o * p.d + i0);
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const uint4 u = __ldg(wp + v);
-        const bf16_t* wb = reinterpret_cast<const bf16_t*>(&u);
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          acc = fmaf(__uint_as_float(r[v * 8 + e]), lsq_factor(__bfloat162float(wb[e]), sc, qmax),
-                     acc);
-      }
-    }
     if (g != cur) {
       if (cur >= 0 && in_bounds(((int64_t)ks * p.M + o) * ng + cur, part_extent, p.status))
         part_out[cur] = p.coef * part;
       part = 0.f;
       cur = g;
     }
-    part += acc;
+    part += lsq_chunk(r, w, sc, qmax);
   }
   if (cur >= 0 && in_bounds(((int64_t)ks * p.M + o) * ng + cur, part_extent, p.status))
     part_out[cur] = p.coef * part;

@@ -117,3 +117,28 @@ def test_ten_candidates_in_one_call_equal_single_calls(shape, T):
         J().jab_loss_forward(c.desc, c.B, c.T, c.X, c.W, A, bits[i:i + 1], scales[i:i + 1], one, ws)
         assert one.item() == loss[i].item(), i
     assert J().jab_get_device_status() == 0
+
+
+def test_scale_gradient_where_the_quotient_takes_the_division():
+    """Chunks with zero weights and groups of tiny ones (quotients outside the corrected reciprocal's
+    window): the LSQ factor of the weight-gradient epilogue against the oracle's."""
+    from dataclasses import replace
+    from tests.harness import COS_MIN, Case, cosine
+    from workloads import WORKLOADS
+    c = Case(replace(WORKLOADS["gpt2_smoke"], shape=BlockShape(256, 4, 1, 64, True, 500.0)), 2, 65, 64)
+    g = torch.Generator().manual_seed(2)
+    w = c.W.float().cpu()
+    w[torch.rand(w.shape, generator=g) < 0.02] = 0
+    w[:, 64:128] *= 1e-25
+    w = w.to(torch.bfloat16)
+    s = (torch.rand((c.D, 4), generator=g) * 0.02 + 0.01).numpy()
+    W, S = w.cuda(), torch.from_numpy(s).cuda()
+    ws = c.workspace()
+    A = torch.empty((c.B, c.T, c.Hq * c.dh), dtype=torch.float32, device="cuda")
+    J().jab_reference_forward(c.desc, c.B, c.T, c.X, W, A, ws)
+    loss = torch.empty(1, dtype=torch.float64, device="cuda")
+    grad = torch.empty_like(S)
+    J().jab_loss_backward_scales(c.desc, c.B, c.T, c.X, W, A, 3, S, 1.0, loss, grad, ws)
+    r = O.jab_loss_and_grad(c.x64, np64(w), s, 3, c.odesc, kappa=1.0)
+    assert cosine(grad.cpu().numpy(), r["grad_s"]) >= COS_MIN
+    assert J().jab_get_device_status() == 0
