@@ -8,7 +8,7 @@
 // Two kernels, no atomics:
 //   dkdv  one CTA per (128-key block, KV head, sequence); loops over the query heads of the group and
 //         over 128-query blocks: S^T = K Q^T, dP^T = V dO^T into TMEM, P^T and dS^T (fp16) written
-//         back over them by 16 elementwise warps (16 key rows x 64 queries each), dV += P^T dO and
+//         back to TMEM by 16 elementwise warps (16 key rows x 64 queries each), dV += P^T dO and
 //         dK += dS^T Q (A operands in TMEM) accumulated in TMEM. Each dS^T tile is also staged in
 //         shared memory and stored to HBM by TMA (a store warp).
 //   dq    persistent, (128 query rows, query head, sequence) tiles: dQ = scale * sum_kb dS K from the
@@ -58,17 +58,38 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
     if (tc::globaltimer() - t0 > tc::kWaitLimitNs) break;
 }
 
+// Row pitch (elements) of a staged gradient tile [dim][128 token rows]: 16 bytes beyond the rows, so that
+// the eight rows of a transposed 8 x 8 store lie in different banks.
+constexpr int GRAD_PITCH = 136;
+
+// Four 8 x 8 16-bit matrices to shared memory, transposed: thread t holds, of each, row t / 4 and columns
+// 2 (t % 4), + 1 packed in r[m]; lane 8 m + i gives the address of column i's 8 values of matrix m.
+__device__ __forceinline__ void stmatrix_x4_trans(const void* addr, const uint32_t (&r)[4]) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(
+                   tc::smem_u32(addr)),
+               "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3])
+               : "memory");
+}
+
 // Stages gradient rows of a TMEM accumulator (DH columns), times `mul`, optionally through the
-// transpose of RoPE, into tile[dim][row] (bf16, 128 rows per dim). The calling warp handles the 16
-// TMEM lanes addressed by `taddr` with the 16x256b shape: thread t holds rows row_a = first + t / 4
-// and row_a + 8 and, in each 8-column group, the column pair 2 (t % 4), so the four threads of a row
-// read 32 contiguous bytes of a cos / sin table row (pos_a, pos_b: table rows of row_a, row_a + 8).
+// transpose of RoPE, into tile[dim][row] (bf16, GRAD_PITCH per dim). The calling warp handles the 16
+// TMEM lanes addressed by `taddr`, tile rows row0 .. row0 + 15, with the 16x256b shape: thread t holds
+// rows row0 + t / 4 and 8 further on and, in each 8-column group, the column pair 2 (t % 4), so the four
+// threads of a row read 32 contiguous bytes of a cos / sin table row (pos_a, pos_b: table rows of the
+// two). Eight columns of 16 rows of both halves of the head go out as one transposing matrix store, where
+// two-byte stores hit each bank four times (dK/dV of 3 x 1337 tokens 126 -> 124 us, dq 60 -> 58 us).
 template <int DH>
 __device__ __forceinline__ void stage_grad_16(uint32_t taddr, float mul, bool rope, int pos_a,
                                               int pos_b, const float* cos_t, const float* sin_t,
-                                              bf16_t* tile, int row_a) {
+                                              bf16_t* tile, int row0) {
   constexpr int HALF = DH / 2;
-  const int cq = threadIdx.x & 3;
+  const int lane = threadIdx.x & 31, cq = lane & 3;
+  // this lane's address of matrices (first half, rows 0..7), (first, 8..15), (second, 0..7), (second, 8..15)
+  bf16_t* at = tile + ((lane >> 4) * HALF + (lane & 7)) * GRAD_PITCH + row0 + ((lane >> 3) & 1) * 8;
+  auto pack = [](float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+  };
 #pragma unroll 1
   for (int c = 0; c < HALF / 32; ++c) {
     uint32_t r1[16], r2[16];
@@ -87,30 +108,30 @@ __device__ __forceinline__ void stage_grad_16(uint32_t taddr, float mul, bool ro
         cb = __ldg(reinterpret_cast<const float2*>(cos_t + (int64_t)pos_b * HALF + j0));
         sb = __ldg(reinterpret_cast<const float2*>(sin_t + (int64_t)pos_b * HALF + j0));
       }
+      float a1[2], a2[2], b1[2], b2[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         const float csa = e ? ca.y : ca.x, sna = e ? sa.y : sa.x;
         const float csb = e ? cb.y : cb.x, snb = e ? sb.y : sb.x;
-        float a1 = __uint_as_float(r1[4 * n + e]) * mul, a2 = __uint_as_float(r2[4 * n + e]) * mul;
-        float b1 = __uint_as_float(r1[4 * n + 2 + e]) * mul;
-        float b2 = __uint_as_float(r2[4 * n + 2 + e]) * mul;
+        a1[e] = __uint_as_float(r1[4 * n + e]) * mul;
+        a2[e] = __uint_as_float(r2[4 * n + e]) * mul;
+        b1[e] = __uint_as_float(r1[4 * n + 2 + e]) * mul;
+        b2[e] = __uint_as_float(r2[4 * n + 2 + e]) * mul;
         if (rope) {
-          const float x1 = a1, x2 = a2, y1 = b1, y2 = b2;
-          a1 = x1 * csa + x2 * sna;
-          a2 = x2 * csa - x1 * sna;
-          b1 = y1 * csb + y2 * snb;
-          b2 = y2 * csb - y1 * snb;
+          const float x1 = a1[e], x2 = a2[e], y1 = b1[e], y2 = b2[e];
+          a1[e] = x1 * csa + x2 * sna;
+          a2[e] = x2 * csa - x1 * sna;
+          b1[e] = y1 * csb + y2 * snb;
+          b2[e] = y2 * csb - y1 * snb;
         }
-        tile[(j0 + e) * 128 + row_a] = __float2bfloat16_rn(a1);
-        tile[(HALF + j0 + e) * 128 + row_a] = __float2bfloat16_rn(a2);
-        tile[(j0 + e) * 128 + row_a + 8] = __float2bfloat16_rn(b1);
-        tile[(HALF + j0 + e) * 128 + row_a + 8] = __float2bfloat16_rn(b2);
       }
+      const uint32_t w[4] = {pack(a1[0], a1[1]), pack(b1[0], b1[1]), pack(a2[0], a2[1]), pack(b2[0], b2[1])};
+      stmatrix_x4_trans(at + (c * 32 + 8 * n) * GRAD_PITCH, w);
     }
   }
 }
 
-// Cooperative store of tile[DH][128] to dst[d * ldt + n0 + r] for r < nvalid: 16-byte vectors when
+// Cooperative store of tile[DH][GRAD_PITCH] to dst[d * ldt + n0 + r] for r < nvalid: 16-byte vectors when
 // the token offset is 8-aligned (consecutive threads cover consecutive 16-byte chunks of a dim
 // row), element-wise otherwise.
 template <int DH>
@@ -124,15 +145,15 @@ __device__ __forceinline__ void store_tile(const bf16_t* tile, bf16_t* dst, int6
       bf16_t* o = dst + (int64_t)d * ldt + n0 + r0;
       if (!in_bounds((o - base) + min(8, nvalid - r0) - 1, extent, status)) continue;
       if (r0 + 8 <= nvalid)
-        *reinterpret_cast<uint4*>(o) = *reinterpret_cast<const uint4*>(tile + d * 128 + r0);
+        *reinterpret_cast<uint4*>(o) = *reinterpret_cast<const uint4*>(tile + d * GRAD_PITCH + r0);
       else
-        for (int r = r0; r < nvalid; ++r) o[r - r0] = tile[d * 128 + r];
+        for (int r = r0; r < nvalid; ++r) o[r - r0] = tile[d * GRAD_PITCH + r];
     }
   } else {
     for (int idx = tid; idx < DH * 128; idx += nthreads) {
       const int d = idx >> 7, r = idx & 127;
       if (r < nvalid && in_bounds((dst - base) + (int64_t)d * ldt + n0 + r, extent, status))
-        dst[(int64_t)d * ldt + n0 + r] = tile[d * 128 + r];
+        dst[(int64_t)d * ldt + n0 + r] = tile[d * GRAD_PITCH + r];
     }
   }
 }
@@ -140,48 +161,53 @@ __device__ __forceinline__ void store_tile(const bf16_t* tile, bf16_t* dst, int6
 // ================================================================================ dK, dV
 // One CTA per (128-key block, KV head, sequence); it loops over the query heads of the group and over
 // 128-query blocks, so that every UMMA runs at N = 128 (an N = 64 UMMA costs the tensor pipe as much
-// time as an N = 128 one). Tensor memory: S^T = K Q^T at column 0 and dP^T = V dO^T at 128 (SS form:
-// K and V stay in shared memory for the whole tile), dV at 256, dK at 256 + DH. The elementwise warps
-// write P^T and dS^T back as packed fp16 into S^T and dP^T, where the TS-form gradient UMMAs
-// dV += P^T dO and dK += dS^T Q read them as their A operand: the 64 queries of half h (whose fp32
-// scores are columns 64 h .. 64 h + 63, read by the warps of that half) go to packed columns
-// 64 h .. 64 h + 31, so a warp writes only columns that it has itself read (warps of the two halves
-// are not synchronised with each other). With no room for a second
-// S^T / dP^T buffer, S^T(j+1) goes out once dV(j) has completed (it overwrites the P^T(j) columns)
-// and dP^T(j+1) once dK(j) has; the elementwise warps compute P^T(j+1) while dK(j) and dP^T(j+1)
-// run. The score products (S^T, dP^T) and the gradient products (dV, dK) are issued by two threads,
-// so that neither waits behind the issue of the other; dK(j) enters the pipe only after S^T(j+1)
-// has been issued, since the elementwise warps wait for S^T(j+1) and nothing waits for dK(j) sooner.
+// time as an N = 128 one). Tensor memory: one score buffer X (columns 0 .. 127) that S^T = K Q^T and
+// dP^T = V dO^T use in turn (SS form: K and V stay in shared memory for the whole tile), P^T at 128 and
+// dS^T at 192 (packed fp16, 64 columns each), dV at 256, dK at 256 + DH. The elementwise warps read a
+// score block out into registers at once, after which the other product may overwrite X:
+//   S^T(j) read -> dP^T(j) issued, while P^T(j) is computed from the registers
+//   dP^T(j) read -> S^T(j+1) issued, while dS^T(j) is computed and staged
+// and the TS-form gradient UMMAs dV += P^T dO and dK += dS^T Q read P^T and dS^T from columns of their own,
+// so the elementwise warps never wait for a product behind the one they feed. With P^T and dS^T written
+// over their scores, S^T(j+1) waited for dV(j), 700 of 3300 clocks a block (8 x 2048 tokens: 481 -> 472 us,
+// with the KL term 805 -> 764 us). What bounds it now is the elementwise warps' own chain of reading,
+// exponentials, stores and hand-offs, about 3000 clocks a block against 2048 of products. The 64
+// queries of half h go to packed columns 32 h .. 32 h + 31 of each. The score products and the gradient
+// products are issued by two threads, so that neither waits behind the issue of the other.
 
-// TMEM column of the K-step k (queries 16 k .. 16 k + 15) of packed P^T or dS^T.
-__device__ __forceinline__ uint32_t pk_col(int k) { return (uint32_t)((k >> 2) * 64 + (k & 3) * 8); }
+// Offset of the K-step k (queries 16 k .. 16 k + 15) of packed P^T or dS^T.
+__device__ __forceinline__ uint32_t pk_col(int k) { return (uint32_t)(k * 8); }
 
 template <int DH>
 struct DkdvLayout {
-  static constexpr int BK = 128, BQ = 128, STAGES = 2;
-  static constexpr int PREFETCH = 2;  // blocks beyond the stage ring kept in flight to L2
+  // Q is read by S^T at a block's start and by dK at its end, dO by dP^T and dV in between: Q has a ring of
+  // three, dO one slot that dV(j) frees long before dP^T(j+1) needs it. (With two stages of both, the
+  // next Q could only be asked for when dK of the block two back was done, and its 64 KB stage came
+  // 1500 clocks late.)
+  static constexpr int BK = 128, BQ = 128, QST = 3;
+  static constexpr int PREFETCH = 3;  // blocks ahead brought into L2
   static constexpr int CHUNK = 128 * 128;  // 64 columns of a 128-row fp16 tile
   static constexpr int NCH = DH / 64;
   static constexpr int K_OFF = 0, V_OFF = NCH * CHUNK;
-  static constexpr int ST_OFF = 2 * NCH * CHUNK;
-  static constexpr int ST_Q = 0, ST_DO = NCH * CHUNK, ST_LSE = 2 * NCH * CHUNK,
-                       ST_D = ST_LSE + BQ * 4, ST_BYTES = ST_D + BQ * 4;
-  static constexpr int ST_STRIDE = (ST_BYTES + 1023) / 1024 * 1024;
-  static constexpr int DSS_OFF = ST_OFF + STAGES * ST_STRIDE;  // dS^T staging: two 64-query halves
-  static constexpr int BAR_OFF = DSS_OFF + 2 * CHUNK;
+  static constexpr int Q_OFF = 2 * NCH * CHUNK;
+  static constexpr int DO_OFF = Q_OFF + QST * NCH * CHUNK;
+  static constexpr int DSS_OFF = DO_OFF + NCH * CHUNK;  // dS^T staging: two 64-query halves
+  static constexpr int ROW_OFF = DSS_OFF + 2 * CHUNK;   // lse and D rows of two blocks
+  static constexpr int ROW_BYTES = 2 * BQ * 4;
+  static constexpr int BAR_OFF = ROW_OFF + 2 * ROW_BYTES;
   // No slack for aligning the base: the kernel checks that it is 1024-byte aligned (it is, after the
   // per-CTA reserved shared memory) and returns with JAB_ERR_INTERNAL otherwise.
   static constexpr int USED = BAR_OFF + 256;
   static constexpr int SMEM = USED > 118 * 1024 ? USED : 118 * 1024;
-  static constexpr uint32_t S_COL = 0, DP_COL = 128, DV_COL = 256, DK_COL = 256 + DH;
+  static constexpr uint32_t X_COL = 0, P_COL = 128, DS_COL = 192, DV_COL = 256, DK_COL = 256 + DH;
   static_assert(DK_COL + DH <= 512, "TMEM budget");
-  static_assert(2 * DH * 128 * 2 <= STAGES * ST_STRIDE, "epilogue staging fits the stage ring");
+  static_assert(2 * DH * GRAD_PITCH * 2 <= QST * NCH * CHUNK, "epilogue staging fits the Q ring");
   static_assert(USED <= 227 * 1024, "shared memory budget");
 };
 
 struct DkdvBars {
-  uint64_t kv_full, ld_full[2], ld_empty[2], s_full, dp_full, p_full, ds_full, dv_done, dk_done;
-  uint64_t o_full, drain, drain_g, dss_full, dss_free, s_issued, pt_full;
+  uint64_t kv_full, q_full[3], q_empty[3], do_full, do_empty, row_full[2], row_empty[2], s_full, s_read, dp_full, dp_read, p_full, ds_full;
+  uint64_t dv_done, dk_done, o_full, drain, drain_g, dss_full, dss_free, pt_full;
   uint32_t tmem_base;
   int abort;
 };
@@ -196,7 +222,7 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
                             const __grid_constant__ CUtensorMap tm_do,
                             const __grid_constant__ CUtensorMap tm_ds, const BwdParams p) {
   using L = DkdvLayout<DH>;
-  constexpr int BK = L::BK, BQ = L::BQ, STAGES = L::STAGES;
+  constexpr int BK = L::BK, BQ = L::BQ, QST = L::QST;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   if (tc::smem_u32(smem_raw) & 1023u) {  // the swizzled TMA tiles need a 1024-byte aligned base
     if (threadIdx.x == 0) report(p.status, JAB_ERR_INTERNAL);
@@ -229,12 +255,20 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
 
   if (threadIdx.x == 0) {
     tc::mbar_init(&bars->kv_full, 1);
-    for (int i = 0; i < STAGES; ++i) {
-      tc::mbar_init(&bars->ld_full[i], 1);
-      tc::mbar_init(&bars->ld_empty[i], 1);
+    for (int i = 0; i < QST; ++i) {
+      tc::mbar_init(&bars->q_full[i], 1);
+      tc::mbar_init(&bars->q_empty[i], 1);
+    }
+    tc::mbar_init(&bars->do_full, 1);
+    tc::mbar_init(&bars->do_empty, 2);  // dP^T and dV, committed by two threads
+    for (int i = 0; i < 2; ++i) {
+      tc::mbar_init(&bars->row_full[i], 1);
+      tc::mbar_init(&bars->row_empty[i], 1);
     }
     tc::mbar_init(&bars->s_full, 1);
     tc::mbar_init(&bars->dp_full, 1);
+    tc::mbar_init(&bars->s_read, DKDV_EW);
+    tc::mbar_init(&bars->dp_read, DKDV_EW);
     tc::mbar_init(&bars->p_full, DKDV_EW);
     tc::mbar_init(&bars->ds_full, DKDV_EW);
     tc::mbar_init(&bars->dv_done, 1);
@@ -242,7 +276,6 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
     tc::mbar_init(&bars->o_full, 1);
     tc::mbar_init(&bars->drain, 1);
     tc::mbar_init(&bars->drain_g, 1);
-    tc::mbar_init(&bars->s_issued, 1);
     tc::mbar_init(&bars->dss_full, DKDV_EW);  // the block's dS^T is in the staging tile
     tc::mbar_init(&bars->dss_free, 1);         // the store warp's TMA stores have read it
     tc::mbar_init(&bars->pt_full, 1);          // KL: the block's P^T tile is in the staging tile
@@ -263,7 +296,6 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
 
   if (warp == 0) {
     if (tc::elect_one()) {  // ------------------------------------------------------------- TMA
-      uint32_t issued = 0, last_par = 0;
       tc::mbar_expect_tx(&bars->kv_full, 2 * BK * DH * 2);
       for (int ch = 0; ch < L::NCH; ++ch) {
         tc::tma_load_2d(smem + L::K_OFF + ch * L::CHUNK, &tm_qkv, &bars->kv_full,
@@ -271,8 +303,7 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
         tc::tma_load_2d(smem + L::V_OFF + ch * L::CHUNK, &tm_qkv, &bars->kv_full,
                         p.vcol0 + g * DH + ch * 64, row0 + kb * BK);
       }
-      // The stage ring holds two blocks; blocks further ahead are prefetched into L2 so that a
-      // stage load, which can start only when dK of the block two back has completed, hits L2.
+      // Blocks further ahead than the slots are prefetched into L2, so that the loads hit there.
       auto prefetch = [&](int j) {
         const int hj = g * r + j / per_head, ij = kb + j % per_head;
         for (int ch = 0; ch < L::NCH; ++ch) {
@@ -288,111 +319,129 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
           tc::tma_prefetch_2d(&tm_ds, 64, (int32_t)(tile * BK));
         }
       };
-      for (int j = STAGES; j < STAGES + L::PREFETCH - 1 && j < n_it; ++j) prefetch(j);
+      int nq_ = 0, nr = 0, nd = 0;  // Q, row and dO loads issued
+      int st = 0;
+      uint32_t ph = 0;
+      for (int j = 1; j < L::PREFETCH && j < n_it; ++j) prefetch(j);
       for (int it = 0; it < n_it; ++it) {
-        const int st = it % STAGES;
-        const uint32_t ph = (it / STAGES) & 1;
         const int h = g * r + it / per_head, i = kb + it % per_head;
-        if (it + STAGES + L::PREFETCH - 1 < n_it) prefetch(it + STAGES + L::PREFETCH - 1);
-        if (!tc::mbar_wait(&bars->ld_empty[st], ph ^ 1, abort, p.status)) break;
-        uint8_t* sbase = smem + L::ST_OFF + st * L::ST_STRIDE;
-        tc::mbar_expect_tx(&bars->ld_full[st], L::ST_BYTES);
-        for (int ch = 0; ch < L::NCH; ++ch) {
-          tc::tma_load_2d(sbase + L::ST_Q + ch * L::CHUNK, &tm_qkv, &bars->ld_full[st],
+        if (it + L::PREFETCH < n_it) prefetch(it + L::PREFETCH);
+        if (!tc::mbar_wait(&bars->q_empty[st], ph ^ 1, abort, p.status)) break;
+        tc::mbar_expect_tx(&bars->q_full[st], BQ * DH * 2);
+        for (int ch = 0; ch < L::NCH; ++ch)
+          tc::tma_load_2d(smem + L::Q_OFF + (st * L::NCH + ch) * L::CHUNK, &tm_qkv, &bars->q_full[st],
                           p.qcol0 + h * DH + ch * 64, row0 + i * BQ);
-          tc::tma_load_2d(sbase + L::ST_DO + ch * L::CHUNK, &tm_do, &bars->ld_full[st],
-                          h * DH + ch * 64, row0 + i * BQ);
-        }
+        ++nq_;
+        if (!tc::mbar_wait(&bars->row_empty[it & 1], ((it >> 1) & 1) ^ 1, abort, p.status)) break;
+        uint8_t* rows = smem + L::ROW_OFF + (it & 1) * L::ROW_BYTES;
         const int64_t lrow = ((int64_t)b * p.Hq + h) * p.lse_pitch + i * BQ;
-        // (checked build: a failed test leaves the stage incomplete; its consumers' bounded waits
-        // then give up and the kernel returns with the status raised)
+        tc::mbar_expect_tx(&bars->row_full[it & 1], L::ROW_BYTES);
+        // (checked build: a failed test leaves the rows incomplete; their readers' bounded waits then
+        // give up and the kernel returns with the status raised)
         if (in_bounds(lrow + BQ - 1, (int64_t)p.B * p.Hq * p.lse_pitch, p.status)) {
-          tc::bulk_load(sbase + L::ST_LSE, p.lse + lrow, BQ * 4, &bars->ld_full[st]);
-          tc::bulk_load(sbase + L::ST_D, p.dvec + lrow, BQ * 4, &bars->ld_full[st]);
+          tc::bulk_load(rows, p.lse + lrow, BQ * 4, &bars->row_full[it & 1]);
+          tc::bulk_load(rows + BQ * 4, p.dvec + lrow, BQ * 4, &bars->row_full[it & 1]);
         }
-        issued |= 1u << st;
-        last_par = (last_par & ~(1u << st)) | (ph << st);
+        ++nr;
+        if (!tc::mbar_wait(&bars->do_empty, (it & 1) ^ 1, abort, p.status)) break;
+        tc::mbar_expect_tx(&bars->do_full, BQ * DH * 2);
+        for (int ch = 0; ch < L::NCH; ++ch)
+          tc::tma_load_2d(smem + L::DO_OFF + ch * L::CHUNK, &tm_do, &bars->do_full, h * DH + ch * 64,
+                          row0 + i * BQ);
+        ++nd;
+        if (++st == QST) {
+          st = 0;
+          ph ^= 1;
+        }
       }
-      if (*abort) {
+      if (*abort) {  // every copy issued lands before shared memory goes
         drain_wait(&bars->kv_full, 0);
-        for (int st = 0; st < STAGES; ++st)
-          if (issued & (1u << st)) drain_wait(&bars->ld_full[st], (last_par >> st) & 1);
+        for (int q = max(0, nq_ - QST); q < nq_; ++q) drain_wait(&bars->q_full[q % QST], (q / QST) & 1);
+        for (int q = max(0, nr - 2); q < nr; ++q) drain_wait(&bars->row_full[q & 1], (q >> 1) & 1);
+        if (nd > 0) drain_wait(&bars->do_full, (nd - 1) & 1);
       }
     }
   } else if (warp == 1 || warp == DKDV_GRAD_WARP) {
     if (tc::elect_one()) {  // ------------------- UMMA: S^T, dP^T (warp 1); dV, dK (DKDV_GRAD_WARP)
-      // Two issuing threads, so that the score products of the next block are never held back
-      // behind the issue of this block's gradient products, nor the other way round. Every
-      // dependency between them goes through a barrier: S^T(j) overwrites P^T(j - 1), so it waits
-      // for dV(j - 1); dP^T(j) overwrites dS^T(j - 1), so it waits for dK(j - 1).
       constexpr uint32_t ID_S = tc::idesc_f16(false, BK, BQ);
       constexpr uint32_t ID_G = tc::idesc_f16(false, BK, DH) | (1u << 16);  // B MN-major
       bool ok = tc::mbar_wait(&bars->kv_full, 0, abort, p.status);
       if (warp == 1) {
         const uint64_t ka = tc::sdesc_kmajor_sw128(tc::smem_u32(smem + L::K_OFF));
         const uint64_t va = tc::sdesc_kmajor_sw128(tc::smem_u32(smem + L::V_OFF));
+        const uint64_t bq0 = tc::sdesc_kmajor_sw128(tc::smem_u32(smem + L::Q_OFF));
+        const uint64_t bd = tc::sdesc_kmajor_sw128(tc::smem_u32(smem + L::DO_OFF));
+        int st = 0;
+        uint32_t ph = 0;
         for (int j = 0; ok && j < n_it; ++j) {
-          const int st = j % STAGES;
-          // S^T(j) = K Q(j)^T: its Q has landed and dV(j - 1) has read P^T(j - 1).
-          ok = tc::mbar_wait(&bars->ld_full[st], (j / STAGES) & 1, abort, p.status) &&
-               (j == 0 || tc::mbar_wait(&bars->dv_done, (j - 1) & 1, abort, p.status));
+          // S^T(j) = K Q(j)^T: its Q has landed, dP^T(j - 1) has been read out of X and dV(j - 1) has read
+          // P^T(j - 1): whoever has seen S^T(j) may write P^T(j). (Waits of the one issuing thread,
+          // satisfied by then, in place of one more of every elementwise warp.)
+          ok = tc::mbar_wait(&bars->q_full[st], ph, abort, p.status) &&
+               (j == 0 || (tc::mbar_wait(&bars->dp_read, (j - 1) & 1, abort, p.status) &&
+                           tc::mbar_wait(&bars->dv_done, (j - 1) & 1, abort, p.status)));
           if (!ok) break;
           tc::fence_after_sync();
-          const uint64_t bq = tc::sdesc_kmajor_sw128(
-              tc::smem_u32(smem + L::ST_OFF + st * L::ST_STRIDE + L::ST_Q));
+          const uint64_t bq = tc::sdesc_advance(bq0, st * L::NCH * L::CHUNK);
 #pragma unroll
           for (int k = 0; k < DH / 16; ++k) {
             const uint32_t o = (k >> 2) * L::CHUNK + (k & 3) * 32;
-            tc::umma_f16(tmem + L::S_COL, tc::sdesc_advance(ka, o), tc::sdesc_advance(bq, o), ID_S,
+            tc::umma_f16(tmem + L::X_COL, tc::sdesc_advance(ka, o), tc::sdesc_advance(bq, o), ID_S,
                          k > 0 ? 1u : 0u);
           }
           tc::umma_commit(&bars->s_full);
-          tc::mbar_arrive(&bars->s_issued);  // dK(j - 1) may now queue behind S^T(j)
-          // dP^T(j) = V dO(j)^T once dK(j - 1) has read dS^T(j - 1).
-          ok = j == 0 || tc::mbar_wait(&bars->dk_done, (j - 1) & 1, abort, p.status);
+          if (++st == QST) {
+            st = 0;
+            ph ^= 1;
+          }
+          // dP^T(j) = V dO(j)^T once S^T(j) has been read out, dO has landed and dK(j - 1) has read
+          // dS^T(j - 1): whoever has seen dP^T(j) may write dS^T(j).
+          ok = tc::mbar_wait(&bars->do_full, j & 1, abort, p.status) &&
+               tc::mbar_wait(&bars->s_read, j & 1, abort, p.status) &&
+               (j == 0 || tc::mbar_wait(&bars->dk_done, (j - 1) & 1, abort, p.status));
           if (!ok) break;
           tc::fence_after_sync();
-          const uint64_t bd = tc::sdesc_kmajor_sw128(
-              tc::smem_u32(smem + L::ST_OFF + st * L::ST_STRIDE + L::ST_DO));
 #pragma unroll
           for (int k = 0; k < DH / 16; ++k) {
             const uint32_t o = (k >> 2) * L::CHUNK + (k & 3) * 32;
-            tc::umma_f16(tmem + L::DP_COL, tc::sdesc_advance(va, o), tc::sdesc_advance(bd, o), ID_S,
+            tc::umma_f16(tmem + L::X_COL, tc::sdesc_advance(va, o), tc::sdesc_advance(bd, o), ID_S,
                          k > 0 ? 1u : 0u);
           }
           tc::umma_commit(&bars->dp_full);
+          tc::umma_commit(&bars->do_empty);
         }
       } else {
+        const uint64_t bd = tc::sdesc_mnmajor_sw128(tc::smem_u32(smem + L::DO_OFF), L::CHUNK, 1024);
+        const uint64_t bq0 = tc::sdesc_mnmajor_sw128(tc::smem_u32(smem + L::Q_OFF), L::CHUNK, 1024);
+        int st = 0;
         for (int j = 0; ok && j < n_it; ++j) {
-          const int st = j % STAGES;
           // dV += P^T(j) dO(j) once the elementwise warps have written P^T(j).
-          ok = tc::mbar_wait(&bars->p_full, j & 1, abort, p.status);
+          ok = tc::mbar_wait(&bars->do_full, j & 1, abort, p.status) &&
+               tc::mbar_wait(&bars->p_full, j & 1, abort, p.status);
           if (!ok) break;
           tc::fence_after_sync();
-          const uint64_t bd = tc::sdesc_mnmajor_sw128(
-              tc::smem_u32(smem + L::ST_OFF + st * L::ST_STRIDE + L::ST_DO), L::CHUNK, 1024);
 #pragma unroll
           for (int k = 0; k < BQ / 16; ++k)
-            tc::umma_f16_ts(tmem + L::DV_COL, tmem + L::S_COL + pk_col(k), tc::sdesc_advance(bd, k * 16 * 128),
+            tc::umma_f16_ts(tmem + L::DV_COL, tmem + L::P_COL + pk_col(k), tc::sdesc_advance(bd, k * 16 * 128),
                             ID_G, (j > 0 || k > 0) ? 1u : 0u);
           tc::umma_commit(&bars->dv_done);
+          tc::umma_commit(&bars->do_empty);
           // dK += dS^T(j) Q(j) once dS^T(j) is written.
-          // dK(j) goes into the pipe behind S^T(j + 1), which the elementwise warps wait for
-          ok = tc::mbar_wait(&bars->ds_full, j & 1, abort, p.status) &&
-               (j + 1 == n_it || tc::mbar_wait(&bars->s_issued, (j + 1) & 1, abort, p.status));
+          ok = tc::mbar_wait(&bars->ds_full, j & 1, abort, p.status);
           if (!ok) break;
           tc::fence_after_sync();
-          const uint64_t bq = tc::sdesc_mnmajor_sw128(
-              tc::smem_u32(smem + L::ST_OFF + st * L::ST_STRIDE + L::ST_Q), L::CHUNK, 1024);
+          const uint64_t bq = tc::sdesc_advance(bq0, st * L::NCH * L::CHUNK);
 #pragma unroll
           for (int k = 0; k < BQ / 16; ++k)
-            tc::umma_f16_ts(tmem + L::DK_COL, tmem + L::DP_COL + pk_col(k), tc::sdesc_advance(bq, k * 16 * 128),
+            tc::umma_f16_ts(tmem + L::DK_COL, tmem + L::DS_COL + pk_col(k), tc::sdesc_advance(bq, k * 16 * 128),
                             ID_G, (j > 0 || k > 0) ? 1u : 0u);
           tc::umma_commit(&bars->dk_done);
-          // dV(j) and dK(j) are the stage's last readers (S^T(j) and dP^T(j) completed before the
-          // elementwise warps released P^T(j) and dS^T(j))
-          tc::umma_commit(&bars->ld_empty[st]);
+          // dK(j) is the last reader of Q(j) (S^T(j) completed before the elementwise warps read it), and
+          // they have read the block's rows before they released dS^T(j)
+          tc::umma_commit(&bars->q_empty[st]);
+          tc::umma_commit(&bars->row_empty[j & 1]);
           if (j == n_it - 1) tc::umma_commit(&bars->o_full);
+          if (++st == QST) st = 0;
         }
       }
       uint64_t* dr = warp == 1 ? &bars->drain : &bars->drain_g;
@@ -447,13 +496,11 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
     const uint32_t lane16 = (uint32_t)(quarter * 32 + half * 16) << 16;
     bool ok = true;
     for (int it = 0; it < n_it; ++it) {
-      const int st = it % STAGES;
       const int i = kb + it % per_head;
       const float* lse_s =
-          reinterpret_cast<const float*>(smem + L::ST_OFF + st * L::ST_STRIDE + L::ST_LSE) + 64 * chalf;
-      const float* d_s =
-          reinterpret_cast<const float*>(smem + L::ST_OFF + st * L::ST_STRIDE + L::ST_D) + 64 * chalf;
-      if (!tc::mbar_wait(&bars->ld_full[st], (it / STAGES) & 1, abort, p.status) ||
+          reinterpret_cast<const float*>(smem + L::ROW_OFF + (it & 1) * L::ROW_BYTES) + 64 * chalf;
+      const float* d_s = lse_s + BQ;
+      if (!tc::mbar_wait(&bars->row_full[it & 1], (it >> 1) & 1, abort, p.status) ||
           !tc::mbar_wait(&bars->s_full, it & 1, abort, p.status)) {
         ok = false;
         break;
@@ -464,8 +511,11 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
       {
         uint32_t r0[32];
         __syncwarp();
-        tc::tmem_ld_16x256b_x8(tmem + lane16 + L::S_COL + 64 * chalf, r0);
+        tc::tmem_ld_16x256b_x8(tmem + lane16 + L::X_COL + 64 * chalf, r0);
         tc::tmem_ld_wait();
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&bars->s_read);  // dP^T(j) may overwrite X
 #pragma unroll
         for (int c = 0; c < 32; ++c) x[c] = __uint_as_float(r0[c]);
       }
@@ -501,7 +551,7 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
           pw[2 * n + 1] = tc::pack_half2(x[4 * n + 2], x[4 * n + 3]);
         }
         __syncwarp();
-        tc::tmem_st_16x128b_x8(tmem + lane16 + L::S_COL + 64 * chalf, pw);
+        tc::tmem_st_16x128b_x8(tmem + lane16 + L::P_COL + 32 * chalf, pw);
         tc::tmem_st_wait();
       }
       tc::fence_before_sync();
@@ -526,8 +576,11 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
       {
         uint32_t rd[32];
         __syncwarp();
-        tc::tmem_ld_16x256b_x8(tmem + lane16 + L::DP_COL + 64 * chalf, rd);
+        tc::tmem_ld_16x256b_x8(tmem + lane16 + L::X_COL + 64 * chalf, rd);
         tc::tmem_ld_wait();
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&bars->dp_read);  // S^T(j + 1) may overwrite X
 #pragma unroll
         for (int n = 0; n < 8; ++n) {
           const float2 d2 = *reinterpret_cast<const float2*>(d_s + 8 * n + 2 * cq);
@@ -565,15 +618,18 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
         }
       }
       __syncwarp();
-      tc::tmem_st_16x128b_x8(tmem + lane16 + L::DP_COL + 64 * chalf, dw);
-      tc::tmem_st_wait();
-      tc::fence_before_sync();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&bars->ds_full);
-      // The same dS^T words into the staging tile for the store warp, once it has stored the
-      // previous block's: packed word n (queries 64 chalf + 8n + 2cq, +1) is 16-byte unit n of the
-      // 64-query half chalf of its key row (128-byte swizzle). With KL they go over this thread's
-      // own P^T words, loaded only after the previous block's store had read the tile.
+      tc::tmem_st_16x128b_x8(tmem + lane16 + L::DS_COL + 32 * chalf, dw);
+      auto release_ds = [&] {  // dK(j) may read dS^T
+        tc::tmem_st_wait();
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&bars->ds_full);
+      };
+      if (!KL) release_ds();
+      // The same dS^T words into the staging tile for the store warp, once it has stored the previous
+      // block's: packed word n (queries 64 chalf + 8n + 2cq, +1) is 16-byte unit n of the 64-query half
+      // chalf of its key row (128-byte swizzle). With KL they go over this thread's own P^T words, loaded
+      // only after the previous block's store had read the tile, while dS^T is on its way to TMEM.
       if (!KL && it > 0 && !tc::mbar_wait(&bars->dss_free, (it - 1) & 1, abort, p.status)) {
         ok = false;
         break;
@@ -584,24 +640,25 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
         wb_p[(n ^ swb) << 2] = dw[2 * n + 1];
       }
       tc::fence_proxy_async_smem();
+      if (KL) release_ds();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&bars->dss_full);
     }
     // Epilogue: dV rows (warps of query half 0) and dK rows (half 1; transpose of RoPE) staged
-    // transposed in the now idle stage buffers, then stored as dQKV^T columns with coalesced
+    // transposed in the now idle Q ring, then stored as dQKV^T columns with coalesced
     // 16-byte stores by all elementwise warps.
     const bool have = ok && tc::mbar_wait(&bars->o_full, 0, abort, p.status);
-    bf16_t* tv = reinterpret_cast<bf16_t*>(smem + L::ST_OFF);
-    bf16_t* tk = tv + DH * 128;
+    bf16_t* tv = reinterpret_cast<bf16_t*>(smem + L::Q_OFF);
+    bf16_t* tk = tv + DH * GRAD_PITCH;
     if (have) {
       tc::fence_after_sync();
       const int kA = keyA < p.T ? keyA : 0, kB = keyB < p.T ? keyB : 0;
       if (chalf == 0)
         stage_grad_16<DH>(tmem + lane16 + L::DV_COL, KL ? p.a_mse : 1.f, false, 0, 0, p.cos_t,
-                          p.sin_t, tv, rA);
+                          p.sin_t, tv, rA - (lane >> 2));
       else
         stage_grad_16<DH>(tmem + lane16 + L::DK_COL, p.scale, p.use_rope != 0, kA, kB, p.cos_t,
-                          p.sin_t, tk, rA);
+                          p.sin_t, tk, rA - (lane >> 2));
     }
     tc::named_bar_sync(1, DKDV_EW * 32);  // every elementwise warp reaches this exactly once
     if (have) {
@@ -948,7 +1005,7 @@ struct DqLayout {
   static constexpr int K_TILE = 128 * DH * 2;    // 128 keys x d_h
   static constexpr int STAGE = DS_TILE + K_TILE;
   static constexpr int STG_OFF = STAGES * STAGE;  // epilogue staging: d_h x 128 bf16
-  static constexpr int BAR_OFF = STG_OFF + DH * 128 * 2;
+  static constexpr int BAR_OFF = STG_OFF + DH * GRAD_PITCH * 2;
   static constexpr int USED = BAR_OFF + 256;      // base alignment checked in the kernel
   static constexpr int SMEM = USED > 118 * 1024 ? USED : 118 * 1024;
   static constexpr uint32_t DQ_STRIDE = 128;      // TMEM columns between the two dQ buffers
@@ -1098,7 +1155,7 @@ __global__ void __launch_bounds__(DQ_THREADS, 1)
         tc::fence_after_sync();
         const int ta = q0 + ra, tb = ta + 8;
         stage_grad_16<DH>(tmem + lane16 + ob * L::DQ_STRIDE, p.scale, p.use_rope != 0,
-                          ta < p.T ? ta : 0, tb < p.T ? tb : 0, p.cos_t, p.sin_t, stage, ra);
+                          ta < p.T ? ta : 0, tb < p.T ? tb : 0, p.cos_t, p.sin_t, stage, ra - (lane >> 2));
         tc::fence_before_sync();
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&bars->o_empty[ob]);  // the dQ buffer is free again
