@@ -156,6 +156,14 @@ bool is_prepared(const void* ws, const void* x, int32_t B, int32_t T, int32_t d)
   return false;
 }
 
+// The reductions' block counter and partial slots in the workspace.
+int* reduce_counter(void* ws, const Workspace& wp) {
+  return reinterpret_cast<int*>(static_cast<char*>(ws) + wp.status);
+}
+double* reduce_slots(void* ws, const Workspace& wp) {
+  return reinterpret_cast<double*>(static_cast<char*>(ws) + wp.red);
+}
+
 // X in fp16 (unless the workspace holds it: x_prepared), the fp16 operand of every candidate (n_cand
 // = 0: W itself; W_dev null: none) and the RoPE table, in one launch. Records X for *_prepared.
 jab_status prepare_inputs(const jab_block_desc* desc, int32_t B, int32_t T, const void* X_dev,
@@ -169,6 +177,7 @@ jab_status prepare_inputs(const jab_block_desc* desc, int32_t B, int32_t T, cons
     in.xh = w + wp.x16;
     in.nx = (int64_t)B * T * desc->d_model;
   }
+  in.counter = reduce_counter(w, wp);
   in.D = (int)block_rows(desc);
   in.d = desc->d_model;
   in.G = desc->group_size;
@@ -238,7 +247,8 @@ jab_status jab_reference_forward(const jab_block_desc* desc, int32_t B, int32_t 
   JAB_SITE("attn_fwd", 1, launch_attn_fwd_tc(L, 0));
   if (a_sqnorm_dev)
     JAB_SITE("loss_reduce", 1, launch_loss_reduce(L.part, 1, B, desc->n_q_heads, L.nP, 1.0,
-                                                  a_sqnorm_dev, nullptr, status, st));
+                                                  a_sqnorm_dev, nullptr, reduce_slots(ws, wp),
+                                                  reduce_counter(ws, wp), status, st));
   return JAB_OK;
 }
 
@@ -288,7 +298,8 @@ static jab_status forward_candidates(const jab_block_desc* desc, int32_t B, int3
   JAB_SITE("attn_fwd", 1, launch_attn_fwd_tc(L, 1));
   const double inv_n = 1.0 / ((double)N * desc->n_q_heads * dh);
   JAB_SITE("loss_reduce", 1, launch_loss_reduce(L.part, n_cand, B, desc->n_q_heads, L.nP, inv_n,
-                                                mse_dev, sse_parts_dev, status, st));
+                                                mse_dev, sse_parts_dev, reduce_slots(ws, wp),
+                                                reduce_counter(ws, wp), status, st));
   *wp_out = wp;
   *status_out = status;
   return JAB_OK;
@@ -368,7 +379,8 @@ jab_status jab_loss_forward_kl(const jab_block_desc* desc, int32_t B, int32_t T,
                                            part, nP, kl_rows_dev, status, st));
   // batchmean (App. B "Effective weight of the KL term"): the sum over rows divided by B
   JAB_SITE("loss_reduce", 1, launch_loss_reduce(part, n_cand, B, desc->n_q_heads, nP, 1.0 / B, kl,
-                                                nullptr, status, st));
+                                                nullptr, reduce_slots(ws, wp), reduce_counter(ws, wp),
+                                                status, st));
   JAB_SITE("loss_combine", 1, launch_loss_combine(mse_dev, kl, (double)lambda_kl, n_cand, loss_dev,
                                                   st));
   return JAB_OK;
@@ -430,7 +442,9 @@ jab_status jab_hutchinson_trace(const jab_block_desc* desc, int32_t B, int32_t T
     double* vhv = vhv_dev ? vhv_dev + pr : tmp;
     // v^T H v = 2 ||J_A v||^2 / n (Eq. 5 at the float weights, MSE term)
     JAB_SITE("loss_reduce", 1, launch_loss_reduce(part, 1, B, desc->n_q_heads, nP,
-                                                  2.0 * rescale / n_el, vhv, nullptr, status, st));
+                                                  2.0 * rescale / n_el, vhv, nullptr,
+                                                  reduce_slots(ws, wp), reduce_counter(ws, wp), status,
+                                                  st));
     JAB_SITE("loss_combine", 1, launch_loss_combine(trace_dev, vhv, 1.0 / n_probes, 1, trace_dev,
                                                     st));
   }
@@ -492,14 +506,15 @@ struct KlTerm {
 };
 
 // Steps shared by the backward entry points (App. B, STE): quantise, project (+ RoPE), attention
-// forward in mode 2 (loss partials, dO = A_hat - A_ref, lse, D), the loss, and the attention backward
-// into dQKV^T (bf16 [D, ldt]) in the workspace; with a KL term also the teacher's probability tiles
-// and the KL value. Checks the arguments common to all.
+// forward in mode 2 (loss partials, dO = A_hat - A_ref, lse, D) and the attention backward into dQKV^T
+// (bf16 [D, ldt]) in the workspace; with a KL term also the teacher's probability tiles and the KL
+// partials. The loss is left to the caller's last launch (*nP_out partials per sequence and head). Checks
+// the arguments common to all.
 static jab_status backward_to_dqkvt(const jab_block_desc* desc, int32_t B, int32_t T,
                                     const void* X_dev, const void* W_dev, const float* A_ref_dev,
                                     int32_t bits, const float* scales_dev, double* loss_dev,
                                     void* ws, size_t ws_bytes, bool x_prepared, cudaStream_t st,
-                                    Workspace* wp_out, int** status_out,
+                                    Workspace* wp_out, int** status_out, int* nP_out,
                                     const KlTerm* kl = nullptr) {
   jab_status s = check_desc(desc);
   if (s != JAB_OK) return s;
@@ -536,28 +551,21 @@ static jab_status backward_to_dqkvt(const jab_block_desc* desc, int32_t B, int32
   L.lse_pitch = (int)wp.tp;
   L.ds = w + wp.ds;
   JAB_SITE("attn_fwd", 1, launch_attn_fwd_tc(L, 2));
-  const double n_el = (double)N * desc->n_q_heads * dh;
-  JAB_SITE("loss_reduce", 1, launch_loss_reduce(L.part, 1, B, desc->n_q_heads, L.nP, 1.0 / n_el,
-                                                loss_dev, nullptr, status, st));
   const float* kl_ab = nullptr;
   if (kl != nullptr) {
     const int Hq = desc->n_q_heads, Hkv = desc->n_kv_heads;
     float* lse_t = reinterpret_cast<float*>(w + wp.lse_t);
     double* klpart = reinterpret_cast<double*>(w + wp.klpart);
-    double* klv = kl->kl_out ? kl->kl_out : reinterpret_cast<double*>(w + wp.scal) + 1;
     JAB_SITE("lse_log2", 1, launch_lse_to_log2(kl->lse_ref, B * Hq, T, (int)wp.tp, lse_t, st));
     JAB_SITE("teacher_p", 1, launch_attn_teacher_p_tc(w + wp.qkv, D, kl->qkv_ref, D, B, T, Hq, Hkv,
                                                       dh, L.scale, lse_t, L.lse, (int)wp.tp, L.ds,
                                                       klpart, status, st));
-    // batchmean (reading R18): the sum over sequences, heads, rows and keys divided by B
-    JAB_SITE("kl_reduce", 1, launch_sum_scaled(klpart, Hkv * B * ((T + 127) / 128), 1.0 / B, klv,
-                                               st));
-    JAB_SITE("loss_combine", 1, launch_loss_combine(loss_dev, klv, kl->lambda, 1, loss_dev, st));
     kl_ab = kl->ab;
   }
   JAB_SITE("attn_bwd", 2, launch_attn_bwd_tc(L, cos_t, sin_t, desc->use_rope, w + wp.dqkvt, kl_ab));
   *wp_out = wp;
   *status_out = status;
+  *nP_out = L.nP;
   return JAB_OK;
 }
 
@@ -578,8 +586,9 @@ static jab_status backward_scales(const jab_block_desc* desc, int32_t B, int32_t
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   Workspace wp;
   int* status;
+  int nP = 0, splits = 1;
   jab_status s = backward_to_dqkvt(desc, B, T, X_dev, W_dev, A_ref_dev, bits, scales_dev, loss_dev,
-                                   ws, ws_bytes, x_prepared, st, &wp, &status, kl);
+                                   ws, ws_bytes, x_prepared, st, &wp, &status, &nP, kl);
   if (s != JAB_OK) return s;
   char* w = static_cast<char*>(ws);
   const int64_t N = (int64_t)B * T;
@@ -589,10 +598,31 @@ static jab_status backward_scales(const jab_block_desc* desc, int32_t B, int32_t
   // with the KL term the attention backward's dQKV^T is a times the MSE term's units
   const float coef = (float)(k * 2.0 / n_el / (kl ? (double)kl->ab[0] : 1.0));
   // per-split partials summed in order: the scale gradient is bit-identical between calls
+  float* gpart = reinterpret_cast<float*>(w + wp.gpart);
   JAB_SITE("wgrad_lsq", 1, launch_wgrad_lsq_tc(w + wp.dqkvt, wp.ldt, X_dev, W_dev, scales_dev, N, D,
-                                               dm, G, bits, coef, grad_scales_dev,
-                                               reinterpret_cast<float*>(w + wp.gpart), status, st));
-  JAB_SITE("check_finite", 1, launch_check_finite(grad_scales_dev, (int64_t)D * (dm / G), status, st));
+                                               dm, G, bits, coef, gpart, &splits, status, st));
+  FinishArgs f{};
+  f.gpart = gpart;
+  f.splits = splits;
+  f.n = (int64_t)D * (dm / G);
+  f.grad = grad_scales_dev;
+  f.part = reinterpret_cast<double*>(w + wp.part);
+  f.nbh = B * desc->n_q_heads;
+  f.nP = nP;
+  f.inv_n = 1.0 / n_el;
+  f.loss = loss_dev;
+  if (kl != nullptr) {
+    f.klpart = reinterpret_cast<double*>(w + wp.klpart);
+    f.nkl = desc->n_kv_heads * B * ((T + 127) / 128);
+    // batchmean (reading R18): the sum over sequences, heads, rows and keys divided by B
+    f.kl_scale = 1.0 / B;
+    f.lambda = kl->lambda;
+    f.kl_out = kl->kl_out;
+  }
+  f.red = reduce_slots(ws, wp);
+  f.counter = reduce_counter(ws, wp);
+  f.status = status;
+  JAB_SITE("finish", 1, launch_finish(f, st));
   return JAB_OK;
 }
 
@@ -681,20 +711,22 @@ jab_status jab_loss_backward_weights(const jab_block_desc* desc, int32_t B, int3
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   Workspace wp;
   int* status;
+  int nP = 0;
   s = backward_to_dqkvt(desc, B, T, X_dev, W_dev, A_ref_dev, bits, scales_dev, loss_dev, ws,
-                        ws_bytes, false, st, &wp, &status);
+                        ws_bytes, false, st, &wp, &status, &nP);
   if (s != JAB_OK) return s;
   char* w = static_cast<char*>(ws);
   const int64_t N = (int64_t)B * T;
   const int D = (int)block_rows(desc), dm = desc->d_model;
   const double n_el = (double)N * desc->n_q_heads * desc->head_dim;
-  JAB_SITE("wgrad_store", 1, launch_wgrad_store_tc(w + wp.dqkvt, wp.ldt, X_dev, N, D, dm,
+  JAB_SITE("loss_reduce", 1, launch_loss_reduce(reinterpret_cast<double*>(w + wp.part), 1, B,
+                                                desc->n_q_heads, nP, 1.0 / n_el, loss_dev, nullptr,
+                                                reduce_slots(ws, wp), reduce_counter(ws, wp), status, st));
+  JAB_SITE("wgrad_store", grad_sqnorm_dev ? 3 : 2, launch_wgrad_store_tc(w + wp.dqkvt, wp.ldt, X_dev, N, D, dm,
                                                    (float)(2.0 / n_el), grad_w_dev, grad_sqnorm_dev,
                                                    reinterpret_cast<float*>(w + wp.dwscr),
                                                    reinterpret_cast<double*>(w + wp.red),
                                                    g_deterministic != 0, status, st));
-  if (grad_w_dev)
-    JAB_SITE("check_finite", 1, launch_check_finite(grad_w_dev, (int64_t)D * dm, status, st));
   return JAB_OK;
 }
 

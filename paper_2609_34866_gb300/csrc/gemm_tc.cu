@@ -51,7 +51,6 @@ struct GemmParams {
   const float* s;
   int d, G, bits;
   float coef;
-  float* ds;
   float* dspart;  // fp32 [splits, M, d/G]: each unit's partial, summed over the splits in order
   // weight-gradient store epilogue (a split K adds partial tiles into a zeroed dw)
   float* dw;
@@ -643,7 +642,7 @@ int choose_splits(int tiles, int k_blocks, int sms) {
 
 cudaError_t launch_wgrad_lsq_tc(const void* dqkvt, int64_t ldt, const void* x, const void* w,
                                 const float* s, int64_t N, int D, int d, int G, int bits,
-                                float coef, float* ds, float* dspart, int* status, cudaStream_t st) {
+                                float coef, float* dspart, int* splits, int* status, cudaStream_t st) {
   CUtensorMap ta, tb;
   if (!make_tmap(&ta, dqkvt, true, N, D, ldt, BM) || !make_tmap(&tb, x, true, d, N, d, BK))
     return cudaErrorInvalidValue;
@@ -663,13 +662,11 @@ cudaError_t launch_wgrad_lsq_tc(const void* dqkvt, int64_t ldt, const void* x, c
   p.G = G;
   p.bits = bits;
   p.coef = coef;
-  p.ds = ds;
   p.dspart = dspart;
-  // every (split, row, group) partial is written once; the splits are summed in order: the scale
-  // gradient is bit-identical between calls
-  cudaError_t e = launch_gemm2<kEpiLsq, true, true>(ta, tb, ta, p, st);
-  if (e != cudaSuccess) return e;
-  return launch_split_sum(dspart, p.splits, (int64_t)D * (d / G), ds, st);
+  // every (split, row, group) partial is written once; the splits are summed in order by the caller's
+  // last launch: the scale gradient is bit-identical between calls
+  *splits = p.splits;
+  return launch_gemm2<kEpiLsq, true, true>(ta, tb, ta, p, st);
 }
 
 cudaError_t launch_wgrad_store_tc(const void* dqkvt, int64_t ldt, const void* x, int64_t N, int D,
@@ -701,8 +698,10 @@ cudaError_t launch_wgrad_store_tc(const void* dqkvt, int64_t ldt, const void* x,
     if (e != cudaSuccess) return e;
   }
   e = launch_gemm2<kEpiStore, true, true>(ta, tb, ta, p, st);
-  if (e != cudaSuccess || sqnorm == nullptr) return e;
-  return launch_sumsq(target, n_w, red, sqnorm, st);  // fixed order
+  if (e != cudaSuccess) return e;
+  // a dW that the caller gets is checked, in the pass over it for its norm where there is one
+  if (sqnorm != nullptr) return launch_sumsq(target, n_w, red, sqnorm, dw != nullptr ? status : nullptr, st);
+  return launch_check_finite(target, n_w, status, st);
 }
 
 }  // namespace jab

@@ -42,6 +42,7 @@ struct PrepInputs {
   float *cos_t, *sin_t;
   int T, dh;
   float theta;
+  int* counter;  // set to 0 (null: none)
 };
 cudaError_t launch_prep(const PrepInputs& in, int* status, int sms, cudaStream_t st);
 cudaError_t launch_quantize(const void* w, const float* s, int D, int d, int G, int bits,
@@ -57,10 +58,10 @@ cudaError_t launch_proj_gemm_tc(const void* A, const void* Bw, void* C, int64_t 
                                 int D, int n_rot, int dh, int T, const float* cos_t,
                                 const float* sin_t, int* status, cudaStream_t st);
 // x: bf16 [N, d] as the caller stores it (no transposed copy)
-// ds: the scale gradient, written (fp32 [D, d/G]); dspart: fp32 [kMaxSplits, D, d/G] scratch
+// dspart: fp32 [kMaxSplits, D, d/G], the scale gradient's partial of each of the *splits K ranges
 cudaError_t launch_wgrad_lsq_tc(const void* dqkvt, int64_t ldt, const void* x, const void* w,
                                 const float* s, int64_t N, int D, int d, int G, int bits,
-                                float coef, float* ds, float* dspart, int* status, cudaStream_t st);
+                                float coef, float* dspart, int* splits, int* status, cudaStream_t st);
 // coef * dQKV^T X stored fp32 [D, d] in dw, or in scratch (fp32 [D, d]) when dw is NULL, and its
 // squared norm in *sqnorm (may be NULL) by a fixed-order reduction (red: fp64 [kRedBlocks]). A split
 // K adds partial tiles with atomics; deterministic keeps one unit per tile (bit-identical dW).
@@ -117,19 +118,42 @@ cudaError_t launch_qerr_partial(const void* w, const float* s, int D, int d, int
                                 double* part, int nblocks, int* status, cudaStream_t st);
 
 // reduce.cu
-// A non-finite total raises JAB_ERR_NONFINITE in *status.
+// red: fp64 [C, kRedBlocks] scratch; counter: an int that is 0 (and is left at 0). A non-finite total raises
+// JAB_ERR_NONFINITE in *status.
 cudaError_t launch_loss_reduce(const double* part, int C, int B, int Hq, int nP, double inv_n,
-                               double* out, double* parts_out, int* status, cudaStream_t st);
+                               double* out, double* parts_out, double* red, int* counter, int* status,
+                               cudaStream_t st);
+// The end of a scale-gradient call: grad[i] = sum over s < splits of gpart[s n + i], in order of s (fp64 sum,
+// fp32 result); *loss = inv_n * sum of part [nbh, nP]; with klpart [nkl] (else null) *kl_out (may be null)
+// = kl_scale * its sum and *loss += lambda * that. red, counter, status as above.
+struct FinishArgs {
+  const float* gpart;
+  int splits;
+  int64_t n;
+  float* grad;
+  const double* part;
+  int nbh, nP;
+  double inv_n;
+  double* loss;
+  const double* klpart;
+  int nkl;
+  double kl_scale, lambda;
+  double* kl_out;
+  double* red;
+  int* counter;
+  int* status;
+  int nblk;  // set by the launcher
+};
+cudaError_t launch_finish(FinishArgs a, cudaStream_t st);
 // out[c] = a[c] + lam * b[c] for c < C
 cudaError_t launch_loss_combine(const double* a, const double* b, double lam, int C, double* out,
                                 cudaStream_t st);
 cudaError_t launch_omega_finish(const double* part, int nblocks, int C, const double* trace,
                                 double layers_after, double* c1, double* c2, cudaStream_t st);
-cudaError_t launch_mean(const double* x, int n, double* out, cudaStream_t st);
 cudaError_t launch_check_finite(const float* x, int64_t n, int* status, cudaStream_t st);
-// *out = sum of x[i]^2 in fp64, fixed order (part: fp64 [kRedBlocks])
-cudaError_t launch_sumsq(const float* x, int64_t n, double* part, double* out, cudaStream_t st);
-// out[i] = sum over s < splits of part[s n + i], in order of s (fp64 sum, fp32 result)
-cudaError_t launch_split_sum(const float* part, int splits, int64_t n, float* out, cudaStream_t st);
+// *out = sum of x[i]^2 to fp64 accuracy, fixed order (part: fp64 [kRedBlocks]; n a multiple of 8, x 16-byte
+// aligned); with a status word, non-finite values raise JAB_ERR_NONFINITE.
+cudaError_t launch_sumsq(const float* x, int64_t n, double* part, double* out, int* status,
+                         cudaStream_t st);
 
 }  // namespace jab

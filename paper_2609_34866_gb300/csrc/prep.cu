@@ -27,6 +27,7 @@ struct PrepArgs {
   int T, half;
   double freq_pi[64];  // theta^(-j / half) / pi
   int* status;
+  int* counter;  // zeroed for the call's reductions
 };
 
 // ---------------------------------------------------------------- X: bf16 -> fp16 (+ range check)
@@ -249,6 +250,7 @@ __device__ __forceinline__ void rope_role(const PrepArgs& p, int blk) {
 // candidates, 2048 rows and 65536 x 4096 of X 462 us, now 248 us (1.37 GB: 202 us at the copy rate).
 __global__ void __launch_bounds__(256, 4) prep_kernel(const __grid_constant__ PrepArgs p) {
   const int blk = blockIdx.x;
+  if (blk == 0 && threadIdx.x == 0 && p.counter != nullptr) *p.counter = 0;
   if (blk < p.nrope)
     rope_role(p, blk);
   else if (blk < p.nrope + p.nw)
@@ -573,6 +575,7 @@ cudaError_t launch_prep(const PrepInputs& in, int* status, int sms, cudaStream_t
   for (int c0 = 0; c0 == 0 || c0 < in.ncand; c0 += PrepArgs::kMaxCand) {
     PrepArgs p{};
     p.status = status;
+    p.counter = in.counter;
     p.D = in.D;
     p.d = in.d;
     p.G = in.G;

@@ -1,31 +1,71 @@
 // Loss reduction (Eq. 3, MSE term): per-tile fp64 partials -> SSE per (candidate, sequence, head)
 // and L = SSE / (B T Hq d_h). Fixed summation order, so repeated calls give identical bits.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "workspace.h"
 
 namespace jab {
 
-__global__ void __launch_bounds__(256) loss_reduce_kernel(const double* __restrict__ part, int B,
-                                                          int Hq, int nP, double inv_n,
-                                                          double* __restrict__ out,
-                                                          double* __restrict__ parts_out,
-                                                          int* status) {
-  __shared__ double red[8];
-  const int c = blockIdx.x;
-  const int nbh = B * Hq;
+// One warp, `blk` of `nblk`: sum of its share of the rows ((sequence, head) pairs, nP partials each; a lane
+// per row, the partials in order). A warp and no more per SM: fp64 additions go at about two a clock there,
+// 16 clocks an instruction of a warp.
+__device__ __forceinline__ double loss_slice(const double* __restrict__ part, int nbh, int nP, int blk,
+                                             int nblk, double* __restrict__ parts_out) {
   double acc = 0.0;
-  for (int i = threadIdx.x; i < nbh; i += blockDim.x) {
-    const double* p = part + ((int64_t)c * nbh + i) * nP;
+  for (int i = blk * 32 + (threadIdx.x & 31); i < nbh; i += nblk * 32) {
+    const double* p = part + (int64_t)i * nP;
     double s = 0.0;
+#pragma unroll 8
     for (int k = 0; k < nP; ++k) s += p[k];
-    if (parts_out) parts_out[(int64_t)c * nbh + i] = s;
+    if (parts_out) parts_out[i] = s;
     acc += s;
   }
-  const double tot = block_sum<256>(acc, red);
-  if (threadIdx.x == 0) {
-    out[c] = tot * inv_n;
-    if (!isfinite(tot)) report(status, JAB_ERR_NONFINITE);
+  return warp_sum(acc);
+}
+
+// Counts a warp's published partial (of `total`); true, in all its lanes, in the one that comes last, with
+// every partial visible. The counter (0 before the launch) is left at 0.
+__device__ __forceinline__ bool last_warp(int* counter, int total) {
+  int last = 0;
+  if ((threadIdx.x & 31) == 0) {
+    __threadfence();
+    last = atomicAdd(counter, 1) == total - 1;
+    if (last) {
+      *counter = 0;
+      __threadfence();
+    }
+  }
+  return __shfl_sync(0xffffffffu, last, 0) != 0;
+}
+
+// Sum of n published partials by one warp, lane-strided and then a fixed tree.
+__device__ __forceinline__ double sum_published(const double* part, int n) {
+  double acc = 0.0;
+  for (int k = threadIdx.x & 31; k < n; k += 32) acc += __ldcg(part + k);
+  return warp_sum(acc);
+}
+
+// nblk one-warp blocks per candidate, the last block of the grid adds their sums (one block per candidate
+// took 88 us for 4096 x 32 partials, 24 us for 5 x 1024 x 32; now 11 us).
+__global__ void __launch_bounds__(32) loss_reduce_kernel(const double* __restrict__ part, int C, int nbh,
+                                                         int nP, int nblk, double inv_n,
+                                                         double* __restrict__ out,
+                                                         double* __restrict__ parts_out,
+                                                         double* __restrict__ red, int* counter,
+                                                         int* status) {
+  const int c = blockIdx.x / nblk, blk = blockIdx.x - c * nblk;
+  const double t = loss_slice(part + (int64_t)c * nbh * nP, nbh, nP, blk, nblk,
+                              parts_out ? parts_out + (int64_t)c * nbh : nullptr);
+  if (threadIdx.x == 0) red[c * kRedBlocks + blk] = t;
+  if (!last_warp(counter, gridDim.x)) return;
+  for (int k = 0; k < C; ++k) {
+    const double tot = sum_published(red + k * kRedBlocks, nblk);
+    if (threadIdx.x == 0) {
+      out[k] = tot * inv_n;
+      if (!isfinite(tot)) report(status, JAB_ERR_NONFINITE);
+    }
   }
 }
 
@@ -55,15 +95,6 @@ __global__ void __launch_bounds__(256) omega_finish_kernel(const double* __restr
   }
 }
 
-// mean over n of a fp64 array (the Hutchinson estimate over its probes), fixed order
-__global__ void mean_kernel(const double* __restrict__ x, int n, double* __restrict__ out) {
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < n; ++i) t += x[i];
-    *out = t / n;
-  }
-}
-
 __global__ void check_finite_kernel(const float* __restrict__ x, int64_t n, int* status) {
   bool bad = false;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -72,27 +103,50 @@ __global__ void check_finite_kernel(const float* __restrict__ x, int64_t n, int*
   if (__syncthreads_or(bad) && threadIdx.x == 0) report(status, JAB_ERR_NONFINITE);
 }
 
-// Sum of squares in fp64: block b sums its contiguous chunk (fixed per-thread order, fixed tree),
-// then one thread adds the kRedBlocks partials in order.
-__global__ void __launch_bounds__(256) sumsq_partial_kernel(const float* __restrict__ x, int64_t n,
-                                                            double* __restrict__ part) {
-  __shared__ double red[8];
-  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-  const int64_t lo = blockIdx.x * chunk, hi = lo + chunk < n ? lo + chunk : n;
-  double acc = 0.0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-    const double v = x[i];
-    acc += v * v;
+// Sum of squares: block b sums its contiguous chunk (fixed per-thread order, fixed tree), one block then
+// adds the kRedBlocks partials. The chip runs about two FP64 operations per clock and SM, and a
+// conversion and a multiply-add per value bounded the kernel (101 us for 25M values, now 32): eight squares
+// are added as unevaluated pairs of floats, errors carried along (2^-46 of the sum), and only that goes to
+// the fp64 accumulator. Values whose largest is outside 2^-40 .. 2^60 are squared in fp64. With `status` a
+// non-finite value is reported.
+__device__ __forceinline__ double sumsq8(const float (&v)[8]) {
+  float big = 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) big = fmaxf(big, fabsf(v[k]));
+  if (!(big >= 9.0949470e-13f && big <= 1.1529215e18f)) {
+    double acc = 0.0;
+    for (int k = 0; k < 8; ++k) acc += (double)v[k] * (double)v[k];
+    return acc;
   }
-  const double t = block_sum<256>(acc, red);
-  if (threadIdx.x == 0) part[blockIdx.x] = t;
+  float sh = 0.f, sl = 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float h = __fmul_rn(v[k], v[k]), l = __fmaf_rn(v[k], v[k], -h);
+    const float t = __fadd_rn(sh, h), bb = __fsub_rn(t, sh);
+    const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bb)), __fsub_rn(h, bb));  // sh + h = t + e
+    sh = t;
+    sl = __fadd_rn(sl, __fadd_rn(e, l));
+  }
+  return (double)sh + (double)sl;
 }
 
-__global__ void sum_in_order_kernel(const double* __restrict__ part, int n, double* __restrict__ out) {
+__global__ void __launch_bounds__(256) sumsq_partial_kernel(const float* __restrict__ x, int64_t n,
+                                                            double* __restrict__ part, int* status) {
+  __shared__ double red[8];
+  const int64_t n8 = n / 8;  // n is a multiple of 64 (rows of a weight)
+  const int64_t chunk = (n8 + gridDim.x - 1) / gridDim.x;
+  const int64_t lo = blockIdx.x * chunk, hi = lo + chunk < n8 ? lo + chunk : n8;
+  const float4* x4 = reinterpret_cast<const float4*>(x);
+  double acc = 0.0;
+  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+    const float4 a = x4[2 * i], b = x4[2 * i + 1];
+    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    acc += sumsq8(v);
+  }
+  const double t = block_sum<256>(acc, red);
   if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < n; ++i) t += part[i];
-    *out = t;
+    part[blockIdx.x] = t;
+    if (status != nullptr && !isfinite(t)) report(status, JAB_ERR_NONFINITE);
   }
 }
 
@@ -120,20 +174,59 @@ __global__ void lse_to_log2_kernel(const float* __restrict__ in, int BH, int T, 
   }
 }
 
-// Sum of the K-split partials of a gradient in the order of the splits (one thread per element).
-__global__ void split_sum_kernel(const float* __restrict__ part, int splits, int64_t n,
-                                 float* __restrict__ out) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+// The end of a scale-gradient call in one launch: every gradient element as the sum of its K-split partials
+// in the order of the splits (a non-finite sum is reported), and in the first blocks' first warps the loss from its partials
+// and, with KL partials, the KL value and loss + lambda KL. (Three to five launches before; 4 x 128 fit 68.7 ->
+// 64 us a call.)
+__global__ void __launch_bounds__(256) finish_kernel(const __grid_constant__ FinishArgs p) {
+  bool bad = false;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n;
        i += (int64_t)gridDim.x * blockDim.x) {
     double t = 0.0;
-    for (int s = 0; s < splits; ++s) t += part[(int64_t)s * n + i];
-    out[i] = (float)t;
+    for (int s = 0; s < p.splits; ++s) t += p.gpart[(int64_t)s * p.n + i];
+    const float v = (float)t;
+    p.grad[i] = v;
+    bad |= !isfinite(v);
+  }
+  if (bad) report(p.status, JAB_ERR_NONFINITE);
+  if ((int)blockIdx.x >= p.nblk || threadIdx.x >= 32) return;
+  const double l = loss_slice(p.part, p.nbh, p.nP, blockIdx.x, p.nblk, nullptr);
+  double kl = 0.0;
+  if (p.klpart != nullptr) {
+    for (int i = blockIdx.x * 32 + threadIdx.x; i < p.nkl; i += p.nblk * 32) kl += p.klpart[i];
+    kl = warp_sum(kl);
+  }
+  if (threadIdx.x == 0) {
+    p.red[blockIdx.x] = l;
+    p.red[kRedBlocks / 2 + blockIdx.x] = kl;
+  }
+  if (!last_warp(p.counter, p.nblk)) return;
+  const double tot = sum_published(p.red, p.nblk);
+  const double ktot = p.klpart != nullptr ? sum_published(p.red + kRedBlocks / 2, p.nblk) : 0.0;
+  if (threadIdx.x == 0) {
+    if (!isfinite(tot)) report(p.status, JAB_ERR_NONFINITE);
+    const double klv = ktot * p.kl_scale;
+    *p.loss = p.klpart != nullptr ? tot * p.inv_n + p.lambda * klv : tot * p.inv_n;
+    if (p.kl_out) *p.kl_out = klv;
   }
 }
 
+// Blocks that a sum over nbh rows is worth (at most half of the kRedBlocks slots).
+static int loss_blocks(int nbh) { return std::min(kRedBlocks / 2, std::max(1, (nbh + 31) / 32)); }
+
 cudaError_t launch_loss_reduce(const double* part, int C, int B, int Hq, int nP, double inv_n,
-                               double* out, double* parts_out, int* status, cudaStream_t st) {
-  loss_reduce_kernel<<<C, 256, 0, st>>>(part, B, Hq, nP, inv_n, out, parts_out, status);
+                               double* out, double* parts_out, double* red, int* counter, int* status,
+                               cudaStream_t st) {
+  const int nbh = B * Hq, nblk = loss_blocks(nbh);
+  loss_reduce_kernel<<<C * nblk, 32, 0, st>>>(part, C, nbh, nP, nblk, inv_n, out, parts_out, red, counter,
+                                              status);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_finish(FinishArgs a, cudaStream_t st) {
+  a.nblk = loss_blocks(std::max(a.nbh, a.klpart != nullptr ? a.nkl : 0));
+  const int64_t blocks = std::min<int64_t>(4096, std::max<int64_t>((a.n + 255) / 256, a.nblk));
+  finish_kernel<<<(unsigned)blocks, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -149,25 +242,12 @@ cudaError_t launch_omega_finish(const double* part, int nblocks, int C, const do
   return cudaGetLastError();
 }
 
-cudaError_t launch_mean(const double* x, int n, double* out, cudaStream_t st) {
-  mean_kernel<<<1, 32, 0, st>>>(x, n, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_sumsq(const float* x, int64_t n, double* part, double* out, cudaStream_t st) {
-  sumsq_partial_kernel<<<kRedBlocks, 256, 0, st>>>(x, n, part);
+cudaError_t launch_sumsq(const float* x, int64_t n, double* part, double* out, int* status,
+                         cudaStream_t st) {
+  sumsq_partial_kernel<<<kRedBlocks, 256, 0, st>>>(x, n, part, status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  sum_in_order_kernel<<<1, 32, 0, st>>>(part, kRedBlocks, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_split_sum(const float* part, int splits, int64_t n, float* out, cudaStream_t st) {
-  int64_t blocks = (n + 255) / 256;
-  if (blocks > 4096) blocks = 4096;
-  if (blocks < 1) blocks = 1;
-  split_sum_kernel<<<(unsigned)blocks, 256, 0, st>>>(part, splits, n, out);
-  return cudaGetLastError();
+  return launch_sum_scaled(part, kRedBlocks, 1.0, out, st);
 }
 
 cudaError_t launch_sum_scaled(const double* part, int n, double scale, double* out, cudaStream_t st) {

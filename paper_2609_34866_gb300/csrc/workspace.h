@@ -19,7 +19,7 @@ struct Workspace {
   size_t qkv;      // fp16 [N, C*D]          projected, RoPE-rotated Q|K|V for every candidate
   size_t rope;     // fp32 [2, T, d_h/2]     cos then sin
   size_t part;     // fp64 [C, B, Hq, nP]    per-tile partial sums (SSE or ||A||^2)
-  size_t status;   // int32 [4]              reserved
+  size_t status;   // int32 [16]             [0]: blocks done of the reduction in flight, else 0
   size_t scal;     // fp64 [2, C]            per-candidate scalars (MSE and KL terms)
   size_t red;      // fp64 [C, kRedBlocks]   per-block partial sums of the quantisation error
   // backward only

@@ -142,3 +142,31 @@ def test_scale_gradient_where_the_quotient_takes_the_division():
     r = O.jab_loss_and_grad(c.x64, np64(w), s, 3, c.odesc, kappa=1.0)
     assert cosine(grad.cpu().numpy(), r["grad_s"]) >= COS_MIN
     assert J().jab_get_device_status() == 0
+
+
+@pytest.mark.parametrize("B,T", [(3, 65), (1, 257), (2, 1)])
+def test_weight_gradient_norm_and_loss_parts_of_odd_batches(B, T):
+    """||dW||^2 from float pairs against the fp64 sum of the returned dW (2^-46 per term, 256-thread fp64
+    sums), alone and beside dW, and the loss as the fixed-order sum of its (sequence, head) parts over
+    numbers of partials that are no power of two."""
+    from dataclasses import replace
+    from tests.harness import Case
+    from workloads import WORKLOADS
+    c = Case(replace(WORKLOADS["gpt2_smoke"], shape=BlockShape(256, 4, 1, 64, True, 500.0)), B, T, 64)
+    ws = c.workspace()
+    A, _, _ = c.gpu_teacher(ws)
+    s = c.gpu_scales(2)
+    loss, sq, sq2 = (torch.empty(1, dtype=torch.float64, device="cuda") for _ in range(3))
+    dw = torch.empty((c.D, 256), dtype=torch.float32, device="cuda")
+    J().jab_set_deterministic(True)
+    try:
+        J().jab_loss_backward_weights(c.desc, B, T, c.X, c.W, A, 2, s, loss, grad_w=dw, grad_sqnorm=sq, ws=ws)
+        J().jab_loss_backward_weights(c.desc, B, T, c.X, c.W, A, 2, s, loss, grad_sqnorm=sq2, ws=ws)
+    finally:
+        J().jab_set_deterministic(False)
+    np.testing.assert_allclose(sq.item(), (dw.double() ** 2).sum().item(), rtol=1e-12)
+    assert sq.item() == sq2.item()
+    parts = torch.empty((1, B, 4), dtype=torch.float64, device="cuda")
+    J().jab_loss_forward(c.desc, B, T, c.X, c.W, A, [2], [s], loss, ws, sse_parts=parts)
+    np.testing.assert_allclose(loss.item(), parts.sum().item() / (B * T * 4 * 64), rtol=1e-13)
+    assert J().jab_get_device_status() == 0
