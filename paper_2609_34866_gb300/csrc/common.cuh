@@ -92,6 +92,20 @@ __device__ __forceinline__ float warp_sum(float x) {
   return x;
 }
 
+// a + b = s + e exactly (Knuth).
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+// Adds the unevaluated pair (h, l) to (hi, lo): about 2^-46 of the sum is lost.
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float h, float l) {
+  float s, e;
+  two_sum(hi, h, s, e);
+  hi = s;
+  lo = __fadd_rn(__fadd_rn(lo, l), e);
+}
+
 // Block-wide sum in a fixed order (deterministic); every thread gets the result.
 template <int NT>
 __device__ __forceinline__ double block_sum(double x, double* smem /* >= NT/32 */) {
@@ -105,6 +119,26 @@ __device__ __forceinline__ double block_sum(double x, double* smem /* >= NT/32 *
   for (int i = 0; i < NT / 32; ++i) t += smem[i];
   return t;
 }
+
+// Division of 0 <= n < 2^30 by a constant of the launch, 1 <= d < 2^30: one wide multiplication by
+// floor(2^k / d) + 1, k = 30 + ceil(log2 d), exact as n (that d - 2^k) < 2^k. A tile's indices take
+// four or five quotients, each some 200 clocks of dependent instructions as plain integer divisions, at a
+// point where every role of a persistent kernel waits for them.
+struct FastDiv {
+  uint64_t m;
+  int d, k;
+  FastDiv() = default;
+  explicit FastDiv(int div) : d(div) {
+    k = 30;
+    while ((1ll << (k - 30)) < div) ++k;
+    m = ((uint64_t)1 << k) / (uint64_t)div + 1;
+  }
+  __device__ __forceinline__ int quot(int n) const { return (int)(((uint64_t)(uint32_t)n * m) >> k); }
+  __device__ __forceinline__ void divmod(int n, int& q, int& r) const {
+    q = quot(n);
+    r = n - q * d;
+  }
+};
 
 // Static schedule of a persistent kernel: the tile a CTA takes in round i when `ntiles` tiles,
 // ordered from the most work to the least, are dealt to `grid` CTAs. Rounds alternate direction

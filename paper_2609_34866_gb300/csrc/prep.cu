@@ -294,12 +294,6 @@ __global__ void rademacher_probe_kernel(uint64_t seed, uint64_t first, int64_t n
 // with the errors carried along, and only that sum goes to the fp64 accumulator: 42 us. Weights and
 // scale are first multiplied by the power of two that brings the scale to [1, 2) (exact), so that no
 // square under- or overflows; a chunk whose values leave that window takes the fp64 form.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
 // Sum of (q s - w)^2 over the 8 weights of a chunk.
 __device__ __forceinline__ double qerr_chunk(const uint4& v, float sc, int qmax) {
   const bf16_t* b = reinterpret_cast<const bf16_t*>(&v);
