@@ -38,6 +38,7 @@ struct BwdParams {
   int T, B, Hq, Hkv, lse_pitch;
   int qcol0, kcol0, vcol0;  // column offsets of Q, K, V heads in the QKV matrix
   int64_t ldt;
+  FastDiv dq_group, by_ratio, by_hkv;  // dQ tiles of a KV group; Hq / Hkv; Hkv
   int npairs;  // (query block, key block) pairs of one (sequence, head): nq (nq + 1) / 2
   float scale, sl2;
   // KL term of Eq. 3 (dK/dV kernel with KL): dS = a_mse P (dP - D) + b_kl (P - P_teacher), dV times
@@ -1025,12 +1026,12 @@ struct DqTile {
 // Tile n: grouped by (sequence, KV group), so that all tiles which read the K blocks of one KV head
 // run close together (K read from HBM once); inside a group query blocks from the last (most keys)
 // to the first, the query heads of the group next to each other.
-__device__ __forceinline__ DqTile dq_tile(int n, int nqb, int Hq, int Hkv) {
-  const int r = Hq / Hkv;
-  const int per_group = r * nqb;
-  const int grp = n / per_group, rem = n - grp * per_group;
-  const int g = grp % Hkv, b = grp / Hkv;
-  return DqTile{nqb - 1 - rem / r, g * r + rem % r, b};
+__device__ __forceinline__ DqTile dq_tile(const BwdParams& p, int n, int nqb) {
+  int grp, rem, q, hu, b, g;
+  p.dq_group.divmod(n, grp, rem);
+  p.by_ratio.divmod(rem, q, hu);
+  p.by_hkv.divmod(grp, b, g);
+  return DqTile{nqb - 1 - q, g * p.by_ratio.d + hu, b};
 }
 
 template <int DH>
@@ -1084,8 +1085,8 @@ __global__ void __launch_bounds__(DQ_THREADS, 1)
       bool ok = true;
       for (int it = 0, tile = sched_tile(0, gridDim.x, blockIdx.x); ok && tile < n_tiles;
            tile = sched_tile(++it, gridDim.x, blockIdx.x)) {
-        const DqTile tl = dq_tile(tile, nqb, p.Hq, p.Hkv);
-        const int g = tl.h / (p.Hq / p.Hkv), nkb = n_kb_of(tl);
+        const DqTile tl = dq_tile(p, tile, nqb);
+        const int g = p.by_ratio.quot(tl.h), nkb = n_kb_of(tl);
         const int64_t pair0 = ((int64_t)tl.b * p.Hq + tl.h) * p.npairs + (int64_t)tl.qb * (tl.qb + 1) / 2;
         for (int kb = 0; kb < nkb; ++kb, ++J) {
           const int st = J % NST;
@@ -1116,7 +1117,7 @@ __global__ void __launch_bounds__(DQ_THREADS, 1)
       int n = 0;
       for (int it = 0, tile = sched_tile(0, gridDim.x, blockIdx.x); ok && tile < n_tiles;
            tile = sched_tile(++it, gridDim.x, blockIdx.x), ++n) {
-        const DqTile tl = dq_tile(tile, nqb, p.Hq, p.Hkv);
+        const DqTile tl = dq_tile(p, tile, nqb);
         const int nkb = n_kb_of(tl), ob = n & 1;
         // the buffer's previous tile (n - 2) must have been read out by the epilogue
         if (n >= 2 && !tc::mbar_wait(&bars->o_empty[ob], ((n >> 1) - 1) & 1, abort, p.status)) break;
@@ -1148,7 +1149,7 @@ __global__ void __launch_bounds__(DQ_THREADS, 1)
     int n = 0;
     for (int it = 0, tile = sched_tile(0, gridDim.x, blockIdx.x); tile < n_tiles;
          tile = sched_tile(++it, gridDim.x, blockIdx.x), ++n) {
-      const DqTile tl = dq_tile(tile, nqb, p.Hq, p.Hkv);
+      const DqTile tl = dq_tile(p, tile, nqb);
       const int ob = n & 1, q0 = tl.qb * BQ;
       const bool have = tc::mbar_wait(&bars->o_full[ob], (n >> 1) & 1, abort, p.status);
       if (have) {
@@ -1269,6 +1270,9 @@ cudaError_t launch_attn_bwd_tc(const AttnLaunch& L, const float* cos_t, const fl
   p.ldt = L.ldt;
   const int nq = (L.T + 127) / 128;
   p.npairs = nq * (nq + 1) / 2;
+  p.dq_group = FastDiv(L.Hq / L.Hkv * nq);
+  p.by_ratio = FastDiv(L.Hq / L.Hkv);
+  p.by_hkv = FastDiv(L.Hkv);
   p.scale = L.scale;
   p.sl2 = L.scale * kLog2e;
   p.a_mse = kl_ab ? kl_ab[0] : 1.f;

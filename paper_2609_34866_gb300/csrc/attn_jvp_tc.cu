@@ -62,7 +62,7 @@ struct JvpBars {
   uint64_t q_full, stg_free, k_full[3], k_empty[3], vd_full[2], vd_empty[2], s_full, s_read, t_full;
   uint64_t t_read, pu_full, z_done, o_full, drain, drain_z;
   uint32_t tmem_base;
-  int abort;
+  int abort, fail[2];       // fail[tile parity]: an elementwise warp gave a wait up
   float2 red[2][EW_WARPS];  // [tile parity][warp]: sum of squares, high and low part
   float rsum[2][128];       // [key half][row] rowsum(P o dS)
 };
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     tc::mbar_init(&bars->o_full, 1);
     tc::mbar_init(&bars->drain, 1);
     tc::mbar_init(&bars->drain_z, 1);
-    bars->abort = 0;
+    bars->abort = bars->fail[0] = bars->fail[1] = 0;
     tc::fence_mbar_init();
     tc::prefetch_tmap(&tm_p);
     tc::prefetch_tmap(&tm_t);
@@ -328,7 +328,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     JvpTile tl = jvp_tile(p, k_first < p.ntiles ? k_first : 0);
     load_lse(tl);
     for (int it = 0, k = sched_tile(0, grid, cta); k < p.ntiles; k = sched_tile(++it, grid, cta)) {
-      if (*abort) break;
       const int q0 = tl.qb * BQ, nkb = tl.qb + 1, row0 = tl.b * p.T;
       const int tA = q0 + rA, tB = q0 + rB;
       const float2 nlA = make_float2(tc::neg_bits(lA * kLog2e), tc::neg_bits(lA * kLog2e));
@@ -503,6 +502,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
       float2* red = bars->red[it & 1];
       if (lane == 0) red[warp - 2] = make_float2(sq, sq_lo);
+      // All elementwise warps leave after the same tile: one that stayed would wait on the next tile's barriers.
+      if (!ok) reinterpret_cast<volatile int*>(bars->fail)[it & 1] = 1;
       tc::named_bar_sync(1, EW_WARPS * 32);  // every elementwise warp reaches this once per tile
       if (warp == 2 && ok) {
         const float2 r = red[lane & (EW_WARPS - 1)];
@@ -511,7 +512,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         for (int o = EW_WARPS / 2; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
         if (lane == 0 && in_bounds(part_at, (int64_t)p.B * p.Hq * p.nP, p.status)) p.part[part_at] = tot;
       }
-      if (!ok) break;
+      if (reinterpret_cast<volatile int*>(bars->fail)[it & 1]) break;
     }
     if (either_at_least(range_bits, kHalfInf)) report(p.status, JAB_ERR_RANGE);  // U out of the fp16 range
   }

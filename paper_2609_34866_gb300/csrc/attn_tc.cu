@@ -27,6 +27,7 @@ constexpr float kRescaleLog2 = 12.f;
 
 struct FwdParams {
   int T, B, C, Hq, Hkv, D, nqb, nP, lse_pitch;
+  FastDiv per_group, by_upg, by_hkv, by_b, by_ratio;  // tiles of a group; head units of a group; Hkv; B; Hq / Hkv
   float sl2;  // softmax scale * log2(e)
   double* part;
   const float* a_ref;
@@ -88,7 +89,7 @@ struct StackBars {
   uint64_t s_full, s_empty, p_full, pv_done, o_full[2], o_empty[2], st_full[2], st_empty[2];
   uint64_t a_full[EPI_WARPS][2], drain, drain_pv;
   uint32_t tmem_base;
-  int abort;
+  int abort, fail[2];               // fail[tile parity]: an epilogue warp gave a wait up
   double red[2][EPI_WARPS];         // [tile parity][TMEM lane quarter]
   float row_m[2][128], row_l[2][128];  // [tile parity][stacked row]: running max (log2), sum
 };
@@ -118,15 +119,15 @@ struct StackTile {
 // blocks of one KV head run close together (K and V read from HBM about once); inside a group query
 // blocks from the last (most key blocks) to the first, the head units of the group next to each
 // other. rph = query rows per head in a tile; units (query heads / HPT) is a multiple of Hkv.
-__device__ __forceinline__ StackTile stack_tile(int k, int units, int Hkv, int nqb, int T, int rph) {
-  const int upg = units / Hkv;  // head units per KV group
-  const int per_group = upg * nqb;
-  const int grp = k / per_group, rem = k - grp * per_group;
+__device__ __forceinline__ StackTile stack_tile(const FwdParams& p, int k, int rph) {
   StackTile t;
-  t.hu = (grp % Hkv) * upg + rem % upg;
-  t.bc = grp / Hkv;
-  t.qb = nqb - 1 - rem / upg;
-  t.nkb = (min((t.qb + 1) * rph, T) + SKB - 1) / SKB;
+  int grp, rem, q, hu, g;
+  p.per_group.divmod(k, grp, rem);
+  p.by_upg.divmod(rem, q, hu);
+  p.by_hkv.divmod(grp, t.bc, g);
+  t.hu = g * p.by_upg.d + hu;
+  t.qb = p.nqb - 1 - q;
+  t.nkb = (min((t.qb + 1) * rph, p.T) + SKB - 1) / SKB;
   return t;
 }
 
@@ -149,10 +150,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   StackBars* bars = reinterpret_cast<StackBars*>(smem + L::BAR_OFF);
   const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   volatile int* abort = &bars->abort;
-  const int units = p.Hq / HPT, BC = p.B * p.C;
-  const int nqb = (p.T + RPH - 1) / RPH;
-  const int ntiles = units * BC * nqb;
-  const int ratio = p.Hq / p.Hkv;
+  const int ntiles = p.Hq / HPT * p.B * p.C * p.nqb;
 
   if (threadIdx.x == 0) {
     tc::mbar_init(&bars->q_full, 1);
@@ -179,7 +177,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       for (int i = 0; i < 2; ++i) tc::mbar_init(&bars->a_full[w][i], 1);
     tc::mbar_init(&bars->drain, 1);
     tc::mbar_init(&bars->drain_pv, 1);
-    bars->abort = 0;
+    bars->abort = bars->fail[0] = bars->fail[1] = 0;
     tc::fence_mbar_init();
     tc::prefetch_tmap(&tm_q);
     tc::prefetch_tmap(&tm_kv);
@@ -207,8 +205,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       const int NST = is_v ? SV_ST : SK_ST;
       for (int it = 0, k = sched_tile(0, gridDim.x, blockIdx.x); ok && k < ntiles;
            k = sched_tile(++it, gridDim.x, blockIdx.x), ++tc_) {
-        const StackTile tl = stack_tile(k, units, p.Hkv, nqb, p.T, RPH);
-        const int b = tl.bc % p.B, c = tl.bc / p.B, h0 = HPT * tl.hu, g = h0 / ratio;
+        const StackTile tl = stack_tile(p, k, RPH);
+        int b, c;
+        p.by_b.divmod(tl.bc, c, b);
+        const int h0 = HPT * tl.hu, g = p.by_ratio.quot(h0);
         const int row0 = b * p.T, q0 = tl.qb * RPH;
         const int col = c * p.D + (is_v ? p.Hq + p.Hkv + g : p.Hq + g) * DH;
         if (!is_v) {
@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       if (warp == 1) {
         if (k < ntiles) ok = load_q(0) && issue_s(0);
         while (ok && k < ntiles) {
-          const StackTile tl = stack_tile(k, units, p.Hkv, nqb, p.T, RPH);
+          const StackTile tl = stack_tile(p, k, RPH);
           const int kn = sched_tile(it + 1, gridDim.x, blockIdx.x);
           for (int j = 0; ok && j < tl.nkb; ++j) {
             const int gg = g0 + j;
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         }
       } else {
         while (ok && k < ntiles) {
-          const StackTile tl = stack_tile(k, units, p.Hkv, nqb, p.T, RPH);
+          const StackTile tl = stack_tile(p, k, RPH);
           for (int j = 0; ok && j < tl.nkb; ++j) ok = issue_pv(g0 + j, j == 0);
           if (!ok) break;
           tc::umma_commit(&bars->o_full[tc_ & 1]);
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     for (int it = 0, k = sched_tile(0, gridDim.x, blockIdx.x); k < ntiles;
          k = sched_tile(++it, gridDim.x, blockIdx.x), ++tc_) {
       if (*abort) break;
-      const StackTile tl = stack_tile(k, units, p.Hkv, nqb, p.T, RPH);
+      const StackTile tl = stack_tile(p, k, RPH);
       const int q0 = tl.qb * RPH;
       const int tA = q0 + (rA & (RPH - 1)), tB = q0 + (rB & (RPH - 1));
       const uint32_t o_col = L::O_COL + (tc_ & 1) * DH;
@@ -505,30 +505,30 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const int64_t ext_p = (int64_t)p.C * p.B * p.Hq * p.nP;       // loss partials
     // This row's A_ref (DH fp32) of tile k into L2, one line at a time.
     auto prefetch_aref = [&](int k) {
-      const StackTile tn = stack_tile(k, units, p.Hkv, nqb, p.T, RPH);
+      const StackTile tn = stack_tile(p, k, RPH);
       const int tt = tn.qb * RPH + (row & (RPH - 1));
       if (tt >= p.T) return;
-      const float* src = p.a_ref + ((int64_t)(tn.bc % p.B) * p.T + tt) * (int64_t)(p.Hq * DH) +
+      const float* src = p.a_ref + ((int64_t)(tn.bc - p.by_b.quot(tn.bc) * p.B) * p.T + tt) * (int64_t)(p.Hq * DH) +
                          (HPT * tn.hu + h_off) * DH;
 #pragma unroll
       for (int l = 0; l < NCH; ++l) tc::prefetch_line_l2(src + 32 * l);
     };
     // The loads of A_ref run two chunks ahead: the next one is chunk lch of tile lt, which is round lit's.
     int lit = 0, lk = sched_tile(0, gridDim.x, blockIdx.x), lch = 0, issued = 0;
-    StackTile lt = stack_tile(lk < ntiles ? lk : 0, units, p.Hkv, nqb, p.T, RPH);
+    StackTile lt = stack_tile(p, lk < ntiles ? lk : 0, RPH);
     auto load_next = [&] {  // the whole warp
       if (lk >= ntiles) return;
       const int i = issued & 1;
       if (tc::elect_one()) {
         tc::mbar_expect_tx(&a_full[i], 4096);
         tc::tma_load_3d(buf + 4096 * i, &tm_a, &a_full[i], (HPT * lt.hu + h_off) * DH + lch * 32,
-                        lt.qb * RPH + y_off, lt.bc % p.B);
+                        lt.qb * RPH + y_off, lt.bc - p.by_b.quot(lt.bc) * p.B);
       }
       ++issued;
       if (++lch == NCH) {
         lch = 0;
         lk = sched_tile(++lit, gridDim.x, blockIdx.x);
-        if (lk < ntiles) lt = stack_tile(lk, units, p.Hkv, nqb, p.T, RPH);
+        if (lk < ntiles) lt = stack_tile(p, lk, RPH);
       }
     };
     if (MODE != 0) {
@@ -537,9 +537,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
     for (int it = 0, k = sched_tile(0, gridDim.x, blockIdx.x); k < ntiles;
          k = sched_tile(++it, gridDim.x, blockIdx.x), ++tc_) {
-      if (*abort) break;
-      const StackTile tl = stack_tile(k, units, p.Hkv, nqb, p.T, RPH);
-      const int b = tl.bc % p.B, c = tl.bc / p.B;
+      const StackTile tl = stack_tile(p, k, RPH);
+      int b, c;
+      p.by_b.divmod(tl.bc, c, b);
       const int h = HPT * tl.hu + h_off;
       const int y0 = tl.qb * RPH + y_off;  // the warp's first query row
       const int t = y0 + lane;
@@ -645,6 +645,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         acc = warp_sum(acc);
         if (lane == 0) bars->red[ob][quarter] = acc;
       }
+      // All epilogue warps leave after the same tile: one that stayed would wait on the next tile's barrier.
+      if (!have) reinterpret_cast<volatile int*>(bars->fail)[ob] = 1;
       tc::named_bar_sync(2, EPI_WARPS * 32);  // every epilogue warp reaches this once per tile
       if (lane == 0 && y_off == 0 && have) {  // the first warp of each head adds its warps' sums
         const double* red = bars->red[ob] + quarter;
@@ -652,7 +654,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         const double v = HPT == 2 ? red[0] + red[1] : ((red[0] + red[1]) + red[2]) + red[3];
         if (in_bounds(pi, ext_p, p.status)) p.part[pi] = v;
       }
-      if (!have) break;
+      if (reinterpret_cast<volatile int*>(bars->fail)[ob]) break;
     }
     if (MODE != 1 && tc::elect_one()) tc::bulk_wait_group<0>();
     if (MODE != 0)  // loads that nobody waited for land before shared memory goes
@@ -730,7 +732,6 @@ cudaError_t launch_attn_fwd_tc(const AttnLaunch& L, int mode) {
   p.Hq = L.Hq;
   p.Hkv = L.Hkv;
   p.D = L.D;
-  p.nqb = (L.T + BQ - 1) / BQ;
   p.nP = L.nP;
   p.lse_pitch = L.lse_pitch;
   p.sl2 = L.scale * kLog2e;
@@ -744,6 +745,13 @@ cudaError_t launch_attn_fwd_tc(const AttnLaunch& L, int mode) {
   // stacked into a tile); otherwise a tile is 128 rows of one head. Same kernel either way.
   const bool pair = (L.Hq / L.Hkv) % 2 == 0;
   const int rph = pair ? SQ : BQ;
+  p.nqb = (L.T + rph - 1) / rph;
+  const int upg = L.Hq / L.Hkv / (pair ? 2 : 1);
+  p.per_group = FastDiv(upg * p.nqb);
+  p.by_upg = FastDiv(upg);
+  p.by_hkv = FastDiv(L.Hkv);
+  p.by_b = FastDiv(L.B);
+  p.by_ratio = FastDiv(L.Hq / L.Hkv);
   CUtensorMap tq, tkv, ta, td;
   const uint64_t cols = (uint64_t)L.Hq * L.dh;
   if (!tmap_rows32(&ta, mode == 0 ? L.a_out : L.a_ref, true, cols, L.T, L.B)) return cudaErrorInvalidValue;
@@ -766,6 +774,7 @@ cudaError_t launch_attn_fwd_tc(const AttnLaunch& L, int mode) {
     if (sms <= 0) sms = 1;
   }
   const int64_t ntiles = (int64_t)(L.Hq / (pair ? 2 : 1)) * L.B * L.C * ((L.T + rph - 1) / rph);
+  if (ntiles >= (1ll << 30)) return cudaErrorInvalidValue;
   const int grid = (int)std::min<int64_t>(ntiles, sms);
 #define JAB_FWD2(DH_, M_, H_) return launch_fwd_pair<DH_, M_, H_>(tq, tkv, ta, td, p, grid, L.stream)
   if (pair) {
