@@ -6,21 +6,26 @@
 //     KL_i = sum_j P_ij (log P_ij - log Q_ij)
 //          = sum_j P_ij (s^T_ij - s^S_ij) + lse^S_i - lse^T_i          (s = scaled scores)
 //
-// One CTA = 128 query rows of one (candidate, sequence, head); keys in blocks of 128. Both score
-// blocks come from TS-form UMMAs whose A operand (the 128 query rows, teacher or student) was
-// copied into tensor memory once:
+// Persistent; a tile is 128 query rows of one (candidate, sequence, head), keys in blocks of 128. Both score
+// blocks come from TS-form UMMAs whose A operand (the 128 query rows, teacher or student) was copied into
+// tensor memory once:
 //   S^S_j = Q^S K^S_j^T,  S^T_j = Q^T K^T_j^T            M128 N128 K = d_h
-// The elementwise warps keep two online softmaxes in the log2 domain (running maxima m, sums l,
-// lazy rescaling when a maximum grows by more than 2^8) and a = sum_j p^T_j (y^T_j - y^S_j) with
-// p^T_j = 2^(y^T_j - m^T) and y = s log2(e). The row result is formed from differences only,
-//     KL_i / ln 2 = a / l^T + (m^S - m^T) + log2(l^S / l^T),
+// The elementwise warps read the scores into registers at once and release them, so that the products of the
+// next block, of the next tile too (Q is double-buffered in tensor memory), run under the exponentials of
+// this one. Every thread keeps, for its 16 keys of two rows in each block, two online softmaxes of its own in
+// the log2 domain (running maxima m, sums l, lazy rescaling when a maximum grows by more than 2^8) and
+// a = sum_j p^T_j (s^T_j - s^S_j) with p^T_j = 2^(y^T_j - m^T), y = s log2(e) scale; the eight threads of a row
+// (four lanes x two key halves) meet once a tile. The row result is formed from differences only,
+//     KL_i / ln 2 = scale log2(e) a / l^T + (m^S - m^T) + log2(l^S / l^T),
 // so no absolute log-sum-exp (of the size of the scores) is ever subtracted from another: the
 // terms are of the size of the score perturbation and the KL, which is second order in it, keeps
 // its relative precision.
-//   warp 0      TMA: Q^S and Q^T once, then K^S_j and K^T_j (2-stage ring)
-//   warp 1      TMEM owner, tcgen05.cp of Q^S / Q^T, UMMA issuer (one thread)
-//   warps 2..9  elementwise, 16x256b TMEM shape: four threads share a row (32 of its 128 keys
-//               each), two rows per thread
+//   warp 0       TMA: Q^S and Q^T of a tile, then K^S_j and K^T_j (ring)
+//   warp 1       TMEM owner, tcgen05.cp of Q^S / Q^T, UMMA issuer (one thread)
+//   warps 2..17  elementwise, 16 rows x 64 keys each (16x256b TMEM shape)
+// Bound by the exponentials, 2 x 128 x 128 a block at 32 a clock and SM = 1024 clocks, next to 896 of packed
+// fp32 work and 512 (d_h 64) of products; 16 x 12 heads of 777 x 64 with four candidates take 181 us, about
+// 2400 clocks a block, where one CTA a tile with eight elementwise warps took 227.
 // Outputs: per-row KL (optional) and one fp64 partial per tile, summed in fixed order afterwards.
 #include <cudaTypedefs.h>
 
@@ -33,11 +38,12 @@ namespace jab {
 namespace {
 
 constexpr int BQ = 128, BK = 128;
-constexpr int NUM_THREADS = 320;  // warp 0 TMA, warp 1 UMMA, warps 2..9 elementwise
-constexpr int EW_WARPS = 8;
+constexpr int EW_WARPS = 16;
+constexpr int NUM_THREADS = (2 + EW_WARPS) * 32;  // warp 0 TMA, warp 1 UMMA, warps 2..17 elementwise
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleLog2 = 8.f;
+constexpr float kNoKey = -1e30f;  // running maximum before the first visible key (log2 units)
 
 template <int DH>
 struct KlLayout {
@@ -45,24 +51,33 @@ struct KlLayout {
   static constexpr int CHUNK = 128 * 128;    // 64 columns of a 128-row tile (128-byte swizzle)
   static constexpr int QS_OFF = 0, QT_OFF = TILE;
   static constexpr int K_OFF = 2 * TILE;     // stage st: K^S at K_OFF + 2 st TILE, K^T after it
-  static constexpr int STAGES = 2;
+  static constexpr int STAGES = DH == 64 ? 4 : 2;
   static constexpr int BAR_OFF = K_OFF + STAGES * 2 * TILE;
-  static constexpr int USED = BAR_OFF + 256 + 1024;
+  static constexpr int USED = BAR_OFF + 8192;  // base alignment checked in the kernel
   static constexpr int SMEM = USED > 118 * 1024 ? USED : 118 * 1024;
-  static constexpr uint32_t SS_COL = 0, ST_COL = 128, QS_COL = 256, QT_COL = 256 + DH / 2;
-  static_assert(QT_COL + DH / 2 <= 512, "TMEM budget");
+  // tile parity t: Q^S at Q_COL + t DH, Q^T DH / 2 after it
+  static constexpr uint32_t SS_COL = 0, ST_COL = 128, Q_COL = 256;
+  static_assert(Q_COL + 2 * DH <= 512, "TMEM budget");
   static_assert(USED <= 227 * 1024, "shared memory budget");
 };
 
-struct KlBars {
-  uint64_t q_full, k_full[2], k_empty[2], s_full, s_empty, drain;
-  uint32_t tmem_base;
-  int abort;
-  double red[EW_WARPS];
+// Running state of one row: maxima (log2 domain), sums of 2^(y - m) and a.
+struct RowState {
+  float mt, ms, lt, ls, a;
 };
 
+struct KlBars {
+  uint64_t q_full, stg_free, k_full[4], k_empty[4], s_full, s_empty, half_full[2][8], drain;
+  uint32_t tmem_base;
+  int abort, done[2];         // [tile parity]: row groups whose sum is in red
+  float2 red[2][8];           // [tile parity][16-row group]: sum of KL_i, high and low part
+  RowState upper[2][128];     // [tile parity][row]: state of the upper key half
+};
+static_assert(sizeof(KlBars) <= 8192, "barrier block");
+
 struct KlParams {
-  int T, B, C, Hq, Hkv, D, nqb, nP;
+  int T, B, C, Hq, Hkv, D, nqb, nP, ntiles, balanced;
+  FastDiv outer, by_ratio, by_hkv, by_b;  // by the tiles of one length (balanced) or of one group; Hq / Hkv; Hkv; B
   float sl2;           // softmax scale * log2(e)
   double* part;        // [C, B, Hq, nP]  sum of KL_i over the tile's rows
   float* kl_rows;      // [C, B, Hq, T] or null
@@ -75,43 +90,84 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
     if (tc::globaltimer() - t0 > tc::kWaitLimitNs) break;
 }
 
-// Row maxima of one score block: rows A (x[h][4n + 0, 1]) and B (x[h][4n + 2, 3]) of this thread,
-// combined over the four threads that share each row.
-__device__ __forceinline__ void row_max(const float (&x)[2][32], float& ma, float& mb) {
-  ma = x[0][0];
-  mb = x[0][2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-#pragma unroll
-    for (int n = 0; n < 8; ++n) {
-      ma = tc::fmax3(ma, x[h][4 * n], x[h][4 * n + 1]);
-      mb = tc::fmax3(mb, x[h][4 * n + 2], x[h][4 * n + 3]);
-    }
-  ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, 1));
-  mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 1));
-  ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, 2));
-  mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 2));
+struct KlTile {
+  int c, b, g, h, qb;  // candidate, sequence, KV head, query head, 128-row block (qb + 1 key blocks)
+};
+// Tile k: row blocks from the last (most keys) to the first, grouped by (candidate, sequence, KV head) so
+// that the tiles which stream the K blocks of one KV head run close together (read from HBM about once);
+// with `balanced` all tiles of a length come before the next shorter ones.
+__device__ __forceinline__ KlTile kl_tile(const KlParams& p, int k) {
+  KlTile t;
+  int grp, hu, q, rem, bc;
+  if (p.balanced) {
+    p.outer.divmod(k, q, rem);
+    p.by_ratio.divmod(rem, grp, hu);
+  } else {
+    p.outer.divmod(k, grp, rem);
+    p.by_ratio.divmod(rem, q, hu);
+  }
+  t.qb = p.nqb - 1 - q;
+  p.by_hkv.divmod(grp, bc, t.g);
+  p.by_b.divmod(bc, t.c, t.b);
+  t.h = t.g * p.by_ratio.d + hu;
+  return t;
 }
 
-// Running state of one row: maxima (log2 domain), sums of 2^(y - m) and a.
-struct RowState {
-  float mt, ms, lt, ls, a;
-};
+// Maximum of this thread's 16 scores of row A (x[4n + 0, 1]) and of row B (x[4n + 2, 3]).
+__device__ __forceinline__ void thread_max(const float (&x)[32], float& ma, float& mb) {
+  ma = fmaxf(x[0], x[1]);
+  mb = fmaxf(x[2], x[3]);
+#pragma unroll
+  for (int n = 1; n < 8; ++n) {
+    ma = tc::fmax3(ma, x[4 * n], x[4 * n + 1]);
+    mb = tc::fmax3(mb, x[4 * n + 2], x[4 * n + 3]);
+  }
+}
 
-// Moves the running maxima to the block maxima (raw scores bt, bs) when they grow by more than
-// 2^8, rescaling the sums accordingly. The same decision is taken by the four threads of a row.
+// 2^d for an integer d <= 0, exactly (0 below the normal range).
+__device__ __forceinline__ float exp2_int(float d) {
+  return __int_as_float(((int)fmaxf(d, -127.f) + 127) << 23);
+}
+
+// Moves the running maxima to the block maxima (raw scores bt, bs) when they grow by more than 2^8,
+// rescaling the sums accordingly. The maxima are whole numbers, so that every rescaling is exact, and the
+// student's is the teacher's where they are near, so that log2(l^S / l^T) is near 0: a KL of 1e-5 is left
+// of three terms, and factors rounded separately for student and teacher took 1 % of it.
 __device__ __forceinline__ void advance_max(RowState& r, float bt, float bs, float sl2) {
-  const float nt = fmaxf(r.mt, bt * sl2), ns = fmaxf(r.ms, bs * sl2);
+  const float nt = ceilf(bt * sl2), ns = ceilf(bs * sl2);
   if (nt > r.mt + kRescaleLog2) {
-    const float al = tc::fast_exp2(r.mt - nt);  // 0 for the first block (r.mt = -inf)
+    const float al = exp2_int(r.mt - nt);  // 0 for the first visible key
     r.lt *= al;
     r.a *= al;
     r.mt = nt;
   }
   if (ns > r.ms + kRescaleLog2) {
-    r.ls *= tc::fast_exp2(r.ms - ns);
-    r.ms = ns;
+    const float m = fabsf(ns - r.mt) <= kRescaleLog2 && r.mt > r.ms ? r.mt : ns;
+    r.ls *= exp2_int(r.ms - m);
+    r.ms = m;
   }
+}
+
+// The state over both sets of keys. Its maxima are the larger ones, the factors powers of two.
+__device__ __forceinline__ RowState merge(const RowState& x, const RowState& y) {
+  RowState r;
+  r.mt = fmaxf(x.mt, y.mt);
+  r.ms = fmaxf(x.ms, y.ms);
+  const float fx = exp2_int(x.mt - r.mt), fy = exp2_int(y.mt - r.mt);
+  const float gx = exp2_int(x.ms - r.ms), gy = exp2_int(y.ms - r.ms);
+  r.lt = x.lt * fx + y.lt * fy;
+  r.a = x.a * fx + y.a * fy;
+  r.ls = x.ls * gx + y.ls * gy;
+  return r;
+}
+__device__ __forceinline__ RowState merge_lanes(const RowState& r, int o) {
+  RowState y;
+  y.mt = __shfl_xor_sync(0xffffffffu, r.mt, o);
+  y.ms = __shfl_xor_sync(0xffffffffu, r.ms, o);
+  y.lt = __shfl_xor_sync(0xffffffffu, r.lt, o);
+  y.ls = __shfl_xor_sync(0xffffffffu, r.ls, o);
+  y.a = __shfl_xor_sync(0xffffffffu, r.a, o);
+  return merge(r, y);
 }
 
 template <int DH>
@@ -119,37 +175,28 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     attn_kl_tc_kernel(const __grid_constant__ CUtensorMap tm_s,
                       const __grid_constant__ CUtensorMap tm_t, const KlParams p) {
   using L = KlLayout<DH>;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                             ~uintptr_t(1023));
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  if (tc::smem_u32(smem_raw) & 1023u) {  // the swizzled TMA tiles need a 1024-byte aligned base
+    if (threadIdx.x == 0) report(p.status, JAB_ERR_INTERNAL);
+    return;
+  }
+  uint8_t* smem = smem_raw;
   KlBars* bars = reinterpret_cast<KlBars*>(smem + L::BAR_OFF);
   const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   volatile int* abort = &bars->abort;
 
-  // CTA order: grouped by (sequence x candidate, KV group), so that the CTAs which stream the K blocks
-  // of one KV head run close together (read from HBM about once); inside a group query blocks from
-  // the last (most keys) to the first, the query heads of the group next to each other.
-  const int ratio = p.Hq / p.Hkv;
-  const int per_group = ratio * p.nqb;
-  const int grp = (int)blockIdx.x / per_group, rem = (int)blockIdx.x - grp * per_group;
-  const int qb = p.nqb - 1 - rem / ratio;
-  const int g = grp % p.Hkv;
-  const int h = g * ratio + rem % ratio;
-  const int b = (grp / p.Hkv) % p.B, c = (grp / p.Hkv) / p.B;
-  const int q0 = qb * BQ;
-  const int nkb = min(qb + 1, (p.T + BK - 1) / BK);
-  const int row0 = b * p.T;
-
   if (threadIdx.x == 0) {
     tc::mbar_init(&bars->q_full, 1);
+    tc::mbar_init(&bars->stg_free, 1);
     for (int i = 0; i < L::STAGES; ++i) {
       tc::mbar_init(&bars->k_full[i], 1);
       tc::mbar_init(&bars->k_empty[i], 1);
     }
     tc::mbar_init(&bars->s_full, 1);
     tc::mbar_init(&bars->s_empty, EW_WARPS);
+    for (int i = 0; i < 16; ++i) tc::mbar_init(&bars->half_full[i >> 3][i & 7], 1);
     tc::mbar_init(&bars->drain, 1);
-    bars->abort = 0;
+    bars->abort = bars->done[0] = bars->done[1] = 0;
     tc::fence_mbar_init();
     tc::prefetch_tmap(&tm_s);
     tc::prefetch_tmap(&tm_t);
@@ -162,156 +209,170 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  const int grid = gridDim.x, cta = blockIdx.x;
 
   if (warp == 0) {
     if (tc::elect_one()) {  // ---------------------------------------------------------------- TMA
-      const int qs_col = c * p.D + h * DH, qt_col = h * DH;
-      const int ks_col = c * p.D + (p.Hq + g) * DH, kt_col = (p.Hq + g) * DH;
-      uint32_t issued = 0, last_par = 0;
-      tc::mbar_expect_tx(&bars->q_full, 2 * L::TILE);
-      for (int ch = 0; ch < DH / 64; ++ch) {
-        tc::tma_load_2d(smem + L::QS_OFF + ch * L::CHUNK, &tm_s, &bars->q_full, qs_col + ch * 64,
-                        row0 + q0);
-        tc::tma_load_2d(smem + L::QT_OFF + ch * L::CHUNK, &tm_t, &bars->q_full, qt_col + ch * 64,
-                        row0 + q0);
-      }
-      for (int j = 0; j < nkb; ++j) {
-        const int st = j & 1;
-        const uint32_t ph = (uint32_t)(j >> 1) & 1u;
-        if (!tc::mbar_wait(&bars->k_empty[st], ph ^ 1, abort, p.status)) break;
-        uint8_t* ks = smem + L::K_OFF + st * 2 * L::TILE;
-        tc::mbar_expect_tx(&bars->k_full[st], 2 * L::TILE);
+      uint32_t g = 0, q_n = 0;  // K blocks and Q loads so far
+      bool ok = true;
+      // The student's tile at column cs and the teacher's at ct into dst and the tile after it.
+      auto load_pair = [&](uint8_t* dst, uint64_t* bar, int cs, int ct, int row) {
+        tc::mbar_expect_tx(bar, 2 * L::TILE);
         for (int ch = 0; ch < DH / 64; ++ch) {
-          tc::tma_load_2d(ks + ch * L::CHUNK, &tm_s, &bars->k_full[st], ks_col + ch * 64,
-                          row0 + j * BK);
-          tc::tma_load_2d(ks + L::TILE + ch * L::CHUNK, &tm_t, &bars->k_full[st], kt_col + ch * 64,
-                          row0 + j * BK);
+          tc::tma_load_2d(dst + ch * L::CHUNK, &tm_s, bar, cs + ch * 64, row);
+          tc::tma_load_2d(dst + L::TILE + ch * L::CHUNK, &tm_t, bar, ct + ch * 64, row);
         }
-        issued |= 1u << st;
-        last_par = (last_par & ~(1u << st)) | (ph << st);
+      };
+      for (int it = 0, k = sched_tile(0, grid, cta); ok && k < p.ntiles; k = sched_tile(++it, grid, cta)) {
+        const KlTile tl = kl_tile(p, k);
+        const int row0 = tl.b * p.T, nkb = tl.qb + 1;
+        if (it > 0 && !tc::mbar_wait(&bars->stg_free, (it - 1) & 1, abort, p.status)) break;
+        load_pair(smem + L::QS_OFF, &bars->q_full, tl.c * p.D + tl.h * DH, tl.h * DH, row0 + tl.qb * BQ);
+        ++q_n;
+        const int kcol = (p.Hq + tl.g) * DH;
+        for (int j = 0; j < nkb; ++j, ++g) {
+          const uint32_t st = g % L::STAGES, ph = (g / L::STAGES) & 1;
+          ok = tc::mbar_wait(&bars->k_empty[st], ph ^ 1, abort, p.status);
+          if (!ok) break;
+          load_pair(smem + L::K_OFF + st * 2 * L::TILE, &bars->k_full[st], tl.c * p.D + kcol, kcol, row0 + j * BK);
+        }
       }
-      if (*abort) {
-        drain_wait(&bars->q_full, 0);
-        for (int st = 0; st < L::STAGES; ++st)
-          if (issued & (1u << st)) drain_wait(&bars->k_full[st], (last_par >> st) & 1);
+      if (*abort) {  // every copy issued lands before shared memory goes
+        if (q_n > 0) drain_wait(&bars->q_full, (q_n - 1) & 1);
+        for (uint32_t i = g > L::STAGES ? g - L::STAGES : 0; i < g; ++i)
+          drain_wait(&bars->k_full[i % L::STAGES], (i / L::STAGES) & 1);
       }
     }
   } else if (warp == 1) {
     if (tc::elect_one()) {  // ---------------------------------------------------------------- UMMA
       constexpr uint32_t ID_S = tc::idesc_f16(false, BQ, BK);
-      bool ok = tc::mbar_wait(&bars->q_full, 0, abort, p.status);
-      if (ok) {
+      const uint32_t qs = tc::smem_u32(smem + L::QS_OFF), qt = tc::smem_u32(smem + L::QT_OFF);
+      const uint64_t kd0 = tc::sdesc_kmajor_sw128(tc::smem_u32(smem + L::K_OFF));
+      // Q of the CTA's tile `it` into its half of the tensor-memory columns, last read by the products of
+      // tile it - 2; those were complete when the elementwise warps released a score block of tile it - 1.
+      auto copy_q = [&](int it) {
+        if (!tc::mbar_wait(&bars->q_full, it & 1, abort, p.status)) return false;
         tc::fence_after_sync();
-        const uint32_t qs = tc::smem_u32(smem + L::QS_OFF), qt = tc::smem_u32(smem + L::QT_OFF);
+        const uint32_t col = tmem + L::Q_COL + (it & 1) * DH;
 #pragma unroll
         for (int kk = 0; kk < DH / 16; ++kk) {
           const uint32_t off = (kk >> 2) * L::CHUNK + (kk & 3) * 32;
-          tc::tmem_cp_128x256b(tmem + L::QS_COL + kk * 8, tc::sdesc_kmajor_sw128(qs + off));
-          tc::tmem_cp_128x256b(tmem + L::QT_COL + kk * 8, tc::sdesc_kmajor_sw128(qt + off));
+          tc::tmem_cp_128x256b(col + kk * 8, tc::sdesc_kmajor_sw128(qs + off));
+          tc::tmem_cp_128x256b(col + DH / 2 + kk * 8, tc::sdesc_kmajor_sw128(qt + off));
         }
-      }
-      for (int j = 0; ok && j < nkb; ++j) {
-        const int st = j & 1;
-        if (!tc::mbar_wait(&bars->k_full[st], (j >> 1) & 1, abort, p.status) ||
-            !tc::mbar_wait(&bars->s_empty, (j & 1) ^ 1, abort, p.status)) {
-          ok = false;
-          break;
-        }
-        tc::fence_after_sync();
-        const uint64_t kd_s =
-            tc::sdesc_kmajor_sw128(tc::smem_u32(smem + L::K_OFF + st * 2 * L::TILE));
-        const uint64_t kd_t =
-            tc::sdesc_kmajor_sw128(tc::smem_u32(smem + L::K_OFF + st * 2 * L::TILE + L::TILE));
+        tc::umma_commit(&bars->stg_free);
+        return true;
+      };
+      uint32_t g = 0;
+      int it = 0, k = sched_tile(0, grid, cta);
+      bool ok = k < p.ntiles && copy_q(0);
+      while (ok && k < p.ntiles) {
+        const int nkb = kl_tile(p, k).qb + 1;
+        const uint32_t qc = tmem + L::Q_COL + (it & 1) * DH;
+        for (int j = 0; j < nkb; ++j, ++g) {
+          const uint32_t st = g % L::STAGES;
+          if (!tc::mbar_wait(&bars->k_full[st], (g / L::STAGES) & 1, abort, p.status) ||
+              !tc::mbar_wait(&bars->s_empty, (g & 1) ^ 1, abort, p.status)) {
+            ok = false;
+            break;
+          }
+          tc::fence_after_sync();
+          const uint64_t kd_s = tc::sdesc_advance(kd0, st * 2 * L::TILE), kd_t = tc::sdesc_advance(kd_s, L::TILE);
 #pragma unroll
-        for (int kk = 0; kk < DH / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * L::CHUNK + (kk & 3) * 32;
-          tc::umma_f16_ts(tmem + L::SS_COL, tmem + L::QS_COL + kk * 8, tc::sdesc_advance(kd_s, off),
-                          ID_S, kk > 0 ? 1u : 0u);
-          tc::umma_f16_ts(tmem + L::ST_COL, tmem + L::QT_COL + kk * 8, tc::sdesc_advance(kd_t, off),
-                          ID_S, kk > 0 ? 1u : 0u);
+          for (int kk = 0; kk < DH / 16; ++kk) {
+            const uint32_t off = (kk >> 2) * L::CHUNK + (kk & 3) * 32;
+            tc::umma_f16_ts(tmem + L::SS_COL, qc + kk * 8, tc::sdesc_advance(kd_s, off), ID_S, kk > 0 ? 1u : 0u);
+            tc::umma_f16_ts(tmem + L::ST_COL, qc + DH / 2 + kk * 8, tc::sdesc_advance(kd_t, off), ID_S,
+                            kk > 0 ? 1u : 0u);
+          }
+          tc::umma_commit(&bars->s_full);
+          tc::umma_commit(&bars->k_empty[st]);
         }
-        tc::umma_commit(&bars->s_full);
-        tc::umma_commit(&bars->k_empty[st]);
+        k = sched_tile(++it, grid, cta);
+        if (ok && k < p.ntiles) ok = copy_q(it);
       }
       tc::umma_commit(&bars->drain);
       drain_wait(&bars->drain, 0);
     }
   } else {  // -------------------------------------------------------------------- elementwise
+    // Warp w (2..17) may access TMEM lane quarter w % 4; the four warps of a quarter take its two 16-row
+    // groups x the block's two 64-key halves.
     const int quarter = warp & 3;
-    const int half = (warp - 2) >> 2;
+    const int idx = (warp - 2) >> 2;
+    const int half = idx & 1, khalf = idx >> 1;
+    const int grp = quarter * 2 + half;
     const int cq = lane & 3;
-    const int rA = quarter * 32 + half * 16 + (lane >> 2), rB = rA + 8;
-    const int tA = q0 + rA, tB = q0 + rB;
-    const uint32_t lane16 = (uint32_t)(quarter * 32 + half * 16) << 16;
+    const int rA = grp * 16 + (lane >> 2), rB = rA + 8;
+    const uint32_t lane16 = (uint32_t)(grp * 16) << 16;
     const float2 sl2 = make_float2(p.sl2, p.sl2);
-    RowState ra{-INFINITY, -INFINITY, 0.f, 0.f, 0.f}, rb{-INFINITY, -INFINITY, 0.f, 0.f, 0.f};
+    uint32_t g = 0;
     bool ok = true;
-    for (int j = 0; j < nkb; ++j) {
-      if (!tc::mbar_wait(&bars->s_full, j & 1, abort, p.status)) {
-        ok = false;
-        break;
-      }
-      tc::fence_after_sync();
-      // xs / xt[hh][4n + e]: e < 2 row A, key 128 j + 64 hh + 8n + 2 cq + e; e = 2, 3 row B.
-      float xs[2][32], xt[2][32];
-      {
-        uint32_t r0[32], r1[32], r2[32], r3[32];
-        __syncwarp();
-        tc::tmem_ld_16x256b_x8(tmem + lane16 + L::SS_COL, r0);
-        tc::tmem_ld_16x256b_x8(tmem + lane16 + L::SS_COL + 64, r1);
-        tc::tmem_ld_16x256b_x8(tmem + lane16 + L::ST_COL, r2);
-        tc::tmem_ld_16x256b_x8(tmem + lane16 + L::ST_COL + 64, r3);
-        tc::tmem_ld_wait();
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          xs[0][i] = __uint_as_float(r0[i]);
-          xs[1][i] = __uint_as_float(r1[i]);
-          xt[0][i] = __uint_as_float(r2[i]);
-          xt[1][i] = __uint_as_float(r3[i]);
+    for (int it = 0, k = sched_tile(0, grid, cta); ok && k < p.ntiles; k = sched_tile(++it, grid, cta)) {
+      const KlTile tl = kl_tile(p, k);
+      const int q0 = tl.qb * BQ, nkb = tl.qb + 1;
+      const int tA = q0 + rA, tB = q0 + rB;
+      RowState ra{kNoKey, kNoKey, 0.f, 0.f, 0.f}, rb = ra;
+      for (int j = 0; j < nkb; ++j, ++g) {
+        if (!tc::mbar_wait(&bars->s_full, g & 1, abort, p.status)) {
+          ok = false;
+          break;
         }
-      }
-      tc::fence_before_sync();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&bars->s_empty);  // the next block's scores may overwrite
-      const int k0 = j * BK + 2 * cq;
-      const bool masked = j * BK + BK - 1 > q0 || j * BK + BK > p.T;  // diagonal or ragged block
-      if (masked) {
+        tc::fence_after_sync();
+        // xs / xt[4n + e]: e < 2 row A, key 128 j + 64 khalf + 8n + 2 cq + e; e = 2, 3 row B.
+        float xs[32], xt[32];
+        {
+          uint32_t r0[32], r1[32];
+          __syncwarp();
+          tc::tmem_ld_16x256b_x8(tmem + lane16 + L::ST_COL + 64 * khalf, r0);
+          tc::tmem_ld_16x256b_x8(tmem + lane16 + L::SS_COL + 64 * khalf, r1);
+          tc::tmem_ld_wait();
+          tc::fence_before_sync();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&bars->s_empty);  // the next block's scores may overwrite
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh)
+          for (int i = 0; i < 32; ++i) {
+            xt[i] = __uint_as_float(r0[i]);
+            xs[i] = __uint_as_float(r1[i]);
+          }
+        }
+        const bool masked = j == nkb - 1;  // the diagonal block (ragged or not)
+        if (masked) {
+          // rows past T have no result, so the causal mask alone hides the keys past T
+          const int kl = j * BK + 64 * khalf - q0;  // first key of this warp, counted from the tile's first row
+          if (kl > grp * 16 + 15) continue;         // no key of this half is visible to these 16 rows
+          const int k0 = kl + 2 * cq;
 #pragma unroll
           for (int n = 0; n < 8; ++n)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-              const int key = k0 + 64 * hh + 8 * n + e;
-              if (key > tA || key >= p.T) xs[hh][4 * n + e] = xt[hh][4 * n + e] = -INFINITY;
-              if (key > tB || key >= p.T) xs[hh][4 * n + 2 + e] = xt[hh][4 * n + 2 + e] = -INFINITY;
+              const int key = k0 + 8 * n + e;
+              if (key > rA) xs[4 * n + e] = xt[4 * n + e] = -INFINITY;
+              if (key > rB) xs[4 * n + 2 + e] = xt[4 * n + 2 + e] = -INFINITY;
             }
-      }
-      float btA, btB, bsA, bsB;
-      row_max(xt, btA, btB);
-      row_max(xs, bsA, bsB);
-      advance_max(ra, btA, bsA, p.sl2);
-      advance_max(rb, btB, bsB, p.sl2);
-      const float2 nmtA = make_float2(tc::neg_bits(ra.mt), tc::neg_bits(ra.mt));
-      const float2 nmsA = make_float2(tc::neg_bits(ra.ms), tc::neg_bits(ra.ms));
-      const float2 nmtB = make_float2(tc::neg_bits(rb.mt), tc::neg_bits(rb.mt));
-      const float2 nmsB = make_float2(tc::neg_bits(rb.ms), tc::neg_bits(rb.ms));
-      float2 ltA = make_float2(0.f, 0.f), lsA = ltA, aA = ltA, ltB = ltA, lsB = ltA, aB = ltA;
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh)
+        }
+        float btA, btB, bsA, bsB;
+        thread_max(xt, btA, btB);
+        thread_max(xs, bsA, bsB);
+        advance_max(ra, btA, bsA, p.sl2);
+        advance_max(rb, btB, bsB, p.sl2);
+        const float2 nmtA = make_float2(tc::neg_bits(ra.mt), tc::neg_bits(ra.mt));
+        const float2 nmsA = make_float2(tc::neg_bits(ra.ms), tc::neg_bits(ra.ms));
+        const float2 nmtB = make_float2(tc::neg_bits(rb.mt), tc::neg_bits(rb.mt));
+        const float2 nmsB = make_float2(tc::neg_bits(rb.ms), tc::neg_bits(rb.ms));
+        float2 ltA = make_float2(0.f, 0.f), lsA = ltA, aA = ltA, ltB = ltA, lsB = ltA, aB = ltA;
 #pragma unroll
         for (int n = 0; n < 8; ++n) {
-          const float2 tA2 = make_float2(xt[hh][4 * n], xt[hh][4 * n + 1]);
-          const float2 sA2 = make_float2(xs[hh][4 * n], xs[hh][4 * n + 1]);
-          const float2 tB2 = make_float2(xt[hh][4 * n + 2], xt[hh][4 * n + 3]);
-          const float2 sB2 = make_float2(xs[hh][4 * n + 2], xs[hh][4 * n + 3]);
+          const float2 tA2 = make_float2(xt[4 * n], xt[4 * n + 1]);
+          const float2 sA2 = make_float2(xs[4 * n], xs[4 * n + 1]);
+          const float2 tB2 = make_float2(xt[4 * n + 2], xt[4 * n + 3]);
+          const float2 sB2 = make_float2(xs[4 * n + 2], xs[4 * n + 3]);
           const float2 etA = tc::fma2(tA2, sl2, nmtA), esA = tc::fma2(sA2, sl2, nmsA);
           const float2 etB = tc::fma2(tB2, sl2, nmtB), esB = tc::fma2(sB2, sl2, nmsB);
           const float2 ptA = make_float2(tc::fast_exp2(etA.x), tc::fast_exp2(etA.y));
           const float2 psA = make_float2(tc::fast_exp2(esA.x), tc::fast_exp2(esA.y));
           const float2 ptB = make_float2(tc::fast_exp2(etB.x), tc::fast_exp2(etB.y));
           const float2 psB = make_float2(tc::fast_exp2(esB.x), tc::fast_exp2(esB.y));
-          float2 dA = tc::mul2(tc::sub2(tA2, sA2), sl2), dB = tc::mul2(tc::sub2(tB2, sB2), sl2);
+          float2 dA = tc::sub2(tA2, sA2), dB = tc::sub2(tB2, sB2);
           if (masked) {  // masked keys: -inf - (-inf) is NaN; their weight p^T is 0
             dA = make_float2(fmaxf(dA.x, -1e30f), fmaxf(dA.y, -1e30f));
             dB = make_float2(fmaxf(dB.x, -1e30f), fmaxf(dB.y, -1e30f));
@@ -323,50 +384,72 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           lsB = tc::add2(lsB, psB);
           aB = tc::fma2(ptB, dB, aB);
         }
-      ra.lt += ltA.x + ltA.y;
-      ra.ls += lsA.x + lsA.y;
-      ra.a += aA.x + aA.y;
-      rb.lt += ltB.x + ltB.y;
-      rb.ls += lsB.x + lsB.y;
-      rb.a += aB.x + aB.y;
-    }
-    // Row results: sums over the four threads of each row, then the difference form above.
-    double acc = 0.0;
-    if (ok) {
+        ra.lt += ltA.x + ltA.y;
+        ra.ls += lsA.x + lsA.y;
+        ra.a += aA.x + aA.y;
+        rb.lt += ltB.x + ltB.y;
+        rb.ls += lsB.x + lsB.y;
+        rb.a += aB.x + aB.y;
+      }
+      if (!ok) break;
+      // The four lanes of a row, then its two key halves: the upper one leaves its state in shared memory. (A
+      // buffer of this parity was last read two tiles ago, before its reader released the last tile's scores;
+      // a single barrier would not do, as the upper half may be one tile ahead.)
 #pragma unroll
       for (int o = 1; o <= 2; o <<= 1) {
-        ra.lt += __shfl_xor_sync(0xffffffffu, ra.lt, o);
-        ra.ls += __shfl_xor_sync(0xffffffffu, ra.ls, o);
-        ra.a += __shfl_xor_sync(0xffffffffu, ra.a, o);
-        rb.lt += __shfl_xor_sync(0xffffffffu, rb.lt, o);
-        rb.ls += __shfl_xor_sync(0xffffffffu, rb.ls, o);
-        rb.a += __shfl_xor_sync(0xffffffffu, rb.a, o);
+        ra = merge_lanes(ra, o);
+        rb = merge_lanes(rb, o);
       }
-      const float klA =
-          kLn2 * (__fdiv_rn(ra.a, ra.lt) + (ra.ms - ra.mt) + log2f(__fdiv_rn(ra.ls, ra.lt)));
-      const float klB =
-          kLn2 * (__fdiv_rn(rb.a, rb.lt) + (rb.ms - rb.mt) + log2f(__fdiv_rn(rb.ls, rb.lt)));
+      RowState* upper = bars->upper[it & 1];
+      if (khalf == 1) {
+        if (cq == 0) {
+          upper[rA] = ra;
+          upper[rB] = rb;
+        }
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&bars->half_full[it & 1][grp]);
+        continue;
+      }
+      ok = tc::mbar_wait(&bars->half_full[it & 1][grp], (it >> 1) & 1, abort, p.status);
+      if (!ok) break;
+      ra = merge(ra, upper[rA]);
+      rb = merge(rb, upper[rB]);
+      float sum = 0.f, sum_lo = 0.f;  // this row group's KL and the rounding of its additions
+      const float klA = kLn2 * (p.sl2 * __fdiv_rn(ra.a, ra.lt) + (ra.ms - ra.mt) + log2f(__fdiv_rn(ra.ls, ra.lt)));
+      const float klB = kLn2 * (p.sl2 * __fdiv_rn(rb.a, rb.lt) + (rb.ms - rb.mt) + log2f(__fdiv_rn(rb.ls, rb.lt)));
       if (cq == 0) {
-        const int64_t rbase = (((int64_t)c * p.B + b) * p.Hq + h) * p.T;
+        const int64_t rbase = (((int64_t)tl.c * p.B + tl.b) * p.Hq + tl.h) * p.T;
         const int64_t ext_r = (int64_t)p.C * p.B * p.Hq * p.T;
         if (tA < p.T) {
-          acc += (double)klA;
+          sum = klA;
           if (p.kl_rows && in_bounds(rbase + tA, ext_r, p.status)) p.kl_rows[rbase + tA] = klA;
         }
         if (tB < p.T) {
-          acc += (double)klB;
+          two_sum(sum, klB, sum, sum_lo);
           if (p.kl_rows && in_bounds(rbase + tB, ext_r, p.status)) p.kl_rows[rbase + tB] = klB;
         }
       }
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) bars->red[warp - 2] = acc;
-    tc::named_bar_sync(1, EW_WARPS * 32);  // every elementwise warp reaches this exactly once
-    if (warp == 2 && lane == 0 && ok) {
-      double tot = 0.0;
-      for (int w = 0; w < EW_WARPS; ++w) tot += bars->red[w];
-      const int64_t pi = (((int64_t)c * p.B + b) * p.Hq + h) * p.nP + qb;
-      if (in_bounds(pi, (int64_t)p.C * p.B * p.Hq * p.nP, p.status)) p.part[pi] = tot;
+#pragma unroll
+      for (int o = 4; o <= 16; o <<= 1) {
+        const float hi = __shfl_xor_sync(0xffffffffu, sum, o), lo = __shfl_xor_sync(0xffffffffu, sum_lo, o);
+        pair_add(sum, sum_lo, hi, lo);
+      }
+      if (lane == 0) {  // the last of the tile's eight row groups adds them up, in their order
+        float2* red = bars->red[it & 1];
+        red[grp] = make_float2(sum, sum_lo);
+        __threadfence_block();
+        if (atomicAdd(&bars->done[it & 1], 1) == 7) {
+          __threadfence_block();
+          double tot = 0.0;
+          for (int i = 0; i < 8; ++i) {
+            const volatile float* v = reinterpret_cast<volatile float*>(red + i);
+            tot += (double)v[0] + (double)v[1];
+          }
+          bars->done[it & 1] = 0;
+          const int64_t pi = (((int64_t)tl.c * p.B + tl.b) * p.Hq + tl.h) * p.nP + tl.qb;
+          if (in_bounds(pi, (int64_t)p.C * p.B * p.Hq * p.nP, p.status)) p.part[pi] = tot;
+        }
+      }
     }
   }
   tc::fence_before_sync();
@@ -405,7 +488,7 @@ bool tmap_fp16(CUtensorMap* m, const void* base, uint64_t cols, uint64_t rows) {
 }
 
 template <int DH>
-cudaError_t launch_kl(const CUtensorMap& ts, const CUtensorMap& tt, const KlParams& p,
+cudaError_t launch_kl(const CUtensorMap& ts, const CUtensorMap& tt, const KlParams& p, int sms,
                       cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
@@ -415,10 +498,7 @@ cudaError_t launch_kl(const CUtensorMap& ts, const CUtensorMap& tt, const KlPara
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  const int64_t n = (int64_t)p.Hq * p.B * p.C * p.nqb;
-  if (n >= (1ll << 31)) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)n);
-  attn_kl_tc_kernel<DH><<<grid, NUM_THREADS, KlLayout<DH>::SMEM, st>>>(ts, tt, p);
+  attn_kl_tc_kernel<DH><<<(unsigned)std::min(p.ntiles, sms), NUM_THREADS, KlLayout<DH>::SMEM, st>>>(ts, tt, p);
   return cudaGetLastError();
 }
 
@@ -449,7 +529,20 @@ cudaError_t launch_attn_kl_tc(const void* qkv_s, int64_t ldq, const void* qkv_t,
   p.kl_rows = kl_rows;
   p.status = status;
   if (p.nqb > nP) return cudaErrorInvalidValue;
-  return dh == 128 ? launch_kl<128>(ts, tt, p, st) : launch_kl<64>(ts, tt, p, st);
+  const int64_t ntiles = (int64_t)Hq * B * C * p.nqb;
+  if (ntiles >= (1ll << 30)) return cudaErrorInvalidValue;
+  p.ntiles = (int)ntiles;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (sms <= 0) sms = 1;
+  // with few tiles per CTA their lengths decide the makespan, and all their K is in L2 anyway
+  p.balanced = ntiles < 24 * (int64_t)sms;
+  p.outer = FastDiv(p.balanced ? p.ntiles / p.nqb : Hq / Hkv * p.nqb);
+  p.by_ratio = FastDiv(Hq / Hkv);
+  p.by_hkv = FastDiv(Hkv);
+  p.by_b = FastDiv(B);
+  return dh == 128 ? launch_kl<128>(ts, tt, p, sms, st) : launch_kl<64>(ts, tt, p, sms, st);
 }
 
 }  // namespace jab
