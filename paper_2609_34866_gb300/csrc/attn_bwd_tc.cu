@@ -294,6 +294,7 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  stream_order();
 
   if (warp == 0) {
     if (tc::elect_one()) {  // ------------------------------------------------------------- TMA
@@ -795,6 +796,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  stream_order();
 
   if (warp == 0) {
     if (tc::elect_one()) {  // ------------------------------------------------------------- TMA
@@ -1078,6 +1080,7 @@ __global__ void __launch_bounds__(DQ_THREADS, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  stream_order();
 
   if (warp == 0) {
     if (tc::elect_one()) {  // ---------------------------------------------------------------- TMA
@@ -1236,22 +1239,15 @@ cudaError_t launch_bwd(const AttnLaunch& L, const BwdParams& p, bool kl) {
   if (e != cudaSuccess) return e;
   const int64_t n_dkdv = (int64_t)L.Hkv * L.B * ((L.T + 127) / 128);
   if (n_dkdv >= (1ll << 31)) return cudaErrorInvalidValue;
-  const dim3 g1((unsigned)n_dkdv);
-  if (kl)
-    attn_bwd_dkdv_tc_kernel<DH, true><<<g1, DKDV_THREADS, DkdvLayout<DH>::SMEM, L.stream>>>(
-        kv128, do128, ds128, p);
-  else
-    attn_bwd_dkdv_tc_kernel<DH, false><<<g1, DKDV_THREADS, DkdvLayout<DH>::SMEM, L.stream>>>(
-        kv128, do128, ds128, p);
-  e = cudaGetLastError();
+  e = launch_after(kl ? attn_bwd_dkdv_tc_kernel<DH, true> : attn_bwd_dkdv_tc_kernel<DH, false>, (unsigned)n_dkdv,
+                   DKDV_THREADS, DkdvLayout<DH>::SMEM, L.stream, kv128, do128, ds128, p);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t dq_tiles = (int64_t)((L.T + 127) / 128) * L.Hq * L.B;
   const unsigned g2 = (unsigned)std::min<int64_t>(dq_tiles, sms > 0 ? sms : 1);
-  attn_bwd_dq_tc_kernel<DH><<<g2, DQ_THREADS, DqLayout<DH>::SMEM, L.stream>>>(ds128, kv128, p);
-  return cudaGetLastError();
+  return launch_after(attn_bwd_dq_tc_kernel<DH>, g2, DQ_THREADS, DqLayout<DH>::SMEM, L.stream, ds128, kv128, p);
 }
 
 }  // namespace
@@ -1300,8 +1296,7 @@ cudaError_t launch_tp(const CUtensorMap& ms, const CUtensorMap& mt, const CUtens
   if (e != cudaSuccess) return e;
   const int64_t n = (int64_t)p.Hkv * p.B * ((p.T + 127) / 128);
   if (n >= (1ll << 31)) return cudaErrorInvalidValue;
-  attn_teacher_p_tc_kernel<DH><<<(unsigned)n, TP_THREADS, TpLayout<DH>::SMEM, st>>>(ms, mt, md, p);
-  return cudaGetLastError();
+  return launch_after(attn_teacher_p_tc_kernel<DH>, (unsigned)n, TP_THREADS, TpLayout<DH>::SMEM, st, ms, mt, md, p);
 }
 }  // namespace
 

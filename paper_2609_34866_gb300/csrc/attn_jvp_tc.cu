@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  stream_order();
   const int grid = gridDim.x, cta = blockIdx.x;
 
   if (warp == 0) {
@@ -562,8 +563,8 @@ cudaError_t launch_jvp(const CUtensorMap& tp, const CUtensorMap& tt, const JvpPa
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  attn_jvp_tc_kernel<DH><<<(unsigned)std::min(p.ntiles, sms), NUM_THREADS, JvpLayout<DH>::SMEM, st>>>(tp, tt, p);
-  return cudaGetLastError();
+  return launch_after(attn_jvp_tc_kernel<DH>, (unsigned)std::min(p.ntiles, sms), NUM_THREADS, JvpLayout<DH>::SMEM, st,
+                      tp, tt, p);
 }
 
 }  // namespace

@@ -209,6 +209,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  stream_order();
   const int grid = gridDim.x, cta = blockIdx.x;
 
   if (warp == 0) {
@@ -498,8 +499,8 @@ cudaError_t launch_kl(const CUtensorMap& ts, const CUtensorMap& tt, const KlPara
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  attn_kl_tc_kernel<DH><<<(unsigned)std::min(p.ntiles, sms), NUM_THREADS, KlLayout<DH>::SMEM, st>>>(ts, tt, p);
-  return cudaGetLastError();
+  return launch_after(attn_kl_tc_kernel<DH>, (unsigned)std::min(p.ntiles, sms), NUM_THREADS, KlLayout<DH>::SMEM, st,
+                      ts, tt, p);
 }
 
 }  // namespace

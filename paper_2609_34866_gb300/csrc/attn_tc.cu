@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  stream_order();
 
   if (warp == 0 || warp == 10) {
     if (tc::elect_one()) {  // --------------------------------------- TMA: Q and K (warp 0), V (10)
@@ -710,9 +711,8 @@ cudaError_t launch_fwd_pair(const CUtensorMap& tq, const CUtensorMap& tkv, const
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  attn_fwd_pair_kernel<DH, MODE, HPT>
-      <<<grid, NUM_THREADS, StackLayout<DH>::SMEM, st>>>(tq, tkv, ta, td, p);
-  return cudaGetLastError();
+  return launch_after(attn_fwd_pair_kernel<DH, MODE, HPT>, (unsigned)grid, NUM_THREADS, StackLayout<DH>::SMEM, st, tq,
+                      tkv, ta, td, p);
 }
 
 }  // namespace

@@ -395,6 +395,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   // both CTAs' barriers are initialised and their tensor memory allocated before any signal crosses
   tc::cluster_sync();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  stream_order();
   const uint32_t full_lead = tc::mapa_shared(tc::smem_u32(&bars->full[0]), 0);
   const uint32_t tempty_lead = tc::mapa_shared(tc::smem_u32(&bars->tempty[0]), 0);
 
@@ -568,7 +569,7 @@ cudaError_t launch_gemm2(const CUtensorMap& ta, const CUtensorMap& tb, const CUt
     attr_set = true;
   }
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2;
   at[0].val.clusterDim.y = 1;
@@ -590,6 +591,9 @@ cudaError_t launch_gemm2(const CUtensorMap& ta, const CUtensorMap& tb, const CUt
   const int64_t total = (int64_t)p.num_m * p.num_n * p.splits;
   const int pairs = (int)std::min<int64_t>(total, std::min(clusters, sms / 2));
   cfg.gridDim = dim3((unsigned)(2 * pairs));
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // stream_order() in the kernel
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, ta, tb, tcm, p);
 }
 

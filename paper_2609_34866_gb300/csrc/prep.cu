@@ -249,6 +249,7 @@ __device__ __forceinline__ void rope_role(const PrepArgs& p, int blk) {
 // 4096 weights and 30-85 us for the table (1337-4096 rows), now 31 us together at 1337 rows; for five
 // candidates, 2048 rows and 65536 x 4096 of X 462 us, now 248 us (1.37 GB: 202 us at the copy rate).
 __global__ void __launch_bounds__(256, 4) prep_kernel(const __grid_constant__ PrepArgs p) {
+  stream_order();
   const int blk = blockIdx.x;
   if (blk == 0 && threadIdx.x == 0 && p.counter != nullptr) *p.counter = 0;
   if (blk < p.nrope)
@@ -609,8 +610,7 @@ cudaError_t launch_prep(const PrepInputs& in, int* status, int sms, cudaStream_t
     }
     const int grid = p.nrope + p.nw + p.nx;
     if (grid == 0) return cudaSuccess;
-    prep_kernel<<<(unsigned)grid, 256, 0, st>>>(p);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_after(prep_kernel, (unsigned)grid, 256, 0, st, p);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(32) loss_reduce_kernel(const double* __restric
                                                          double* __restrict__ parts_out,
                                                          double* __restrict__ red, int* counter,
                                                          int* status) {
+  stream_order();
   const int c = blockIdx.x / nblk, blk = blockIdx.x - c * nblk;
   const double t = loss_slice(part + (int64_t)c * nbh * nP, nbh, nP, blk, nblk,
                               parts_out ? parts_out + (int64_t)c * nbh : nullptr);
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(32) loss_reduce_kernel(const double* __restric
 
 __global__ void loss_combine_kernel(const double* __restrict__ a, const double* __restrict__ b,
                                     double lam, int C, double* __restrict__ out) {
+  stream_order();
   for (int c = threadIdx.x; c < C; c += blockDim.x) out[c] = a[c] + lam * b[c];
 }
 
@@ -166,6 +168,7 @@ __global__ void __launch_bounds__(256) sum_scaled_kernel(const double* __restric
 // Natural-log log-sum-exp rows [BH, T] to log2 units with the row pitch of the backward workspace.
 __global__ void lse_to_log2_kernel(const float* __restrict__ in, int BH, int T, int pitch,
                                    float* __restrict__ out) {
+  stream_order();
   const int64_t n = (int64_t)BH * T;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -179,6 +182,7 @@ __global__ void lse_to_log2_kernel(const float* __restrict__ in, int BH, int T, 
 // and, with KL partials, the KL value and loss + lambda KL. (Three to five launches before; 4 x 128 fit 68.7 ->
 // 64 us a call.)
 __global__ void __launch_bounds__(256) finish_kernel(const __grid_constant__ FinishArgs p) {
+  stream_order();
   bool bad = false;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -218,22 +222,19 @@ cudaError_t launch_loss_reduce(const double* part, int C, int B, int Hq, int nP,
                                double* out, double* parts_out, double* red, int* counter, int* status,
                                cudaStream_t st) {
   const int nbh = B * Hq, nblk = loss_blocks(nbh);
-  loss_reduce_kernel<<<C * nblk, 32, 0, st>>>(part, C, nbh, nP, nblk, inv_n, out, parts_out, red, counter,
-                                              status);
-  return cudaGetLastError();
+  return launch_after(loss_reduce_kernel, (unsigned)(C * nblk), 32, 0, st, part, C, nbh, nP, nblk, inv_n, out, parts_out,
+                      red, counter, status);
 }
 
 cudaError_t launch_finish(FinishArgs a, cudaStream_t st) {
   a.nblk = loss_blocks(std::max(a.nbh, a.klpart != nullptr ? a.nkl : 0));
   const int64_t blocks = std::min<int64_t>(4096, std::max<int64_t>((a.n + 255) / 256, a.nblk));
-  finish_kernel<<<(unsigned)blocks, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_after(finish_kernel, (unsigned)blocks, 256, 0, st, a);
 }
 
 cudaError_t launch_loss_combine(const double* a, const double* b, double lam, int C, double* out,
                                 cudaStream_t st) {
-  loss_combine_kernel<<<1, 128, 0, st>>>(a, b, lam, C, out);
-  return cudaGetLastError();
+  return launch_after(loss_combine_kernel, 1, 128, 0, st, a, b, lam, C, out);
 }
 
 cudaError_t launch_omega_finish(const double* part, int nblocks, int C, const double* trace,
@@ -260,8 +261,7 @@ cudaError_t launch_lse_to_log2(const float* in, int BH, int T, int pitch, float*
   int64_t blocks = ((int64_t)BH * T + 255) / 256;
   if (blocks > 4096) blocks = 4096;
   if (blocks < 1) blocks = 1;
-  lse_to_log2_kernel<<<(unsigned)blocks, 256, 0, st>>>(in, BH, T, pitch, out);
-  return cudaGetLastError();
+  return launch_after(lse_to_log2_kernel, (unsigned)blocks, 256, 0, st, in, BH, T, pitch, out);
 }
 
 cudaError_t launch_check_finite(const float* x, int64_t n, int* status, cudaStream_t st) {
