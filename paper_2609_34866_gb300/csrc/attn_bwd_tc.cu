@@ -44,6 +44,7 @@ struct BwdParams {
   // KL term of Eq. 3 (dK/dV kernel with KL): dS = a_mse P (dP - D) + b_kl (P - P_teacher), dV times
   // a_mse; the caller's coefficient of the whole gradient is divided by a_mse
   float a_mse, b_kl;
+  const uint4* pt;  // KL: the P^T tiles, in the dS^T tiles' place (pt_word)
   const float* lse;
   const float* dvec;
   const float* cos_t;
@@ -208,15 +209,23 @@ struct DkdvLayout {
 
 struct DkdvBars {
   uint64_t kv_full, q_full[3], q_empty[3], do_full, do_empty, row_full[2], row_empty[2], s_full, s_read, dp_full, dp_read, p_full, ds_full;
-  uint64_t dv_done, dk_done, o_full, drain, drain_g, dss_full, dss_free, pt_full;
+  uint64_t dv_done, dk_done, o_full, drain, drain_g, dss_full, dss_free;
   uint32_t tmem_base;
   int abort;
 };
 
 // KL: the teacher's probabilities P^T of each (query block, key block) tile were stored in the dS^T
-// tile buffer (attn_teacher_p_tc_kernel); the store warp loads the tile into the staging buffer
-// before the block's dS, the elementwise warps add b_kl (P - P^T) to a_mse P (dP - D) and write
-// dS^T over it, and the tile goes back to the same place.
+// tile's place (attn_teacher_p_tc_kernel), in the order of the elementwise threads' registers (pt_word):
+// each thread loads its 16 words while dP^T is on its way, adds b_kl (P - P^T) to a_mse P (dP - D), and the
+// dS^T tile is stored over them. (Through shared memory, where it had to share the dS^T staging tile, a
+// block's P^T could be loaded only when the previous dS^T had been stored, a round trip per block: a whole
+// fitting step of 8 x 2048 tokens took 2605 us against 2469 us.)
+
+// First of the four 16-byte words, 512 bytes apart, that a lane of elementwise warp w (0 .. 15) holds of a
+// P^T tile of 32 KB: its packed words 4 q .. 4 q + 3 in word q, so that a warp moves 512 bytes at a time.
+__device__ __forceinline__ int64_t pt_word(int64_t tile, int w, int lane) {
+  return tile * 2048 + w * 128 + lane;
+}
 template <int DH, bool KL>
 __global__ void __launch_bounds__(DKDV_THREADS, 1)
     attn_bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap tm_qkv,
@@ -279,7 +288,6 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
     tc::mbar_init(&bars->drain_g, 1);
     tc::mbar_init(&bars->dss_full, DKDV_EW);  // the block's dS^T is in the staging tile
     tc::mbar_init(&bars->dss_free, 1);         // the store warp's TMA stores have read it
-    tc::mbar_init(&bars->pt_full, 1);          // KL: the block's P^T tile is in the staging tile
     bars->abort = 0;
     tc::fence_mbar_init();
     tc::prefetch_tmap(&tm_qkv);
@@ -317,8 +325,7 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
         tc::prefetch_l2(p.dvec + lrow, BQ * 4);
         if constexpr (KL) {
           const int64_t tile = ((int64_t)b * p.Hq + hj) * p.npairs + (int64_t)ij * (ij + 1) / 2 + kb;
-          tc::tma_prefetch_2d(&tm_ds, 0, (int32_t)(tile * BK));
-          tc::tma_prefetch_2d(&tm_ds, 64, (int32_t)(tile * BK));
+          tc::prefetch_l2(p.pt + tile * 2048, 2 * L::CHUNK);
         }
       };
       int nq_ = 0, nr = 0, nd = 0;  // Q, row and dO loads issued
@@ -458,15 +465,6 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
         const int h = g * r + it / per_head, i = kb + it % per_head;
         return ((int64_t)b * p.Hq + h) * p.npairs + (int64_t)i * (i + 1) / 2 + kb;
       };
-      int pt_issued = 0;  // KL: P^T tiles loaded into the staging tile so far
-      auto load_pt = [&](int it) {  // KL: block it's P^T tile into the staging tile
-        const int32_t y = (int32_t)(tile_of(it) * BK);
-        tc::mbar_expect_tx(&bars->pt_full, 2 * L::CHUNK);
-        tc::tma_load_2d(smem + L::DSS_OFF, &tm_ds, &bars->pt_full, 0, y);
-        tc::tma_load_2d(smem + L::DSS_OFF + L::CHUNK, &tm_ds, &bars->pt_full, 64, y);
-        ++pt_issued;
-      };
-      if constexpr (KL) load_pt(0);
       for (int it = 0; it < n_it; ++it) {
         if (!tc::mbar_wait(&bars->dss_full, it & 1, abort, p.status)) break;
         const int64_t tile = tile_of(it);
@@ -474,15 +472,9 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
         tc::tma_store_2d(&tm_ds, smem + L::DSS_OFF + L::CHUNK, 64, (int32_t)(tile * BK));
         tc::bulk_commit_group();
         tc::bulk_wait_group_read<0>();  // the staging tile may be rewritten
-        if constexpr (KL) {
-          if (it + 1 < n_it) load_pt(it + 1);
-        } else {
-          tc::mbar_arrive(&bars->dss_free);
-        }
+        tc::mbar_arrive(&bars->dss_free);
       }
       tc::bulk_wait_group<0>();
-      // KL: a P^T load that nobody waited for (the loop gave up) lands before shared memory goes
-      if (KL && pt_issued > 0) drain_wait(&bars->pt_full, (pt_issued - 1) & 1);
     }
   } else {  // ------------------------------------ elementwise: 16 key rows x 64 queries per warp
     // Warp w (2..17) may access TMEM lane quarter w % 4; the four warps of a quarter take its two
@@ -559,6 +551,14 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&bars->p_full);
+      uint4 pt[4];  // KL: this thread's words of P^T, in the order of dw
+      if constexpr (KL) {
+        const int64_t tile = ((int64_t)b * p.Hq + g * r + it / per_head) * p.npairs + (int64_t)i * (i + 1) / 2 + kb;
+        const int64_t w0 = pt_word(tile, warp - 2, lane);
+        const bool in = in_bounds(w0 + 96, (int64_t)p.B * p.Hq * p.npairs * 2048, p.status);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) pt[q] = in ? __ldcg(p.pt + w0 + 32 * q) : make_uint4(0, 0, 0, 0);
+      }
       if (!tc::mbar_wait(&bars->dp_full, it & 1, abort, p.status)) {
         ok = false;
         break;
@@ -571,10 +571,6 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
       uint32_t* wa_p = reinterpret_cast<uint32_t*>(hb + rA * 128 + cq * 4);
       uint32_t* wb_p = reinterpret_cast<uint32_t*>(hb + (rA + 8) * 128 + cq * 4);
       const int swa = rA & 7, swb = (rA + 8) & 7;
-      if (KL && !tc::mbar_wait(&bars->pt_full, it & 1, abort, p.status)) {
-        ok = false;
-        break;
-      }
       {
         uint32_t rd[32];
         __syncwarp();
@@ -594,10 +590,9 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
           float2 db = tc::mul2(pb, tb);
           if constexpr (KL) {
             // + b_kl (P - P^T): the teacher's probabilities of the same entries (0 where masked)
-            const float2 qa = __half22float2(
-                *reinterpret_cast<const __half2*>(&wa_p[(n ^ swa) << 2]));
-            const float2 qb = __half22float2(
-                *reinterpret_cast<const __half2*>(&wb_p[(n ^ swb) << 2]));
+            const uint32_t ua = n & 1 ? pt[n >> 1].z : pt[n >> 1].x, ub = n & 1 ? pt[n >> 1].w : pt[n >> 1].y;
+            const float2 qa = __half22float2(*reinterpret_cast<const __half2*>(&ua));
+            const float2 qb = __half22float2(*reinterpret_cast<const __half2*>(&ub));
             const float2 am = make_float2(p.a_mse, p.a_mse), bk = make_float2(p.b_kl, p.b_kl);
             const float2 ka = tc::mul2(tc::sub2(pa, qa), bk), kb2 = tc::mul2(tc::sub2(pb, qb), bk);
             float2 ea = tc::fma2(da, am, ka), eb = tc::fma2(db, am, kb2);
@@ -621,18 +616,15 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
       }
       __syncwarp();
       tc::tmem_st_16x128b_x8(tmem + lane16 + L::DS_COL + 32 * chalf, dw);
-      auto release_ds = [&] {  // dK(j) may read dS^T
-        tc::tmem_st_wait();
-        tc::fence_before_sync();
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&bars->ds_full);
-      };
-      if (!KL) release_ds();
+      tc::tmem_st_wait();
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&bars->ds_full);  // dK(j) may read dS^T
       // The same dS^T words into the staging tile for the store warp, once it has stored the previous
       // block's: packed word n (queries 64 chalf + 8n + 2cq, +1) is 16-byte unit n of the 64-query half
-      // chalf of its key row (128-byte swizzle). With KL they go over this thread's own P^T words, loaded
-      // only after the previous block's store had read the tile, while dS^T is on its way to TMEM.
-      if (!KL && it > 0 && !tc::mbar_wait(&bars->dss_free, (it - 1) & 1, abort, p.status)) {
+      // chalf of its key row (128-byte swizzle). (With KL every thread has read its P^T words of the tile
+      // that the store goes to: dS^T depends on them.)
+      if (it > 0 && !tc::mbar_wait(&bars->dss_free, (it - 1) & 1, abort, p.status)) {
         ok = false;
         break;
       }
@@ -642,7 +634,6 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
         wb_p[(n ^ swb) << 2] = dw[2 * n + 1];
       }
       tc::fence_proxy_async_smem();
-      if (KL) release_ds();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&bars->dss_full);
     }
@@ -687,8 +678,8 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
 // The KL term of Eq. 3 (D_KL(P || Q), P the teacher's map) for the STE gradient: its gradient with
 // respect to the student's scaled scores is (lambda / B)(Q - P), so the backward needs the teacher's
 // probabilities P of every (query, key) entry that the dS tiles hold. This kernel writes P^T into
-// the dS^T tile buffer in the dS^T layout (the dK/dV kernel then reads each tile, forms dS and
-// stores it back over it), and the KL value itself, using the two softmax normalisers of the
+// the dS^T tile buffer, straight from the registers that hold it and in their order (pt_word: the dK/dV
+// kernel's threads hold the same entries of a tile; it stores dS^T over them), and the KL value itself, using the two softmax normalisers of the
 // forward passes (teacher: jab_reference_forward; student: the loss+backward forward):
 //   KL_row i = sum_j P_ij (s^T_ij - s^S_ij) + lse^S_i - lse^T_i,  s = scale Q K^T (natural units),
 //   P_ij = exp(s^T_ij - lse^T_i).
@@ -696,12 +687,14 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
 // heads and query blocks: S_t^T = K_t Q_t^T and S_s^T = K_s Q_s^T into one of two TMEM buffers
 // (the next block's products run while the elementwise warps read this one), P^T = exp2(s_t^T sl2 -
 // lse2_t) with the causal mask, the CTA's partial sum of P (s_t - s_s) (and, in the key-block-0 CTAs
-// that see every query row once, of lse^S - lse^T), and P^T staged and stored by TMA.
+// that see every query row once, of lse^S - lse^T). It writes 32 KB a block, 1.14 GB for 8 x 32 heads of 2048,
+// which take 168 us at the copy rate; the kernel takes some 310 us (363 with P^T staged in shared memory, one
+// tile at a time, and with stages that the elementwise warps held for their log-sum-exp rows). Next to the
+// stores, its SS products and the loads of 64 KB a block keep shared memory busy for 1600 of 2500 clocks.
 //   warp 0      TMA: K_t, K_s once; per block Q_t, Q_s and the two rows of lse (log2 units)
 //   warp 1      TMEM owner, UMMA issuer
 //   warps 2..17 elementwise, 16 key rows x 64 queries each (the dK/dV kernel's layout)
-//   warp 18     P^T tiles to global memory
-constexpr int TP_THREADS = (2 + DKDV_EW + 1) * 32;
+constexpr int TP_THREADS = (2 + DKDV_EW) * 32;
 
 struct TpParams {
   int T, B, Hq, Hkv, lse_pitch, npairs;
@@ -709,6 +702,7 @@ struct TpParams {
   float scale, sl2;
   const float* lse2_t;  // teacher log-sum-exp, log2 units, [B, Hq, lse_pitch]
   const float* lse2_s;  // student log-sum-exp, log2 units, [B, Hq, lse_pitch]
+  uint4* pt;            // P^T tiles (pt_word)
   double* part;         // [gridDim.x] KL partial of each CTA (natural units)
   int* status;
 };
@@ -720,18 +714,21 @@ struct TpLayout {
   static constexpr int NCH = DH / 64;
   static constexpr int KT_OFF = 0, KS_OFF = NCH * CHUNK;
   static constexpr int ST_OFF = 2 * NCH * CHUNK;
-  static constexpr int ST_QT = 0, ST_QS = NCH * CHUNK, ST_LT = 2 * NCH * CHUNK,
-                       ST_LS = ST_LT + BQ * 4, ST_BYTES = ST_LS + BQ * 4;
-  static constexpr int ST_STRIDE = (ST_BYTES + 1023) / 1024 * 1024;
-  static constexpr int DSS_OFF = ST_OFF + STAGES * ST_STRIDE;
-  static constexpr int BAR_OFF = DSS_OFF + 2 * CHUNK;
+  static constexpr int ST_QT = 0, ST_QS = NCH * CHUNK, ST_BYTES = 2 * NCH * CHUNK;
+  // The log-sum-exp rows have slots of their own, so that a stage is free when its products are done and not
+  // only when the elementwise warps have read it. Block it may take the slot of block it - 8 without a wait:
+  // its stage came free with the products of it - 2, which followed the reading of the scores of it - 4, so
+  // all elementwise warps are through with block it - 5.
+  static constexpr int ROWS = 8, ROW_OFF = ST_OFF + STAGES * ST_BYTES, ROW_BYTES = 2 * BQ * 4;
+  static constexpr int PREFETCH = 4;  // blocks ahead brought into L2
+  static constexpr int BAR_OFF = ROW_OFF + ROWS * ROW_BYTES;
   static constexpr int USED = BAR_OFF + 512;  // base alignment checked in the kernel
   static constexpr int SMEM = USED > 118 * 1024 ? USED : 118 * 1024;
   static_assert(USED <= 227 * 1024, "shared memory budget");
 };
 
 struct TpBars {
-  uint64_t kv_full, ld_full[2], ld_empty[2], s_full[2], s_free[2], dss_full, dss_free, drain;
+  uint64_t kv_full, ld_full[2], ld_empty[2], row_full[8], s_full[2], s_free[2], drain;
   uint32_t tmem_base;
   int abort;
   double red[DKDV_EW];
@@ -740,8 +737,7 @@ struct TpBars {
 template <int DH>
 __global__ void __launch_bounds__(TP_THREADS, 1)
     attn_teacher_p_tc_kernel(const __grid_constant__ CUtensorMap tm_s,
-                             const __grid_constant__ CUtensorMap tm_t,
-                             const __grid_constant__ CUtensorMap tm_ds, const TpParams p) {
+                             const __grid_constant__ CUtensorMap tm_t, const TpParams p) {
   using L = TpLayout<DH>;
   constexpr int BK = L::BK, BQ = L::BQ, STAGES = L::STAGES;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -775,18 +771,16 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
     tc::mbar_init(&bars->kv_full, 1);
     for (int i = 0; i < STAGES; ++i) {
       tc::mbar_init(&bars->ld_full[i], 1);
-      tc::mbar_init(&bars->ld_empty[i], 1 + DKDV_EW);  // the products and the lse readers
+      tc::mbar_init(&bars->ld_empty[i], 1);
       tc::mbar_init(&bars->s_full[i], 1);
       tc::mbar_init(&bars->s_free[i], DKDV_EW);
     }
-    tc::mbar_init(&bars->dss_full, DKDV_EW);
-    tc::mbar_init(&bars->dss_free, 1);
+    for (int i = 0; i < L::ROWS; ++i) tc::mbar_init(&bars->row_full[i], 1);
     tc::mbar_init(&bars->drain, 1);
     bars->abort = 0;
     tc::fence_mbar_init();
     tc::prefetch_tmap(&tm_s);
     tc::prefetch_tmap(&tm_t);
-    tc::prefetch_tmap(&tm_ds);
   }
   if (warp == 1) {
     tc::tmem_alloc(&bars->tmem_base, 512);
@@ -808,12 +802,22 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         tc::tma_load_2d(smem + L::KS_OFF + ch * L::CHUNK, &tm_s, &bars->kv_full,
                         p.kcol0 + g * DH + ch * 64, row0 + kb * BK);
       }
+      auto prefetch = [&](int j) {
+        const int hj = g * r + j / per_head, ij = kb + j % per_head;
+        for (int ch = 0; ch < L::NCH; ++ch) {
+          tc::tma_prefetch_2d(&tm_t, p.qcol0 + hj * DH + ch * 64, row0 + ij * BQ);
+          tc::tma_prefetch_2d(&tm_s, p.qcol0 + hj * DH + ch * 64, row0 + ij * BQ);
+        }
+      };
+      int rows_issued = 0;
+      for (int j = STAGES; j < L::PREFETCH && j < n_it; ++j) prefetch(j);
       for (int it = 0; it < n_it; ++it) {
         const int st = it % STAGES;
         const uint32_t ph = (it / STAGES) & 1;
         const int h = g * r + it / per_head, i = kb + it % per_head;
+        if (it + L::PREFETCH < n_it) prefetch(it + L::PREFETCH);
         if (!tc::mbar_wait(&bars->ld_empty[st], ph ^ 1, abort, p.status)) break;
-        uint8_t* sbase = smem + L::ST_OFF + st * L::ST_STRIDE;
+        uint8_t* sbase = smem + L::ST_OFF + st * L::ST_BYTES;
         tc::mbar_expect_tx(&bars->ld_full[st], L::ST_BYTES);
         for (int ch = 0; ch < L::NCH; ++ch) {
           tc::tma_load_2d(sbase + L::ST_QT + ch * L::CHUNK, &tm_t, &bars->ld_full[st],
@@ -822,10 +826,13 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
                           p.qcol0 + h * DH + ch * 64, row0 + i * BQ);
         }
         const int64_t lrow = ((int64_t)b * p.Hq + h) * p.lse_pitch + i * BQ;
+        uint8_t* rows = smem + L::ROW_OFF + (it % L::ROWS) * L::ROW_BYTES;
+        tc::mbar_expect_tx(&bars->row_full[it % L::ROWS], L::ROW_BYTES);
         if (in_bounds(lrow + BQ - 1, (int64_t)p.B * p.Hq * p.lse_pitch, p.status)) {
-          tc::bulk_load(sbase + L::ST_LT, p.lse2_t + lrow, BQ * 4, &bars->ld_full[st]);
-          tc::bulk_load(sbase + L::ST_LS, p.lse2_s + lrow, BQ * 4, &bars->ld_full[st]);
+          tc::bulk_load(rows, p.lse2_t + lrow, BQ * 4, &bars->row_full[it % L::ROWS]);
+          tc::bulk_load(rows + BQ * 4, p.lse2_s + lrow, BQ * 4, &bars->row_full[it % L::ROWS]);
         }
+        ++rows_issued;
         issued |= 1u << st;
         last_par = (last_par & ~(1u << st)) | (ph << st);
       }
@@ -833,6 +840,8 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         drain_wait(&bars->kv_full, 0);
         for (int st = 0; st < STAGES; ++st)
           if (issued & (1u << st)) drain_wait(&bars->ld_full[st], (last_par >> st) & 1);
+        for (int q = max(0, rows_issued - L::ROWS); q < rows_issued; ++q)
+          drain_wait(&bars->row_full[q % L::ROWS], (q / L::ROWS) & 1);
       }
     }
   } else if (warp == 1) {
@@ -848,7 +857,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
              (j < 2 || tc::mbar_wait(&bars->s_free[bf], ((j >> 1) - 1) & 1, abort, p.status));
         if (!ok) break;
         tc::fence_after_sync();
-        const uint32_t sb = tc::smem_u32(smem + L::ST_OFF + st * L::ST_STRIDE);
+        const uint32_t sb = tc::smem_u32(smem + L::ST_OFF + st * L::ST_BYTES);
         const uint64_t bt = tc::sdesc_kmajor_sw128(sb + L::ST_QT);
         const uint64_t bs = tc::sdesc_kmajor_sw128(sb + L::ST_QS);
 #pragma unroll
@@ -869,20 +878,6 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       tc::umma_commit(&bars->drain);
       drain_wait(&bars->drain, 0);
     }
-  } else if (warp == 2 + DKDV_EW) {
-    if (tc::elect_one()) {  // ------------------------------------------------- P^T tiles to global
-      for (int it = 0; it < n_it; ++it) {
-        if (!tc::mbar_wait(&bars->dss_full, it & 1, abort, p.status)) break;
-        const int h = g * r + it / per_head, i = kb + it % per_head;
-        const int64_t tile = ((int64_t)b * p.Hq + h) * p.npairs + (int64_t)i * (i + 1) / 2 + kb;
-        tc::tma_store_2d(&tm_ds, smem + L::DSS_OFF, 0, (int32_t)(tile * BK));
-        tc::tma_store_2d(&tm_ds, smem + L::DSS_OFF + L::CHUNK, 64, (int32_t)(tile * BK));
-        tc::bulk_commit_group();
-        tc::bulk_wait_group_read<0>();
-        tc::mbar_arrive(&bars->dss_free);
-      }
-      tc::bulk_wait_group<0>();
-    }
   } else {  // ------------------------------------ elementwise: 16 key rows x 64 queries per warp
     const int quarter = warp & 3;
     const int idx = (warp - 2) >> 2;
@@ -895,12 +890,11 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
     float2 acc = make_float2(0.f, 0.f);  // sum of P (s_t - s_s) in raw score units (times scale later)
     double rows = 0.0;                   // key-block-0 CTAs, warp 2: sum of lse2_s - lse2_t
     for (int it = 0; it < n_it; ++it) {
-      const int st = it % STAGES, bf = it & 1;
-      const int i = kb + it % per_head;
-      const float* sbase = reinterpret_cast<const float*>(smem + L::ST_OFF + st * L::ST_STRIDE);
-      const float* lt = sbase + L::ST_LT / 4;
-      const float* ls = sbase + L::ST_LS / 4;
-      if (!tc::mbar_wait(&bars->ld_full[st], (it / STAGES) & 1, abort, p.status) ||
+      const int bf = it & 1;
+      const int h = g * r + it / per_head, i = kb + it % per_head;
+      const float* lt = reinterpret_cast<const float*>(smem + L::ROW_OFF + (it % L::ROWS) * L::ROW_BYTES);
+      const float* ls = lt + BQ;
+      if (!tc::mbar_wait(&bars->row_full[it % L::ROWS], (it / L::ROWS) & 1, abort, p.status) ||
           !tc::mbar_wait(&bars->s_full[bf], (it >> 1) & 1, abort, p.status))
         break;
       tc::fence_after_sync();
@@ -949,21 +943,13 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         }
         rows += t;
       }
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&bars->ld_empty[st]);  // this warp has read the lse rows
-      if (it > 0 && !tc::mbar_wait(&bars->dss_free, (it - 1) & 1, abort, p.status)) break;
-      {
-        uint8_t* hb = smem + L::DSS_OFF + chalf * L::CHUNK;
+      const int64_t tile = ((int64_t)b * p.Hq + h) * p.npairs + (int64_t)i * (i + 1) / 2 + kb;
+      const int64_t w0 = pt_word(tile, warp - 2, lane);
+      if (in_bounds(w0 + 96, (int64_t)p.B * p.Hq * p.npairs * 2048, p.status)) {
 #pragma unroll
-        for (int n = 0; n < 8; ++n) {
-          *reinterpret_cast<uint32_t*>(hb + rA * 128 + ((n ^ (rA & 7)) << 4) + cq * 4) = pw[2 * n];
-          *reinterpret_cast<uint32_t*>(hb + (rA + 8) * 128 + ((n ^ ((rA + 8) & 7)) << 4) + cq * 4) =
-              pw[2 * n + 1];
-        }
+        for (int q = 0; q < 4; ++q)
+          __stcg(p.pt + w0 + 32 * q, make_uint4(pw[4 * q], pw[4 * q + 1], pw[4 * q + 2], pw[4 * q + 3]));
       }
-      tc::fence_proxy_async_smem();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&bars->dss_full);
     }
     // The CTA's partial: the warps' sums in a fixed order (natural units).
     float v = acc.x + acc.y;
@@ -1273,6 +1259,7 @@ cudaError_t launch_attn_bwd_tc(const AttnLaunch& L, const float* cos_t, const fl
   p.sl2 = L.scale * kLog2e;
   p.a_mse = kl_ab ? kl_ab[0] : 1.f;
   p.b_kl = kl_ab ? kl_ab[1] : 0.f;
+  p.pt = static_cast<const uint4*>(L.ds);
   p.lse = L.lse;
   p.dvec = L.dvec;
   p.cos_t = cos_t;
@@ -1289,14 +1276,13 @@ cudaError_t launch_attn_bwd_tc(const AttnLaunch& L, const float* cos_t, const fl
 
 namespace {
 template <int DH>
-cudaError_t launch_tp(const CUtensorMap& ms, const CUtensorMap& mt, const CUtensorMap& md,
-                      const TpParams& p, cudaStream_t st) {
+cudaError_t launch_tp(const CUtensorMap& ms, const CUtensorMap& mt, const TpParams& p, cudaStream_t st) {
   static bool attr = false;
   cudaError_t e = set_smem(attn_teacher_p_tc_kernel<DH>, TpLayout<DH>::SMEM, attr);
   if (e != cudaSuccess) return e;
   const int64_t n = (int64_t)p.Hkv * p.B * ((p.T + 127) / 128);
   if (n >= (1ll << 31)) return cudaErrorInvalidValue;
-  return launch_after(attn_teacher_p_tc_kernel<DH>, (unsigned)n, TP_THREADS, TpLayout<DH>::SMEM, st, ms, mt, md, p);
+  return launch_after(attn_teacher_p_tc_kernel<DH>, (unsigned)n, TP_THREADS, TpLayout<DH>::SMEM, st, ms, mt, p);
 }
 }  // namespace
 
@@ -1320,6 +1306,7 @@ cudaError_t launch_attn_teacher_p_tc(const void* qkv_s, int64_t ldq_s, const voi
   p.sl2 = scale * kLog2e;
   p.lse2_t = lse2_t;
   p.lse2_s = lse2_s;
+  p.pt = static_cast<uint4*>(ds);
   p.part = part;
   p.status = status;
   if ((reinterpret_cast<uintptr_t>(lse2_t) & 15u) || (reinterpret_cast<uintptr_t>(lse2_s) & 15u) ||
@@ -1327,11 +1314,11 @@ cudaError_t launch_attn_teacher_p_tc(const void* qkv_s, int64_t ldq_s, const voi
       part == nullptr || (dh != 64 && dh != 128))
     return cudaErrorInvalidValue;
   const uint64_t ds_rows = (uint64_t)B * Hq * p.npairs * 128;
-  CUtensorMap ms, mt, md;
+  CUtensorMap ms, mt;
   if (!tmap_rows(&ms, qkv_s, ldq_s, N, 128) || !tmap_rows(&mt, qkv_t, ldq_t, N, 128) ||
-      !tmap_rows(&md, ds, 128, ds_rows, 128) || ds_rows >= (1ull << 31))
+      ds_rows >= (1ull << 31))
     return cudaErrorInvalidValue;
-  return dh == 128 ? launch_tp<128>(ms, mt, md, p, st) : launch_tp<64>(ms, mt, md, p, st);
+  return dh == 128 ? launch_tp<128>(ms, mt, p, st) : launch_tp<64>(ms, mt, p, st);
 }
 
 }  // namespace jab
