@@ -7,10 +7,11 @@
 // a pair computes a 256 x 256 tile with M256 N256 K16 UMMAs issued by its even CTA; each CTA holds
 // 128 rows of A, half of the B tile and 128 lanes of the accumulator (details above the kernel).
 //   warp 0      TMA producer: the CTA's 128x64 A tile and 128x64 half of B per stage, 6-stage ring
-//   warp 1      TMEM owner (512 columns, allocated by the pair) and, in the even CTA, UMMA issuer
+//   warp 1      TMEM owner (two accumulators, allocated by the pair) and, in the even CTA, UMMA issuer
 //   warps 2..5  epilogue: tcgen05.ld of the CTA's 128 x 256 fp32 accumulator, one lane per thread;
 //               the projection's fp16 results leave by TMA through two boxes per warp
 // Two accumulators (2 x 256 TMEM columns) let the epilogue of one tile overlap the next mainloop.
+// With few tiles a pair takes 256 x 128 of C instead (tile_cols).
 //
 // Epilogues:
 //   projection  [Q|K|V] = X w_hat^T: rotate-half RoPE on the Q and K heads (partner column +-d_h/2
@@ -30,10 +31,9 @@
 namespace jab {
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64;  // BM: rows of one CTA (an epilogue's 128 TMEM lanes)
+constexpr int BM = 128, BK = 64;  // BM: rows of one CTA (an epilogue's 128 TMEM lanes); BN: 256 or 128 (tile_cols)
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int NUM_THREADS = 192;
-constexpr uint32_t TMEM_COLS = 2 * BN;
 
 enum EpiKind { kEpiRope = 0, kEpiLsq = 1, kEpiStore = 2 };
 
@@ -88,6 +88,7 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
 // blocks) that took 11.5k clocks a tile where the products take 6.1k (65536 x 9216: 735 us, now 526). The
 // warp's 32 rows x 64 columns go through a swizzled box in shared memory and leave by TMA (rows past M
 // are clipped by the tensor map). buf: the warp's two boxes.
+template <int BN>
 __device__ __forceinline__ void epi_rope(const GemmParams& p, const CUtensorMap* tmC, uint32_t taddr,
                                          int mb, int nb, int row, uint8_t* buf) {
   const int lane = row & 31;
@@ -187,6 +188,7 @@ __device__ __forceinline__ void epi_rope(const GemmParams& p, const CUtensorMap*
 // STE weight gradient (App. B: d w_hat / d w = 1, so dL/dW = dL/dw_hat = coef * dQKV^T X): the
 // tile times coef stored as fp32 rows of dw (with a split K each unit's partial tile is added with
 // vector atomics). Packed FP32 pairs, as this runs beside the next tile's UMMAs.
+template <int BN>
 __device__ __forceinline__ void epi_store(const GemmParams& p, uint32_t taddr, int mb, int nb,
                                           int row) {
   const int64_t o = (int64_t)mb * BM + row;  // M = D is a multiple of 128: every row is valid
@@ -273,6 +275,7 @@ __device__ __forceinline__ float lsq_chunk(const uint32_t (&g)[32], const uint4 
   return acc.x + acc.y;
 }
 
+template <int BN>
 __device__ __forceinline__ void epi_lsq(const GemmParams& p, uint32_t taddr, int mb, int nb,
                                         int ks, int row) {
   const int o = mb * BM + row;  // M = D is a multiple of 128: every row is valid
@@ -340,28 +343,31 @@ __device__ __forceinline__ void epi_lsq(const GemmParams& p, uint32_t taddr, int
 //               the even CTA's barrier
 constexpr int STAGES2 = 6;
 constexpr int BM2 = 2 * BM;                 // rows of A per pair tile
-constexpr int B2_ROWS = BN / 2;             // rows (K-major) or columns (MN-major) of B per CTA
-constexpr int B2_BYTES = B2_ROWS * BK * 2;  // 16 KB
-constexpr int STAGE2_BYTES = A_BYTES + B2_BYTES;
+template <int BN>
+constexpr int B2_ROWS = BN / 2;  // rows (K-major) or columns (MN-major) of B per CTA
+template <int BN>
+constexpr int STAGE2_BYTES = A_BYTES + B2_ROWS<BN> * BK * 2;
 constexpr int EPI2_BYTES = 4 * 2 * 4096;  // two output boxes per epilogue warp
-constexpr int SMEM2_BYTES = STAGES2 * STAGE2_BYTES + EPI2_BYTES + 1024 + 256;
+template <int BN>
+constexpr int SMEM2_BYTES = STAGES2 * STAGE2_BYTES<BN> + EPI2_BYTES + 1024 + 256;
 
 struct Bars2 {
   uint64_t full[STAGES2], empty[STAGES2], tfull[2], tempty[2], drain;
   uint32_t tmem_base;
   int abort;
 };
-static_assert(STAGES2 * STAGE2_BYTES + EPI2_BYTES + (int)sizeof(Bars2) <= SMEM2_BYTES - 1024, "shared memory");
-static_assert(SMEM2_BYTES <= 227 * 1024, "shared memory budget");
+static_assert(sizeof(Bars2) <= 256, "barrier block");
+static_assert(SMEM2_BYTES<256> <= 227 * 1024, "shared memory budget");
 
-template <int EPI, bool BF16, bool B_MN>
+template <int EPI, bool BF16, bool B_MN, int BN>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     gemm2_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmC, const GemmParams p) {
+  constexpr int SB = STAGE2_BYTES<BN>, BR = B2_ROWS<BN>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
-  Bars2* bars = reinterpret_cast<Bars2*>(smem + STAGES2 * STAGE2_BYTES + EPI2_BYTES);
+  Bars2* bars = reinterpret_cast<Bars2*>(smem + STAGES2 * SB + EPI2_BYTES);
   const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = tc::cluster_ctarank();  // 0: issues the pair's UMMAs
   const bool leader = rank == 0;
@@ -386,7 +392,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     if (EPI == kEpiRope) tc::prefetch_tmap(&tmC);
   }
   if (warp == 1) {
-    tc::tmem_alloc2(&bars->tmem_base, TMEM_COLS);
+    tc::tmem_alloc2(&bars->tmem_base, 2 * BN);
     tc::tmem_relinquish2();
   }
   tc::fence_before_sync();
@@ -410,16 +416,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         k_range(p, ks, kb0, kb1);
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!tc::mbar_wait(&bars->empty[stage], phase ^ 1, abort, p.status)) break;
-          uint8_t* sa = smem + stage * STAGE2_BYTES;
+          uint8_t* sa = smem + stage * SB;
           const uint32_t bar = full_lead + stage * 8;
-          if (leader) tc::mbar_expect_tx(&bars->full[stage], 2 * STAGE2_BYTES);
+          if (leader) tc::mbar_expect_tx(&bars->full[stage], 2 * SB);
           tc::tma_load_2d_pair(sa, &tmA, bar, kb * BK, mb * BM2 + (int)rank * BM);
           if (B_MN)  // B stored [k][n]: this CTA's two boxes of BK rows x 64 columns
-            for (int c = 0; c < B2_ROWS / 64; ++c)
+            for (int c = 0; c < BR / 64; ++c)
               tc::tma_load_2d_pair(sa + A_BYTES + c * (BK * 128), &tmB, bar,
-                                   nb * BN + (int)rank * B2_ROWS + c * 64, kb * BK);
+                                   nb * BN + (int)rank * BR + c * 64, kb * BK);
           else
-            tc::tma_load_2d_pair(sa + A_BYTES, &tmB, bar, kb * BK, nb * BN + (int)rank * B2_ROWS);
+            tc::tma_load_2d_pair(sa + A_BYTES, &tmB, bar, kb * BK, nb * BN + (int)rank * BR);
           issued |= 1u << stage;
           last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
           if (++stage == STAGES2) {
@@ -453,7 +459,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             break;
           }
           tc::fence_after_sync();
-          const uint32_t a0 = tc::smem_u32(smem + stage * STAGE2_BYTES);
+          const uint32_t a0 = tc::smem_u32(smem + stage * SB);
           const uint32_t b0 = a0 + A_BYTES;
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
@@ -487,13 +493,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + acc * BN;
       const int mb128 = 2 * mb + (int)rank;  // this CTA's 128-row block
       if (EPI == kEpiRope)
-        epi_rope(p, &tmC, taddr, mb128, nb, row,  // rows past M are masked there
-                 smem + STAGES2 * STAGE2_BYTES + q * 8192);
+        epi_rope<BN>(p, &tmC, taddr, mb128, nb, row,  // rows past M are masked there
+                 smem + STAGES2 * SB + q * 8192);
       else if ((int64_t)mb128 * BM < p.M) {  // M is a multiple of 128: whole halves are valid or not
         if (EPI == kEpiLsq)
-          epi_lsq(p, taddr, mb128, nb, ks, row);
+          epi_lsq<BN>(p, taddr, mb128, nb, ks, row);
         else
-          epi_store(p, taddr, mb128, nb, row);
+          epi_store<BN>(p, taddr, mb128, nb, row);
       }
       tc::fence_before_sync();
       __syncwarp();
@@ -514,7 +520,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   tc::fence_after_sync();
   if (warp == 1) {
     __syncwarp();
-    tc::tmem_dealloc2(tmem, TMEM_COLS);
+    tc::tmem_dealloc2(tmem, 2 * BN);
   }
 }
 
@@ -556,15 +562,27 @@ int sm_count() {
   return n > 0 ? n : 1;
 }
 
+// Columns of a pair's tile. 256 is the better tile (a 128 one reads A and B from shared memory as often for
+// half the products), but with few tiles a narrow one puts twice as many SMs to work, each with half the
+// products and half the epilogue: taken when its rounds over the pairs, each reckoned 15 % dearer than half a
+// round of wide tiles, take less. GPT-2 block, fitting step 4 x 128 (18 and 27 wide tiles on 76 pairs):
+// 45.3 -> 40.3 us; a teacher pass of 16 x 1024 (576 wide tiles, 8 rounds against 16) keeps the wide tile.
+int tile_cols(int num_m, int n, int splits) {
+  const int64_t pairs = std::max(sm_count() / 2, 1), u = (int64_t)num_m * splits;
+  const int64_t wide = (u * ((n + 255) / 256) + pairs - 1) / pairs, narrow = (u * ((n + 127) / 128) + pairs - 1) / pairs;
+  return 0.575 * (double)narrow < (double)wide ? 128 : 256;
+}
+
 // CTA-pair launch: clusters of two, one pair per two SMs (as many pairs as fit at once).
-template <int EPI, bool BF16, bool B_MN>
+template <int EPI, bool BF16, bool B_MN, int BN>
 cudaError_t launch_gemm2(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tcm,
                          GemmParams& p, cudaStream_t st) {
-  auto kern = gemm2_tc_kernel<EPI, BF16, B_MN>;
+  auto kern = gemm2_tc_kernel<EPI, BF16, B_MN, BN>;
+  p.num_n = (p.Nn + BN - 1) / BN;
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES<BN>);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
@@ -577,7 +595,7 @@ cudaError_t launch_gemm2(const CUtensorMap& ta, const CUtensorMap& tb, const CUt
   cfg.attrs = at;
   cfg.numAttrs = 1;
   cfg.blockDim = dim3(NUM_THREADS);
-  cfg.dynamicSmemBytes = SMEM2_BYTES;
+  cfg.dynamicSmemBytes = SMEM2_BYTES<BN>;
   cfg.stream = st;
   const int sms = sm_count();
   // The pairs that fit at once depend only on the kernel and the device: asked once, so that a
@@ -603,7 +621,8 @@ cudaError_t launch_proj_gemm_tc(const void* A, const void* Bw, void* C, int64_t 
                                 int D, int n_rot, int dh, int T, const float* cos_t,
                                 const float* sin_t, int* status, cudaStream_t st) {
   CUtensorMap ta, tb, tcm;
-  if (!make_tmap(&ta, A, false, K, M, K, BM) || !make_tmap(&tb, Bw, false, K, Nn, K, B2_ROWS) ||
+  const int bn = tile_cols((int)((M + BM2 - 1) / BM2), Nn, 1);
+  if (!make_tmap(&ta, A, false, K, M, K, BM) || !make_tmap(&tb, Bw, false, K, Nn, K, bn / 2) ||
       !make_tmap(&tcm, C, false, Nn, M, Nn, 32))
     return cudaErrorInvalidValue;
   GemmParams p{};
@@ -611,7 +630,6 @@ cudaError_t launch_proj_gemm_tc(const void* A, const void* Bw, void* C, int64_t 
   p.Nn = Nn;
   p.K = K;
   p.num_m = (int)((M + BM2 - 1) / BM2);  // 256-row blocks: CTA pairs
-  p.num_n = (Nn + BN - 1) / BN;
   p.splits = 1;
   p.k_blocks = K / BK;
   p.group_m = 16;  // 16 pair rows = 4096 rows of X and all of W in L2 while the N tiles pass
@@ -622,7 +640,8 @@ cudaError_t launch_proj_gemm_tc(const void* A, const void* Bw, void* C, int64_t 
   p.T = T;
   p.cos_t = cos_t;
   p.sin_t = sin_t;
-  return launch_gemm2<kEpiRope, false, false>(ta, tb, tcm, p, st);
+  return bn == 128 ? launch_gemm2<kEpiRope, false, false, 128>(ta, tb, tcm, p, st)
+                   : launch_gemm2<kEpiRope, false, false, 256>(ta, tb, tcm, p, st);
 }
 
 // Split K so that the units (tile x K range) fill whole waves of the persistent grid: the makespan
@@ -655,9 +674,8 @@ cudaError_t launch_wgrad_lsq_tc(const void* dqkvt, int64_t ldt, const void* x, c
   p.Nn = d;
   p.K = (int)std::min<int64_t>(N, INT32_MAX);
   p.num_m = (D + BM2 - 1) / BM2;  // 256-row blocks: CTA pairs
-  p.num_n = (d + BN - 1) / BN;
   p.k_blocks = (int)((N + BK - 1) / BK);
-  p.splits = choose_splits(p.num_m * p.num_n, p.k_blocks, sm_count() / 2);
+  p.splits = choose_splits(p.num_m * ((d + 255) / 256), p.k_blocks, sm_count() / 2);
   p.group_m = 8;
   p.status = status;
   p.w = static_cast<const bf16_t*>(w);
@@ -670,7 +688,9 @@ cudaError_t launch_wgrad_lsq_tc(const void* dqkvt, int64_t ldt, const void* x, c
   // every (split, row, group) partial is written once; the splits are summed in order by the caller's
   // last launch: the scale gradient is bit-identical between calls
   *splits = p.splits;
-  return launch_gemm2<kEpiLsq, true, true>(ta, tb, ta, p, st);
+  // a tile covers whole groups: the narrow one only those that divide it
+  return 128 % G == 0 && tile_cols(p.num_m, d, p.splits) == 128 ? launch_gemm2<kEpiLsq, true, true, 128>(ta, tb, ta, p, st)
+                                                                : launch_gemm2<kEpiLsq, true, true, 256>(ta, tb, ta, p, st);
 }
 
 cudaError_t launch_wgrad_store_tc(const void* dqkvt, int64_t ldt, const void* x, int64_t N, int D,
@@ -684,7 +704,6 @@ cudaError_t launch_wgrad_store_tc(const void* dqkvt, int64_t ldt, const void* x,
   p.Nn = d;
   p.K = (int)std::min<int64_t>(N, INT32_MAX);
   p.num_m = (D + BM2 - 1) / BM2;  // 256-row blocks: CTA pairs
-  p.num_n = (d + BN - 1) / BN;
   p.k_blocks = (int)((N + BK - 1) / BK);
   p.group_m = 8;
   p.status = status;
@@ -694,14 +713,15 @@ cudaError_t launch_wgrad_store_tc(const void* dqkvt, int64_t ldt, const void* x,
   // the deterministic mode keeps one unit per tile.
   const int64_t n_w = (int64_t)D * d;
   float* target = dw != nullptr ? dw : scratch;
-  p.splits = deterministic ? 1 : choose_splits(p.num_m * p.num_n, p.k_blocks, sm_count() / 2);
+  p.splits = deterministic ? 1 : choose_splits(p.num_m * ((d + 255) / 256), p.k_blocks, sm_count() / 2);
   p.dw = target;
   cudaError_t e;
   if (p.splits > 1) {
     e = cudaMemsetAsync(target, 0, (size_t)n_w * sizeof(float), st);
     if (e != cudaSuccess) return e;
   }
-  e = launch_gemm2<kEpiStore, true, true>(ta, tb, ta, p, st);
+  e = tile_cols(p.num_m, d, p.splits) == 128 ? launch_gemm2<kEpiStore, true, true, 128>(ta, tb, ta, p, st)
+                                             : launch_gemm2<kEpiStore, true, true, 256>(ta, tb, ta, p, st);
   if (e != cudaSuccess) return e;
   // a dW that the caller gets is checked, in the pass over it for its norm where there is one
   if (sqnorm != nullptr) return launch_sumsq(target, n_w, red, sqnorm, dw != nullptr ? status : nullptr, st);

@@ -170,3 +170,35 @@ def test_weight_gradient_norm_and_loss_parts_of_odd_batches(B, T):
     J().jab_loss_forward(c.desc, B, T, c.X, c.W, A, [2], [s], loss, ws, sse_parts=parts)
     np.testing.assert_allclose(loss.item(), parts.sum().item() / (B * T * 4 * 64), rtol=1e-13)
     assert J().jab_get_device_status() == 0
+
+
+@pytest.mark.parametrize("shape,B,T", [(BlockShape(768, 12, 12, 64, False), 1, 70),
+                                       (BlockShape(768, 12, 12, 64, False), 1, 1337),
+                                       (BlockShape(512, 4, 2, 128, True, 1e4), 3, 43),
+                                       (BlockShape(512, 20, 2, 128, True, 1e4), 4, 301),
+                                       (BlockShape(256, 4, 1, 64, True, 500.0), 2, 65)])
+def test_projection_with_narrow_and_wide_tiles(shape, B, T):
+    """[Q | K | V] with RoPE from 128- and 256-column tiles (few tiles, or most of a round of CTA pairs),
+    ragged in rows and in the last column tile. Against float64 on the fp16 operands: half an ulp of the
+    fp16 result, and for the fp32 sums of K products K 2^-24 of the sum of their magnitudes, of both
+    halves of a rotated pair."""
+    from dataclasses import replace
+    from tests.harness import Case
+    from workloads import WORKLOADS
+    c = Case(replace(WORKLOADS["gpt2_smoke"], shape=shape), B, T, 64)
+    out = torch.empty((B, T, c.D), dtype=torch.float16, device="cuda")
+    J().jab_reference_projection(c.desc, B, T, c.X, c.W, out, c.workspace())
+    assert J().jab_get_device_status() == 0
+    x, w = np64(c.X.half()), np64(c.W.half())
+    ref, mag = x @ w.T, np.abs(x) @ np.abs(w).T
+    if shape.use_rope:
+        cos, sin = O.rope_tables(T, c.dh, shape.rope_theta)
+        nr = (c.Hq + shape.n_kv_heads) * c.dh
+        rot = ref[..., :nr].reshape(B, T, -1, c.dh)
+        ref[..., :nr] = O.apply_rope(rot, cos, sin).reshape(B, T, nr)
+        m = mag[..., :nr].reshape(B, T, -1, 2, c.dh // 2).sum(3, keepdims=True)
+        mag[..., :nr] = np.broadcast_to(m, (B, T, m.shape[2], 2, c.dh // 2)).reshape(B, T, nr)
+    # (the rotation's own roundings and the tables': four more of 2^-24)
+    bound = 2.0 ** -11 * np.abs(ref) + (shape.d_model + 4) * 2.0 ** -24 * mag + 2.0 ** -25
+    err = np.abs(np64(out) - ref)
+    assert (err <= bound).all(), (err / bound).max()
