@@ -202,3 +202,38 @@ def test_projection_with_narrow_and_wide_tiles(shape, B, T):
     bound = 2.0 ** -11 * np.abs(ref) + (shape.d_model + 4) * 2.0 ** -24 * mag + 2.0 ** -25
     err = np.abs(np64(out) - ref)
     assert (err <= bound).all(), (err / bound).max()
+
+
+@pytest.mark.parametrize("shape", [BlockShape(256, 4, 1, 64, True, 500.0), BlockShape(512, 4, 2, 128, True, 1e4)])
+@pytest.mark.parametrize("T", [128, 333])
+def test_persistent_maps_equal_single_sequences(shape, T):
+    """KL maps and Hessian products of a batch with several tiles per persistent CTA (and, in the longer
+    one, of several lengths): every KL row has the bits of a call with that sequence alone, and the
+    probes' v^T H v, sums of per-sequence values over n, agree to the fp64 sums' 2^-52 a term."""
+    from dataclasses import replace
+    from tests.harness import Case
+    from workloads import WORKLOADS
+    B, bits = 96, [2, 4]
+    c = Case(replace(WORKLOADS["gpt2_smoke"], shape=shape), B, T, 64)
+
+    def run(X):
+        n = X.shape[0]
+        ws = J().Workspace(c.desc, n, T, 2, True)
+        A = torch.empty((n, T, c.Hq * c.dh), dtype=torch.float32, device="cuda")
+        lse = torch.empty((n, c.Hq, T), dtype=torch.float32, device="cuda")
+        qkv = torch.empty((n, T, c.D), dtype=torch.float16, device="cuda")
+        rows = torch.empty((2, n, c.Hq, T), dtype=torch.float32, device="cuda")
+        loss, kl = (torch.empty(2, dtype=torch.float64, device="cuda") for _ in range(2))
+        vhv, trace = (torch.empty(k, dtype=torch.float64, device="cuda") for k in (2, 1))
+        J().jab_reference_forward(c.desc, n, T, X, c.W, A, ws, lse=lse)
+        J().jab_reference_projection(c.desc, n, T, X, c.W, qkv, ws)
+        J().jab_loss_forward_kl(c.desc, n, T, X, c.W, A, qkv, bits, [c.gpu_scales(b) for b in bits], 0.1,
+                                loss, ws, kl=kl, kl_rows=rows)
+        J().jab_hutchinson_trace(c.desc, n, T, X, c.W, A, lse, 2, 7, trace, ws, vhv=vhv)
+        assert J().jab_get_device_status() == 0
+        return rows, vhv
+
+    rows, vhv = run(c.X)
+    ones = [run(c.X[b:b + 1].contiguous()) for b in range(B)]
+    assert torch.equal(rows, torch.cat([r for r, _ in ones], 1))
+    np.testing.assert_allclose(vhv.cpu(), torch.stack([v for _, v in ones]).mean(0).cpu(), rtol=1e-12)
