@@ -160,14 +160,26 @@ __device__ __forceinline__ RowState merge(const RowState& x, const RowState& y) 
   r.ls = x.ls * gx + y.ls * gy;
   return r;
 }
-__device__ __forceinline__ RowState merge_lanes(const RowState& r, int o) {
-  RowState y;
-  y.mt = __shfl_xor_sync(0xffffffffu, r.mt, o);
-  y.ms = __shfl_xor_sync(0xffffffffu, r.ms, o);
-  y.lt = __shfl_xor_sync(0xffffffffu, r.lt, o);
-  y.ls = __shfl_xor_sync(0xffffffffu, r.ls, o);
-  y.a = __shfl_xor_sync(0xffffffffu, r.a, o);
-  return merge(r, y);
+// The state over the keys of the four lanes of a row, in all of them: the maxima first, then one rescaling.
+__device__ __forceinline__ void merge_lanes(RowState& r) {
+  float mt = r.mt, ms = r.ms;
+#pragma unroll
+  for (int o = 1; o <= 2; o <<= 1) {
+    mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+    ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
+  }
+  const float ft = exp2_int(r.mt - mt), fs = exp2_int(r.ms - ms);
+  r.mt = mt;
+  r.ms = ms;
+  r.lt *= ft;
+  r.a *= ft;
+  r.ls *= fs;
+#pragma unroll
+  for (int o = 1; o <= 2; o <<= 1) {
+    r.lt += __shfl_xor_sync(0xffffffffu, r.lt, o);
+    r.a += __shfl_xor_sync(0xffffffffu, r.a, o);
+    r.ls += __shfl_xor_sync(0xffffffffu, r.ls, o);
+  }
 }
 
 template <int DH>
@@ -311,7 +323,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     for (int it = 0, k = sched_tile(0, grid, cta); ok && k < p.ntiles; k = sched_tile(++it, grid, cta)) {
       const KlTile tl = kl_tile(p, k);
       const int q0 = tl.qb * BQ, nkb = tl.qb + 1;
-      const int tA = q0 + rA, tB = q0 + rB;
       RowState ra{kNoKey, kNoKey, 0.f, 0.f, 0.f}, rb = ra;
       for (int j = 0; j < nkb; ++j, ++g) {
         if (!tc::mbar_wait(&bars->s_full, g & 1, abort, p.status)) {
@@ -396,39 +407,32 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       // The four lanes of a row, then its two key halves: the upper one leaves its state in shared memory. (A
       // buffer of this parity was last read two tiles ago, before its reader released the last tile's scores;
       // a single barrier would not do, as the upper half may be one tile ahead.)
-#pragma unroll
-      for (int o = 1; o <= 2; o <<= 1) {
-        ra = merge_lanes(ra, o);
-        rb = merge_lanes(rb, o);
-      }
+      merge_lanes(ra);
+      merge_lanes(rb);
+      // Lane 0 of a row's four goes on with row A, lane 1 with row B.
+      RowState r = cq & 1 ? rb : ra;
+      const int row = cq & 1 ? rB : rA;
       RowState* upper = bars->upper[it & 1];
       if (khalf == 1) {
-        if (cq == 0) {
-          upper[rA] = ra;
-          upper[rB] = rb;
-        }
+        if (cq < 2) upper[row] = r;
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&bars->half_full[it & 1][grp]);
         continue;
       }
       ok = tc::mbar_wait(&bars->half_full[it & 1][grp], (it >> 1) & 1, abort, p.status);
       if (!ok) break;
-      ra = merge(ra, upper[rA]);
-      rb = merge(rb, upper[rB]);
+      r = merge(r, upper[row]);
       float sum = 0.f, sum_lo = 0.f;  // this row group's KL and the rounding of its additions
-      const float klA = kLn2 * (p.sl2 * __fdiv_rn(ra.a, ra.lt) + (ra.ms - ra.mt) + log2f(__fdiv_rn(ra.ls, ra.lt)));
-      const float klB = kLn2 * (p.sl2 * __fdiv_rn(rb.a, rb.lt) + (rb.ms - rb.mt) + log2f(__fdiv_rn(rb.ls, rb.lt)));
-      if (cq == 0) {
-        const int64_t rbase = (((int64_t)tl.c * p.B + tl.b) * p.Hq + tl.h) * p.T;
-        const int64_t ext_r = (int64_t)p.C * p.B * p.Hq * p.T;
-        if (tA < p.T) {
-          sum = klA;
-          if (p.kl_rows && in_bounds(rbase + tA, ext_r, p.status)) p.kl_rows[rbase + tA] = klA;
-        }
-        if (tB < p.T) {
-          two_sum(sum, klB, sum, sum_lo);
-          if (p.kl_rows && in_bounds(rbase + tB, ext_r, p.status)) p.kl_rows[rbase + tB] = klB;
-        }
+      const float kl = kLn2 * (p.sl2 * __fdiv_rn(r.a, r.lt) + (r.ms - r.mt) + log2f(__fdiv_rn(r.ls, r.lt)));
+      const int t = q0 + row;
+      if (cq < 2 && t < p.T) {
+        sum = kl;
+        const int64_t at = (((int64_t)tl.c * p.B + tl.b) * p.Hq + tl.h) * p.T + t;
+        if (p.kl_rows && in_bounds(at, (int64_t)p.C * p.B * p.Hq * p.T, p.status)) p.kl_rows[at] = kl;
+      }
+      {  // rows A and B, then the eight pairs of them
+        const float other = __shfl_xor_sync(0xffffffffu, sum, 1);
+        two_sum(sum, other, sum, sum_lo);
       }
 #pragma unroll
       for (int o = 4; o <= 16; o <<= 1) {
