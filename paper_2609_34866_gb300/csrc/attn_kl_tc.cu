@@ -23,9 +23,11 @@
 //   warp 0       TMA: Q^S and Q^T of a tile, then K^S_j and K^T_j (ring)
 //   warp 1       TMEM owner, tcgen05.cp of Q^S / Q^T, UMMA issuer (one thread)
 //   warps 2..17  elementwise, 16 rows x 64 keys each (16x256b TMEM shape)
+//   warp 18      row results of the tile before, from the states of its two key halves in shared memory
 // Bound by the exponentials, 2 x 128 x 128 a block at 32 a clock and SM = 1024 clocks, next to 896 of packed
-// fp32 work and 512 (d_h 64) of products; 16 x 12 heads of 777 x 64 with four candidates take 181 us, about
-// 2400 clocks a block, where one CTA a tile with eight elementwise warps took 227.
+// fp32 work and 512 (d_h 64) of products; 16 x 12 heads of 777 x 64 with four candidates take 136 us, about
+// 1800 clocks a block and 2500 a tile (one CTA a tile with eight elementwise warps: 227 us; with the rows'
+// results in those warps, 4000 clocks more a tile: 173 us).
 // Outputs: per-row KL (optional) and one fp64 partial per tile, summed in fixed order afterwards.
 #include <cudaTypedefs.h>
 
@@ -39,7 +41,7 @@ namespace {
 
 constexpr int BQ = 128, BK = 128;
 constexpr int EW_WARPS = 16;
-constexpr int NUM_THREADS = (2 + EW_WARPS) * 32;  // warp 0 TMA, warp 1 UMMA, warps 2..17 elementwise
+constexpr int NUM_THREADS = (2 + EW_WARPS + 1) * 32;  // warp 0 TMA, warp 1 UMMA, warps 2..17 elementwise, 18 rows
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleLog2 = 8.f;
@@ -53,7 +55,7 @@ struct KlLayout {
   static constexpr int K_OFF = 2 * TILE;     // stage st: K^S at K_OFF + 2 st TILE, K^T after it
   static constexpr int STAGES = DH == 64 ? 4 : 2;
   static constexpr int BAR_OFF = K_OFF + STAGES * 2 * TILE;
-  static constexpr int USED = BAR_OFF + 8192;  // base alignment checked in the kernel
+  static constexpr int USED = BAR_OFF + 12288;  // base alignment checked in the kernel
   static constexpr int SMEM = USED > 118 * 1024 ? USED : 118 * 1024;
   // tile parity t: Q^S at Q_COL + t DH, Q^T DH / 2 after it
   static constexpr uint32_t SS_COL = 0, ST_COL = 128, Q_COL = 256;
@@ -67,13 +69,12 @@ struct RowState {
 };
 
 struct KlBars {
-  uint64_t q_full, stg_free, k_full[4], k_empty[4], s_full, s_empty, half_full[2][8], drain;
+  uint64_t q_full, stg_free, k_full[4], k_empty[4], s_full, s_empty, st_full[2], st_free[2], drain;
   uint32_t tmem_base;
-  int abort, done[2];         // [tile parity]: row groups whose sum is in red
-  float2 red[2][8];           // [tile parity][16-row group]: sum of KL_i, high and low part
-  RowState upper[2][128];     // [tile parity][row]: state of the upper key half
+  int abort;
+  RowState state[2][2][128];  // [tile parity][key half][row]
 };
-static_assert(sizeof(KlBars) <= 8192, "barrier block");
+static_assert(sizeof(KlBars) <= 12288, "barrier block");
 
 struct KlParams {
   int T, B, C, Hq, Hkv, D, nqb, nP, ntiles, balanced;
@@ -206,9 +207,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
     tc::mbar_init(&bars->s_full, 1);
     tc::mbar_init(&bars->s_empty, EW_WARPS);
-    for (int i = 0; i < 16; ++i) tc::mbar_init(&bars->half_full[i >> 3][i & 7], 1);
+    for (int i = 0; i < 2; ++i) {
+      tc::mbar_init(&bars->st_full[i], EW_WARPS);
+      tc::mbar_init(&bars->st_free[i], 1);
+    }
     tc::mbar_init(&bars->drain, 1);
-    bars->abort = bars->done[0] = bars->done[1] = 0;
+    bars->abort = 0;
     tc::fence_mbar_init();
     tc::prefetch_tmap(&tm_s);
     tc::prefetch_tmap(&tm_t);
@@ -307,7 +311,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       tc::umma_commit(&bars->drain);
       drain_wait(&bars->drain, 0);
     }
-  } else {  // -------------------------------------------------------------------- elementwise
+  } else if (warp < 2 + EW_WARPS) {  // -------------------------------------------- elementwise
     // Warp w (2..17) may access TMEM lane quarter w % 4; the four warps of a quarter take its two 16-row
     // groups x the block's two 64-key halves.
     const int quarter = warp & 3;
@@ -404,57 +408,44 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         rb.a += aB.x + aB.y;
       }
       if (!ok) break;
-      // The four lanes of a row, then its two key halves: the upper one leaves its state in shared memory. (A
-      // buffer of this parity was last read two tiles ago, before its reader released the last tile's scores;
-      // a single barrier would not do, as the upper half may be one tile ahead.)
+      // The four lanes of a row here; its two key halves and the row's result are left to the last warp, so
+      // that these go on with the next tile (done by the lower half, 3k clocks a tile).
       merge_lanes(ra);
       merge_lanes(rb);
-      // Lane 0 of a row's four goes on with row A, lane 1 with row B.
-      RowState r = cq & 1 ? rb : ra;
-      const int row = cq & 1 ? rB : rA;
-      RowState* upper = bars->upper[it & 1];
-      if (khalf == 1) {
-        if (cq < 2) upper[row] = r;
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&bars->half_full[it & 1][grp]);
-        continue;
-      }
-      ok = tc::mbar_wait(&bars->half_full[it & 1][grp], (it >> 1) & 1, abort, p.status);
+      const int pb = it & 1;
+      ok = it < 2 || tc::mbar_wait(&bars->st_free[pb], ((it >> 1) - 1) & 1, abort, p.status);
       if (!ok) break;
-      r = merge(r, upper[row]);
-      float sum = 0.f, sum_lo = 0.f;  // this row group's KL and the rounding of its additions
-      const float kl = kLn2 * (p.sl2 * __fdiv_rn(r.a, r.lt) + (r.ms - r.mt) + log2f(__fdiv_rn(r.ls, r.lt)));
-      const int t = q0 + row;
-      if (cq < 2 && t < p.T) {
-        sum = kl;
-        const int64_t at = (((int64_t)tl.c * p.B + tl.b) * p.Hq + tl.h) * p.T + t;
-        if (p.kl_rows && in_bounds(at, (int64_t)p.C * p.B * p.Hq * p.T, p.status)) p.kl_rows[at] = kl;
-      }
-      {  // rows A and B, then the eight pairs of them
-        const float other = __shfl_xor_sync(0xffffffffu, sum, 1);
-        two_sum(sum, other, sum, sum_lo);
-      }
+      if (cq < 2) bars->state[pb][khalf][cq == 0 ? rA : rB] = cq == 0 ? ra : rb;
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&bars->st_full[pb]);
+    }
+  } else {  // --------------------------------------------------------------------- row results
+    for (int it = 0, k = sched_tile(0, grid, cta); k < p.ntiles; k = sched_tile(++it, grid, cta)) {
+      const KlTile tl = kl_tile(p, k);
+      const int pb = it & 1, q0 = tl.qb * BQ;
+      if (!tc::mbar_wait(&bars->st_full[pb], (it >> 1) & 1, abort, p.status)) break;
+      RowState r[4];
 #pragma unroll
-      for (int o = 4; o <= 16; o <<= 1) {
-        const float hi = __shfl_xor_sync(0xffffffffu, sum, o), lo = __shfl_xor_sync(0xffffffffu, sum_lo, o);
-        pair_add(sum, sum_lo, hi, lo);
-      }
-      if (lane == 0) {  // the last of the tile's eight row groups adds them up, in their order
-        float2* red = bars->red[it & 1];
-        red[grp] = make_float2(sum, sum_lo);
-        __threadfence_block();
-        if (atomicAdd(&bars->done[it & 1], 1) == 7) {
-          __threadfence_block();
-          double tot = 0.0;
-          for (int i = 0; i < 8; ++i) {
-            const volatile float* v = reinterpret_cast<volatile float*>(red + i);
-            tot += (double)v[0] + (double)v[1];
-          }
-          bars->done[it & 1] = 0;
-          const int64_t pi = (((int64_t)tl.c * p.B + tl.b) * p.Hq + tl.h) * p.nP + tl.qb;
-          if (in_bounds(pi, (int64_t)p.C * p.B * p.Hq * p.nP, p.status)) p.part[pi] = tot;
+      for (int i = 0; i < 4; ++i)
+        r[i] = merge(bars->state[pb][0][32 * i + lane], bars->state[pb][1][32 * i + lane]);
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&bars->st_free[pb]);
+      float sum = 0.f, sum_lo = 0.f;  // KL over the tile's rows and the rounding of its additions
+      const int64_t head = ((int64_t)tl.c * p.B + tl.b) * p.Hq + tl.h;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float kl =
+            kLn2 * (p.sl2 * __fdiv_rn(r[i].a, r[i].lt) + (r[i].ms - r[i].mt) + log2f(__fdiv_rn(r[i].ls, r[i].lt)));
+        const int t = q0 + 32 * i + lane;
+        if (t < p.T) {
+          pair_add(sum, sum_lo, kl, 0.f);
+          if (p.kl_rows && in_bounds(head * p.T + t, (int64_t)p.C * p.B * p.Hq * p.T, p.status))
+            p.kl_rows[head * p.T + t] = kl;
         }
       }
+      warp_pair_sum(sum, sum_lo);
+      const int64_t pi = head * p.nP + tl.qb;
+      if (lane == 0 && in_bounds(pi, (int64_t)p.C * p.B * p.Hq * p.nP, p.status)) p.part[pi] = pair_value(sum, sum_lo);
     }
   }
   tc::fence_before_sync();

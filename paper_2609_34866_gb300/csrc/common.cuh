@@ -106,6 +106,21 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float h, float l)
   lo = __fadd_rn(__fadd_rn(lo, l), e);
 }
 
+// Value of a sum kept as a pair (the low part of an infinite one is NaN).
+__device__ __forceinline__ double pair_value(float hi, float lo) {
+  return fabsf(hi) < INFINITY ? (double)hi + (double)lo : (double)hi;
+}
+
+// Sum of a warp's pairs (hi, lo), in every lane. (The chip runs two FP64 operations a clock and SM: an fp64
+// warp_sum holds a role that others wait for ten times as long.)
+__device__ __forceinline__ void warp_pair_sum(float& hi, float& lo) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+    pair_add(hi, lo, h, l);
+  }
+}
+
 // Block-wide sum in a fixed order (deterministic); every thread gets the result.
 template <int NT>
 __device__ __forceinline__ double block_sum(double x, double* smem /* >= NT/32 */) {
