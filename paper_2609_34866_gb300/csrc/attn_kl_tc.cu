@@ -45,7 +45,8 @@ constexpr int NUM_THREADS = (2 + EW_WARPS + 1) * 32;  // warp 0 TMA, warp 1 UMMA
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleLog2 = 8.f;
-constexpr float kNoKey = -1e30f;  // running maximum before the first visible key (log2 units)
+constexpr float kNoKey = -1e30f;   // running maximum before the first visible key (log2 units)
+constexpr float kMasked = -1e38f;  // score of a hidden key: times the softmax scale far below kNoKey
 
 template <int DH>
 struct KlLayout {
@@ -356,14 +357,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           // rows past T have no result, so the causal mask alone hides the keys past T
           const int kl = j * BK + 64 * khalf - q0;  // first key of this warp, counted from the tile's first row
           if (kl > grp * 16 + 15) continue;         // no key of this half is visible to these 16 rows
-          const int k0 = kl + 2 * cq;
+          const uint32_t va = tc::columns_upto(rA - kl - 2 * cq), vb = tc::columns_upto(rB - kl - 2 * cq);
+          // (a finite score: no weight either, and the difference of two is 0)
 #pragma unroll
           for (int n = 0; n < 8; ++n)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-              const int key = k0 + 8 * n + e;
-              if (key > rA) xs[4 * n + e] = xt[4 * n + e] = -INFINITY;
-              if (key > rB) xs[4 * n + 2 + e] = xt[4 * n + 2 + e] = -INFINITY;
+              const int bit = 2 * n + e;
+              xs[4 * n + e] = (va >> bit) & 1 ? xs[4 * n + e] : kMasked;
+              xt[4 * n + e] = (va >> bit) & 1 ? xt[4 * n + e] : kMasked;
+              xs[4 * n + 2 + e] = (vb >> bit) & 1 ? xs[4 * n + 2 + e] : kMasked;
+              xt[4 * n + 2 + e] = (vb >> bit) & 1 ? xt[4 * n + 2 + e] : kMasked;
             }
         }
         float btA, btB, bsA, bsB;
@@ -388,11 +392,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           const float2 psA = make_float2(tc::fast_exp2(esA.x), tc::fast_exp2(esA.y));
           const float2 ptB = make_float2(tc::fast_exp2(etB.x), tc::fast_exp2(etB.y));
           const float2 psB = make_float2(tc::fast_exp2(esB.x), tc::fast_exp2(esB.y));
-          float2 dA = tc::sub2(tA2, sA2), dB = tc::sub2(tB2, sB2);
-          if (masked) {  // masked keys: -inf - (-inf) is NaN; their weight p^T is 0
-            dA = make_float2(fmaxf(dA.x, -1e30f), fmaxf(dA.y, -1e30f));
-            dB = make_float2(fmaxf(dB.x, -1e30f), fmaxf(dB.y, -1e30f));
-          }
+          const float2 dA = tc::sub2(tA2, sA2), dB = tc::sub2(tB2, sB2);
           ltA = tc::add2(ltA, ptA);
           lsA = tc::add2(lsA, psA);
           aA = tc::fma2(ptA, dA, aA);

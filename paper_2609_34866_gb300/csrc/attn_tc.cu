@@ -376,16 +376,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&bars->s_empty);  // S_{g+1} may overwrite the columns
         const int k0 = j * SKB + 2 * cq;
-        if (j * SKB + SKB - 1 > q0 || j * SKB + SKB > p.T) {  // diagonal or ragged block: mask
+        if (j * SKB + SKB - 1 > q0) {  // diagonal block (a ragged one is the last query rows' diagonal)
+          // rows past T have no result, so the causal mask alone hides the keys past T
+          const uint32_t va = tc::columns_upto(tA - k0), vb = tc::columns_upto(tB - k0);
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh)
 #pragma unroll
             for (int n = 0; n < 8; ++n)
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
-                const int key = k0 + 64 * hh + 8 * n + e;
-                if (key > tA || key >= p.T) x[hh][4 * n + e] = -INFINITY;
-                if (key > tB || key >= p.T) x[hh][4 * n + 2 + e] = -INFINITY;
+                const int bit = 2 * (8 * hh + n) + e;
+                x[hh][4 * n + e] = (va >> bit) & 1 ? x[hh][4 * n + e] : -INFINITY;
+                x[hh][4 * n + 2 + e] = (vb >> bit) & 1 ? x[hh][4 * n + 2 + e] : -INFINITY;
               }
         }
         float mxA = x[0][0], mxB = x[0][2];
