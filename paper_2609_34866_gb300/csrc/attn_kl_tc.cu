@@ -25,8 +25,8 @@
 //   warps 2..17  elementwise, 16 rows x 64 keys each (16x256b TMEM shape)
 //   warp 18      row results of the tile before, from the states of its two key halves in shared memory
 // Bound by the exponentials, 2 x 128 x 128 a block at 32 a clock and SM = 1024 clocks, next to 896 of packed
-// fp32 work and 512 (d_h 64) of products; 16 x 12 heads of 777 x 64 with four candidates take 136 us, about
-// 1800 clocks a block and 2500 a tile (one CTA a tile with eight elementwise warps: 227 us; with the rows'
+// fp32 work and 512 (d_h 64) of products; 16 x 12 heads of 777 x 64 with three candidates take 133 us,
+// about 1700 clocks a block and 2700 a tile (one CTA a tile with eight elementwise warps: 227 us; with the rows'
 // results in those warps, 4000 clocks more a tile: 173 us).
 // Outputs: per-row KL (optional) and one fp64 partial per tile, summed in fixed order afterwards.
 #include <cudaTypedefs.h>
