@@ -598,7 +598,9 @@ static jab_status backward_scales(const jab_block_desc* desc, int32_t B, int32_t
   // with the KL term the attention backward's dQKV^T is a times the MSE term's units
   const float coef = (float)(k * 2.0 / n_el / (kl ? (double)kl->ab[0] : 1.0));
   // per-split partials summed in order: the scale gradient is bit-identical between calls
-  float* gpart = reinterpret_cast<float*>(w + wp.gpart);
+  // (groups over several tiles have more partials than K ranges; at most kMaxSplits (G / 256 + 2) <= G of
+  // them per group, which the dW scratch holds)
+  float* gpart = reinterpret_cast<float*>(w + (lsq_group_parts(G) > 1 ? wp.dwscr : wp.gpart));
   JAB_SITE("wgrad_lsq", 1, launch_wgrad_lsq_tc(w + wp.dqkvt, wp.ldt, X_dev, W_dev, scales_dev, N, D,
                                                dm, G, bits, coef, gpart, &splits, status, st));
   FinishArgs f{};

@@ -51,7 +51,8 @@ struct GemmParams {
   const float* s;
   int d, G, bits;
   float coef;
-  float* dspart;  // fp32 [splits, M, d/G]: each unit's partial, summed over the splits in order
+  int parts;      // tiles that a group may touch (lsq_group_parts)
+  float* dspart;  // fp32 [splits, parts, M, d/G]: each unit's partials, summed in order afterwards
   // weight-gradient store epilogue (a split K adds partial tiles into a zeroed dw)
   float* dw;
 };
@@ -281,9 +282,24 @@ __device__ __forceinline__ void epi_lsq(const GemmParams& p, uint32_t taddr, int
   const int o = mb * BM + row;  // M = D is a multiple of 128: every row is valid
   const int qmax = qmax_of(p.bits);
   const int ng = p.d / p.G;
-  // one value per (split, row, group): this unit's tile covers whole groups (BN is a multiple of G)
-  float* part_out = p.dspart + ((int64_t)ks * p.M + o) * ng;
-  const int64_t part_extent = (int64_t)p.splits * p.M * ng;
+  // One value per (split, part, row, group): with parts = 1 this unit's tile covers whole groups (BN is a
+  // multiple of G); otherwise the tile is the group's part nb - (its first tile), and the one in which the
+  // group ends writes zeros for the parts it does not have.
+  const int64_t part_extent = (int64_t)p.splits * p.parts * p.M * ng;
+  float* part_out = p.dspart + ((int64_t)ks * p.parts * p.M + o) * ng;
+  const int64_t at0 = ((int64_t)ks * p.parts * p.M + o) * ng;
+  auto put = [&](int g, float v) {
+    if (p.parts == 1) {
+      if (in_bounds(at0 + g, part_extent, p.status)) part_out[g] = v;
+      return;
+    }
+    const int q0 = nb - (int)((int64_t)g * p.G / BN);
+    const int q1 = (int64_t)(g + 1) * p.G > (int64_t)(nb + 1) * BN ? q0 : p.parts - 1;
+    for (int q = q0; q <= q1; ++q) {
+      const int64_t at = (int64_t)q * p.M * ng + g;
+      if (in_bounds(at0 + at, part_extent, p.status)) part_out[at] = q == q0 ? v : 0.f;
+    }
+  };
   float part = 0.f;
   int cur = -1;
   // The weights and scale of a chunk are loaded while the one before it is summed.
@@ -315,15 +331,13 @@ __device__ __forceinline__ void epi_lsq(const GemmParams& p, uint32_t taddr, int
     tc::tmem_ld_wait();
     const int g = i0 / p.G;
     if (g != cur) {
-      if (cur >= 0 && in_bounds(((int64_t)ks * p.M + o) * ng + cur, part_extent, p.status))
-        part_out[cur] = p.coef * part;
+      if (cur >= 0) put(cur, p.coef * part);
       part = 0.f;
       cur = g;
     }
     part += lsq_chunk(r, w, sc, qmax);
   }
-  if (cur >= 0 && in_bounds(((int64_t)ks * p.M + o) * ng + cur, part_extent, p.status))
-    part_out[cur] = p.coef * part;
+  if (cur >= 0) put(cur, p.coef * part);
 }
 
 // ------------------------------------------------------------------ CTA-pair variant (cta_group::2)
@@ -663,6 +677,10 @@ int choose_splits(int tiles, int k_blocks, int sms) {
   return splits;
 }
 
+int lsq_group_parts(int G) {
+  return 256 % G == 0 ? 1 : G % 256 == 0 ? G / 256 : (G - 1) / 256 + 2;
+}
+
 cudaError_t launch_wgrad_lsq_tc(const void* dqkvt, int64_t ldt, const void* x, const void* w,
                                 const float* s, int64_t N, int D, int d, int G, int bits,
                                 float coef, float* dspart, int* splits, int* status, cudaStream_t st) {
@@ -685,9 +703,10 @@ cudaError_t launch_wgrad_lsq_tc(const void* dqkvt, int64_t ldt, const void* x, c
   p.bits = bits;
   p.coef = coef;
   p.dspart = dspart;
-  // every (split, row, group) partial is written once; the splits are summed in order by the caller's
+  // every (split, part, row, group) partial is written once; they are summed in order by the caller's
   // last launch: the scale gradient is bit-identical between calls
-  *splits = p.splits;
+  p.parts = lsq_group_parts(G);
+  *splits = p.splits * p.parts;
   // a tile covers whole groups: the narrow one only those that divide it
   return 128 % G == 0 && tile_cols(p.num_m, d, p.splits) == 128 ? launch_gemm2<kEpiLsq, true, true, 128>(ta, tb, ta, p, st)
                                                                 : launch_gemm2<kEpiLsq, true, true, 256>(ta, tb, ta, p, st);

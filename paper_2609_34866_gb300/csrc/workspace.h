@@ -30,7 +30,8 @@ struct Workspace {
   size_t ds;       // fp16 [B, Hq, nq (nq + 1) / 2, 128, 128]   dS^T tile of every (query block,
                    //                        key block <= query block) pair, nq = ceil(T / 128)
   size_t gpart;    // fp32 [kMaxSplits, D, d/G]  scale-gradient partial of every K split (summed in order)
-  size_t dwscr;    // fp32 [D, d]            dW when only its squared norm is asked for
+  size_t dwscr;    // fp32 [D, d]            dW when only its squared norm is asked for; the scale gradient's
+                   //                        partials where a group spans several GEMM tiles
   size_t lse_t;    // fp32 [B, Hq, Tp]       teacher log-sum-exp in log2 units (KL term's gradient)
   size_t klpart;   // fp64 [Hkv, B, nq]      KL partial sum of every teacher-probability CTA
   int64_t ldt;     // row pitch (elements) of dqkvt: N rounded up to 64

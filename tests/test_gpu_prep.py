@@ -237,3 +237,33 @@ def test_persistent_maps_equal_single_sequences(shape, T):
     ones = [run(c.X[b:b + 1].contiguous()) for b in range(B)]
     assert torch.equal(rows, torch.cat([r for r, _ in ones], 1))
     np.testing.assert_allclose(vhv.cpu(), torch.stack([v for _, v in ones]).mean(0).cpu(), rtol=1e-12)
+
+
+@pytest.mark.parametrize("d,G", [(768, 192), (960, 320), (768, 384), (1024, 512), (1280, 640), (768, 768), (768, 256)])
+@pytest.mark.parametrize("T", [65, 2600])
+def test_scale_gradient_of_groups_over_several_tiles(d, G, T):
+    """Groups that begin and end inside 256-column tiles or span several, with one K range and with
+    several (2600 tokens): the scale gradient against sums over each group of dL/dW times the LSQ factor,
+    dW from the weight-gradient call. The factors are exact fp32 and the sums over G products in fp32 differ
+    in order only: (G + 1) 2^-23 of the sum of magnitudes, and the splits' atomic order in dW as much again."""
+    from dataclasses import replace
+    from tests.harness import Case
+    from workloads import WORKLOADS
+    c = Case(replace(WORKLOADS["gpt2_smoke"], shape=BlockShape(d, 4, 1, 64, True, 500.0)), 1, T, G)
+    ws = c.workspace()
+    A, _, _ = c.gpu_teacher(ws)
+    s = c.gpu_scales(3)
+    loss = torch.empty(1, dtype=torch.float64, device="cuda")
+    grad, dw = torch.empty_like(s), torch.empty((c.D, d), dtype=torch.float32, device="cuda")
+    J().jab_loss_backward_scales(c.desc, 1, T, c.X, c.W, A, 3, s, 1.0, loss, grad, ws)
+    again = torch.empty_like(grad)
+    J().jab_loss_backward_scales(c.desc, 1, T, c.X, c.W, A, 3, s, 1.0, loss, again, ws)
+    J().jab_loss_backward_weights(c.desc, 1, T, c.X, c.W, A, 3, s, loss, grad_w=dw, ws=ws)
+    assert J().jab_get_device_status() == 0
+    assert torch.equal(grad, again)
+    q = (c.W.float().view(c.D, -1, G) / s[:, :, None]).double()
+    r = torch.where(q.abs() <= 3, torch.round(q) - q, torch.sign(q) * 3)
+    terms = r * dw.double().view(c.D, -1, G)
+    bound = 2 * (G + 1) * 2.0 ** -23 * terms.abs().sum(2)
+    err = (terms.sum(2) - grad.double()).abs()
+    assert bool((err <= bound).all()), (err / bound).max().item()
