@@ -21,9 +21,10 @@ constexpr int BQ = 128;          // query rows of a tile
 constexpr int EW_WARPS = 8;      // softmax warps
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
-// O is rescaled only when a row's maximum grows by more than 2^12: P then stays below 2^12, far inside
-// fp16, and large scores, which grow by 2^8 in most blocks of a heavy-tailed batch, rescale less often.
-constexpr float kRescaleLog2 = 12.f;
+// O is rescaled only when a row's maximum grows by more than 2^8, so P stays below 2^8, inside fp16. The
+// threshold is part of the result: P is rounded to fp16 relative to the running maximum, and another one
+// (2^12 rescales a heavy-tailed batch less often) moves the scale gradients of such batches by 1e-3.
+constexpr float kRescaleLog2 = 8.f;
 
 struct FwdParams {
   int T, B, C, Hq, Hkv, D, nqb, nP, lse_pitch;

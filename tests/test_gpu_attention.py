@@ -1,0 +1,72 @@
+"""The attention kernels at the points where their fast forms could go wrong: rounding of the forward's
+probabilities, extreme softmax scales, odd head ratios, grouped tile orders."""
+import numpy as np
+import pytest
+import torch
+
+from tests.harness import J
+from workloads import WORKLOADS, BlockShape
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2609_34866_gb300 import build
+    build.build()
+    J().jab_get_device_status()
+
+
+def _blockwise(qkv, shape, threshold):
+    """Causal attention of [T, D] fp16 projections over key blocks of 128 in float64, with the forward's one
+    rounding that is seen: P to fp16 relative to a running row maximum (log2 units) that moves to the
+    block's when it is exceeded by more than `threshold`; the row sums take P unrounded."""
+    T, (hq, hkv, dh) = qkv.shape[0], (shape.n_q_heads, shape.n_kv_heads, shape.head_dim)
+    y = qkv.double().reshape(T, -1, dh).transpose(0, 1)
+    q, k, v = y[:hq], y[hq:hq + hkv].repeat_interleave(hq // hkv, 0), y[hq + hkv:].repeat_interleave(hq // hkv, 0)
+    sl2 = float(np.float32(np.float32(1 / np.sqrt(dh)) * np.float32(1.4426950408889634)))
+    m = torch.full((hq, T, 1), -torch.inf, dtype=torch.float64, device=qkv.device)
+    den = torch.zeros_like(m)
+    out = torch.zeros((hq, T, dh), dtype=torch.float64, device=qkv.device)
+    for k0 in range(0, T, 128):
+        s = q @ k[:, k0:k0 + 128].transpose(1, 2)
+        hidden = torch.arange(k0, min(k0 + 128, T), device=s.device)[None, :] > torch.arange(T, device=s.device)[:, None]
+        s.masked_fill_(hidden, -torch.inf)
+        top = (s.amax(2, keepdim=True).float() * sl2).double()  # (float, as the kernel forms it)
+        moved = torch.maximum(m, top)
+        new = torch.where(moved > m + threshold, moved, m)
+        p = torch.where(hidden, 0.0, torch.exp2(s * sl2 - new))
+        old = torch.where(new > m, torch.exp2(m - new), 1.0)
+        den = den * old + p.sum(2, keepdim=True)
+        out = out * old + p.half().double() @ v[:, k0:k0 + 128]
+        m = new
+    return (out / den).transpose(0, 1).reshape(T, hq * dh)
+
+
+@pytest.mark.parametrize("shape", [BlockShape(256, 4, 1, 64, False), BlockShape(256, 3, 1, 128, False)])
+def test_forward_rounds_p_at_a_maximum_moved_beyond_two_to_the_eight(shape):
+    """Later key blocks have larger scores, so that row maxima grow by 2^8 .. 2^12 from one block to the
+    next. The output is that of P rounded to fp16 relative to a maximum that has moved, not one that has
+    stayed: in rows where the two differ they are independent roundings of 2^-11, while the fp32 scores
+    and exponentials (about 1e-5 relative here) turn a few roundings in a hundred."""
+    from dataclasses import replace
+    from tests.harness import Case
+    T = 384
+    c = Case(replace(WORKLOADS["gpt2_smoke"], shape=shape), 2, T, 64)
+    c.X.mul_(torch.tensor([1.0, 2.0, 3.0], device="cuda").repeat_interleave(128)[None, :, None])
+    c.W.mul_(3.0)
+    A, _, _ = c.gpu_teacher()
+    qkv = torch.empty((c.B, T, c.D), dtype=torch.float16, device="cuda")
+    J().jab_reference_projection(c.desc, c.B, T, c.X, c.W, qkv, c.workspace())
+    assert J().jab_get_device_status() == 0
+    eight, twelve = (torch.stack([_blockwise(qkv[b], shape, th) for b in range(c.B)]) for th in (8.0, 12.0))
+    differ = (eight != twelve).reshape(c.B, T, c.Hq, -1).any(-1, keepdim=True)
+    assert differ.float().mean() > 0.02, differ.float().mean()
+
+    def distance(e):
+        return ((A.double() - e).reshape(c.B, T, c.Hq, -1) * differ).norm().item()
+
+    assert distance(eight) < 0.5 * distance(twelve), (distance(eight), distance(twelve))
