@@ -163,7 +163,9 @@ jab_status jab_rademacher_probes(uint64_t seed, int64_t first, int64_t n, void* 
  *   C1: Omega(b) = Tr(H) ||Q_b(W) - W||_F^2,   C2: (L - i) Omega(b) with layers_after = L - i.
  *   trace_dev      fp64 [1] on the device (e.g. from jab_hutchinson_trace)
  *   c1_dev         out fp64 [n_cand];  c2_dev  out fp64 [n_cand] or NULL
- *   ws             at least jab_workspace_size(desc, 1, 1, n_cand, 0) bytes
+ *   ws             at least jab_workspace_size(desc, 1, 1, n_cand, 0) bytes. An X converted into it
+ *                  (jab_prepare_x) stays if ws_bytes leaves n_cand * 8192 bytes behind it; else
+ *                  *_prepared calls return JAB_ERR_INVALID_ARG until X is converted again
  * The squared error is summed in fp64 in a fixed order (repeated calls give identical bits). */
 jab_status jab_omega_scores(const jab_block_desc* desc, const void* W_dev, int32_t n_cand,
                             const int32_t* bits_host, const float* const* scales_host,

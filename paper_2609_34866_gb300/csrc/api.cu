@@ -156,6 +156,22 @@ bool is_prepared(const void* ws, const void* x, int32_t B, int32_t T, int32_t d)
   return false;
 }
 
+// Where a call that converts no X into the workspace may put `bytes` of scratch that its own layout has at
+// offset `at`: there, or behind the X that the workspace holds in fp16 (x16: its offset, the same in every
+// layout), or, where that is past ws_bytes, there all the same, and the X counts as gone.
+size_t beside_prepared(const void* ws, size_t ws_bytes, size_t x16, size_t at, size_t bytes) {
+  std::lock_guard<std::mutex> lk(g_prep_mu);
+  for (auto e = g_prep.begin(); e != g_prep.end(); ++e)
+    if (e->ws == ws) {
+      const size_t end = align_up(x16 + (size_t)e->B * e->T * e->d * 2, 256);
+      if (at >= end || at + bytes <= x16) return at;
+      if (end + bytes <= ws_bytes) return end;
+      g_prep.erase(e);
+      return at;
+    }
+  return at;
+}
+
 // The reductions' block counter and partial slots in the workspace.
 int* reduce_counter(void* ws, const Workspace& wp) {
   return reinterpret_cast<int*>(static_cast<char*>(ws) + wp.status);
@@ -482,7 +498,9 @@ jab_status jab_omega_scores(const jab_block_desc* desc, const void* W_dev, int32
   int sms;
   if ((s = device_info(&status, &sms)) != JAB_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  double* red = reinterpret_cast<double*>(static_cast<char*>(ws) + wp.red);
+  // (this call's own small layout has the partials where a larger one keeps the fp16 X of the *_prepared calls)
+  double* red = reinterpret_cast<double*>(
+      static_cast<char*>(ws) + beside_prepared(ws, ws_bytes, wp.x16, wp.red, (size_t)n_cand * kRedBlocks * 8));
   const int D = (int)block_rows(desc), dm = desc->d_model;
   for (int c = 0; c < n_cand; ++c)
     JAB_SITE("qerr", 1, launch_qerr_partial(W_dev, scales_host[c], D, dm, desc->group_size,

@@ -267,3 +267,36 @@ def test_scale_gradient_of_groups_over_several_tiles(d, G, T):
     bound = 2 * (G + 1) * 2.0 ** -23 * terms.abs().sum(2)
     err = (terms.sum(2) - grad.double()).abs()
     assert bool((err <= bound).all()), (err / bound).max().item()
+
+
+def test_omega_scores_keep_the_prepared_x():
+    """jab_prepare_x, jab_omega_scores and the prepared fit on one workspace: Omega's partials lie behind
+    the converted X, and the fit has the plain call's bits. Where the workspace given to Omega is too small
+    for that, the prepared call is refused."""
+    from dataclasses import replace
+    from tests.harness import Case
+    from workloads import WORKLOADS
+    c = Case(replace(WORKLOADS["gpt2_smoke"], shape=BlockShape(256, 4, 1, 64, True, 500.0)), 8, 256, 64)
+    ws = c.workspace(n_cand=2)
+    A, _, _ = c.gpu_teacher(ws)
+    s = c.gpu_scales(3)
+    bits, scales = [3, 4], [s, c.gpu_scales(4)]
+    one = torch.ones(1, dtype=torch.float64, device="cuda")
+    want, got = torch.empty(2, dtype=torch.float64, device="cuda"), torch.empty(2, dtype=torch.float64, device="cuda")
+    J().jab_omega_scores(c.desc, c.W, bits, scales, one, 1, want, J().Workspace(c.desc, 1, 1, 2, False))
+    l0, l1 = (torch.empty(1, dtype=torch.float64, device="cuda") for _ in range(2))
+    g0, g1 = torch.empty_like(s), torch.empty_like(s)
+    J().jab_loss_backward_scales(c.desc, c.B, c.T, c.X, c.W, A, 3, s, 0.0, l0, g0, ws)
+    J().jab_prepare_x(c.desc, c.B, c.T, c.X, ws)
+    J().jab_omega_scores(c.desc, c.W, bits, scales, one, 1, got, ws)
+    J().jab_loss_backward_scales_prepared(c.desc, c.B, c.T, c.X, c.W, A, 3, s, 0.0, l1, g1, ws)
+    assert l0.item() == l1.item() and torch.equal(g0, g1) and torch.equal(want, got)
+    small = J().Workspace(c.desc, 1, 1, 2, False)
+    small.buf = ws.buf                                 # the same memory, fewer bytes of it
+    assert small.nbytes < c.B * c.T * 256 * 2
+    J().jab_prepare_x(c.desc, c.B, c.T, c.X, ws)
+    J().jab_omega_scores(c.desc, c.W, bits, scales, one, 1, got, small)
+    with pytest.raises(J().JabError) as e:
+        J().jab_loss_backward_scales_prepared(c.desc, c.B, c.T, c.X, c.W, A, 3, s, 0.0, l1, g1, ws)
+    assert e.value.status == 1 and torch.equal(want, got)
+    assert J().jab_get_device_status() == 0
