@@ -45,8 +45,11 @@ constexpr int NUM_THREADS = (2 + EW_WARPS + 1) * 32;  // warp 0 TMA, warp 1 UMMA
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleLog2 = 8.f;
-constexpr float kNoKey = -1e30f;   // running maximum before the first visible key (log2 units)
-constexpr float kMasked = -1e38f;  // score of a hidden key: times the softmax scale far below kNoKey
+// Score of a hidden key: finite, so that the difference of two is 0. Products of fp16 rows stay below 2^40, so
+// with the running maximum before the first visible key at no_key = -(2^41 sl2 + 2^10) every visible
+// score is above it and a hidden one, times sl2, more than 2^10 below, for every sl2 from kMinSl2 on.
+constexpr float kMasked = -3e38f;
+constexpr float kMinSl2 = 1e-34f;
 
 template <int DH>
 struct KlLayout {
@@ -81,6 +84,7 @@ struct KlParams {
   int T, B, C, Hq, Hkv, D, nqb, nP, ntiles, balanced;
   FastDiv outer, by_ratio, by_hkv, by_b;  // by the tiles of one length (balanced) or of one group; Hq / Hkv; Hkv; B
   float sl2;           // softmax scale * log2(e)
+  float no_key;        // running maximum before the first visible key (log2 units)
   double* part;        // [C, B, Hq, nP]  sum of KL_i over the tile's rows
   float* kl_rows;      // [C, B, Hq, T] or null
   int* status;
@@ -328,7 +332,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     for (int it = 0, k = sched_tile(0, grid, cta); ok && k < p.ntiles; k = sched_tile(++it, grid, cta)) {
       const KlTile tl = kl_tile(p, k);
       const int q0 = tl.qb * BQ, nkb = tl.qb + 1;
-      RowState ra{kNoKey, kNoKey, 0.f, 0.f, 0.f}, rb = ra;
+      RowState ra{p.no_key, p.no_key, 0.f, 0.f, 0.f}, rb = ra;
       for (int j = 0; j < nkb; ++j, ++g) {
         if (!tc::mbar_wait(&bars->s_full, g & 1, abort, p.status)) {
           ok = false;
@@ -520,7 +524,8 @@ cudaError_t launch_attn_kl_tc(const void* qkv_s, int64_t ldq, const void* qkv_t,
   p.D = D;
   p.nqb = (T + BQ - 1) / BQ;
   p.nP = nP;
-  p.sl2 = scale * kLog2e;
+  p.sl2 = std::max(scale * kLog2e, kMinSl2);  // (far above it already every map is uniform)
+  p.no_key = -std::min(2199023255552.f * p.sl2 + 1024.f, 3e38f);
   p.part = part;
   p.kl_rows = kl_rows;
   p.status = status;

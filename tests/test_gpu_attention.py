@@ -70,3 +70,29 @@ def test_forward_rounds_p_at_a_maximum_moved_beyond_two_to_the_eight(shape):
         return ((A.double() - e).reshape(c.B, T, c.Hq, -1) * differ).norm().item()
 
     assert distance(eight) < 0.5 * distance(twelve), (distance(eight), distance(twelve))
+
+
+@pytest.mark.parametrize("scale", [1e-6, 1e-9, 1e-30, 1e-37])
+@pytest.mark.parametrize("T", [5, 200])
+def test_kl_rows_vanish_with_the_softmax_scale(scale, T):
+    """With a softmax scale near 0 both maps are uniform over the visible keys: the KL of a row is of the
+    size of the squared score differences, 1e-11 at most here, and the difference form rounds to 1e-7 of
+    its terms. Hidden keys keep no weight, however small the scale that multiplies their score."""
+    from dataclasses import replace
+    from tests.harness import KL_ROW_ATOL, Case
+    c = Case(replace(WORKLOADS["gpt2_smoke"], shape=BlockShape(256, 4, 1, 64, True, 500.0)), 2, T, 64)
+    c.desc.softmax_scale = scale
+    ws = c.workspace(with_bwd=False)
+    A, _, _ = c.gpu_teacher(ws)
+    qkv = torch.empty((c.B, T, c.D), dtype=torch.float16, device="cuda")
+    rows = torch.empty((1, c.B, c.Hq, T), dtype=torch.float32, device="cuda")
+    loss, kl = (torch.empty(1, dtype=torch.float64, device="cuda") for _ in range(2))
+    J().jab_reference_projection(c.desc, c.B, T, c.X, c.W, qkv, ws)
+    J().jab_loss_forward_kl(c.desc, c.B, T, c.X, c.W, A, qkv, [3], [c.gpu_scales(3)], 0.1, loss, ws, kl=kl,
+                            kl_rows=rows)
+    assert J().jab_get_device_status() == 0
+    assert rows.abs().max().item() <= KL_ROW_ATOL, rows.abs().max()
+    np.testing.assert_allclose(kl.item(), rows.double().sum().item() / c.B, rtol=1e-6, atol=1e-12)
+    v = qkv[..., -c.dh:].double()  # (one KV head) the uniform map's output: the mean of the visible values
+    mean = (v.cumsum(1) / torch.arange(1, T + 1, device="cuda")[:, None]).repeat(1, 1, c.Hq)
+    assert (A.double() - mean).abs().max() <= 2e-3 * mean.abs().max()
