@@ -64,7 +64,7 @@ __device__ __forceinline__ void convert_x_role(const uint4* __restrict__ x, uint
 }
 
 // ---------------------------------------------------------------- quantiser (Section 2.1, Eq. 2)
-// Codes of 8 weights that share a scale, as floats: clip(rint(fl32(w / s))).
+// Codes of 8 weights that share a scale, as floats: clip(rint(fl32(w / s))), a zero of either sign.
 __device__ __forceinline__ void quant_codes8(const uint4& v, float sc, int qmax, float (&q)[8]) {
   const uint32_t w2[4] = {v.x, v.y, v.z, v.w};
   const bf16_t* b = reinterpret_cast<const bf16_t*>(&v);
@@ -158,8 +158,11 @@ __global__ void __launch_bounds__(256) quantize_kernel(const uint4* __restrict__
       *reinterpret_cast<uint2*>(codes + i * 8) = make_uint2(c[0], c[1]);
     }
     if (w_hat32) {
+      const uint32_t w2[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int k = 0; k < 8; ++k) q[k] = __fmul_rn(q[k], sc);
+      for (int k = 0; k < 8; ++k)  // with the weight's sign, which rint keeps in a code of 0 and quant_codes8 does not
+        q[k] = __uint_as_float(__float_as_uint(__fmul_rn(q[k], sc)) |
+                               ((k & 1 ? w2[k / 2] : w2[k / 2] << 16) & 0x80000000u));
       reinterpret_cast<float4*>(w_hat32 + i * 8)[0] = make_float4(q[0], q[1], q[2], q[3]);
       reinterpret_cast<float4*>(w_hat32 + i * 8)[1] = make_float4(q[4], q[5], q[6], q[7]);
     }

@@ -300,3 +300,24 @@ def test_omega_scores_keep_the_prepared_x():
         J().jab_loss_backward_scales_prepared(c.desc, c.B, c.T, c.X, c.W, A, 3, s, 0.0, l1, g1, ws)
     assert e.value.status == 1 and torch.equal(want, got)
     assert J().jab_get_device_status() == 0
+
+
+@pytest.mark.parametrize("bits", [2, 8])
+@pytest.mark.parametrize("s_mul", [1.0, 1e-25])
+def test_w_hat_of_small_negative_weights_is_negative_zero(bits, s_mul):
+    """A weight below half a step has the code 0, and fl32(0 s) the weight's sign as rint gives it, by the
+    corrected reciprocal (scale 1) and by the division (scale 1e-25) alike."""
+    d, G = 128, 64
+    g = torch.Generator().manual_seed(7)
+    w = torch.randn((256, d), generator=g) * 0.5
+    w[:, ::5] *= 0.0                                   # +0 and -0
+    w = (w * s_mul).to(torch.bfloat16)
+    s = np.full((256, d // G), s_mul, dtype=np.float32)
+    desc = J().desc_from_shape(BlockShape(d, 2, 1, 64, False), G)
+    w_hat = torch.empty(w.shape, dtype=torch.float32, device="cuda")
+    J().jab_quantize(desc, bits, w.cuda(), torch.from_numpy(s).cuda(), w_hat=w_hat)
+    _, ow, _ = O.quantize(np64(w), s, bits, G)
+    want = ow.astype(np.float32)
+    assert (np.signbit(want) & (want == 0)).any()
+    np.testing.assert_array_equal(w_hat.cpu().numpy().view(np.uint32), want.view(np.uint32))
+    assert J().jab_get_device_status() == 0
