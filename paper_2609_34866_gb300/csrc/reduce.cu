@@ -107,10 +107,11 @@ __global__ void check_finite_kernel(const float* __restrict__ x, int64_t n, int*
 
 // Sum of squares: block b sums its contiguous chunk (fixed per-thread order, fixed tree), one block then
 // adds the kRedBlocks partials. The chip runs about two FP64 operations per clock and SM, and a
-// conversion and a multiply-add per value bounded the kernel (101 us for 25M values, now 32): eight squares
-// are added as unevaluated pairs of floats, errors carried along (2^-46 of the sum), and only that goes to
-// the fp64 accumulator. Values whose largest is outside 2^-40 .. 2^60 are squared in fp64. With `status` a
-// non-finite value is reported.
+// conversion and a multiply-add per value bounded the kernel (101 us for 25M values, now 43): eight squares
+// are added in floats with every rounding error carried along, and only that goes to the fp64 accumulator.
+// The products' low parts are a pair of their own: their last bits do not round evenly (an odd
+// square is 1 modulo 8), and with all errors in one float the sum came out 1.1e-15 small. Values whose
+// largest is outside 2^-40 .. 2^60 are squared in fp64. With `status` a non-finite value is reported.
 __device__ __forceinline__ double sumsq8(const float (&v)[8]) {
   float big = 0.f;
 #pragma unroll
@@ -120,16 +121,21 @@ __device__ __forceinline__ double sumsq8(const float (&v)[8]) {
     for (int k = 0; k < 8; ++k) acc += (double)v[k] * (double)v[k];
     return acc;
   }
-  float sh = 0.f, sl = 0.f;
+  float sh = 0.f, se = 0.f, sl = 0.f, s3 = 0.f;  // products and their sums' errors, low parts and theirs
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const float h = __fmul_rn(v[k], v[k]), l = __fmaf_rn(v[k], v[k], -h);
-    const float t = __fadd_rn(sh, h), bb = __fsub_rn(t, sh);
-    const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bb)), __fsub_rn(h, bb));  // sh + h = t + e
+    float t, e;
+    two_sum(sh, h, t, e);
     sh = t;
-    sl = __fadd_rn(sl, __fadd_rn(e, l));
+    se = __fadd_rn(se, e);
+    two_sum(sl, l, t, e);
+    sl = t;
+    s3 = __fadd_rn(s3, e);
   }
-  return (double)sh + (double)sl;
+  float a, b;
+  two_sum(se, sl, a, b);
+  return (double)sh + ((double)a + (double)__fadd_rn(b, s3));
 }
 
 __global__ void __launch_bounds__(256) sumsq_partial_kernel(const float* __restrict__ x, int64_t n,

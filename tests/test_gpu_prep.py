@@ -321,3 +321,27 @@ def test_w_hat_of_small_negative_weights_is_negative_zero(bits, s_mul):
     assert (np.signbit(want) & (want == 0)).any()
     np.testing.assert_array_equal(w_hat.cpu().numpy().view(np.uint32), want.view(np.uint32))
     assert J().jab_get_device_status() == 0
+
+
+def test_weight_gradient_norm_is_not_biased():
+    """||dW||^2 against the exact sum of the returned dW's squares (fp32 squares are exact in fp64): eight
+    batches' errors are independent roundings of about 2^-53 in the last additions, so that their mean is
+    below 2^-52; low parts that are dropped would all fall on one side."""
+    import math
+    from dataclasses import replace
+    from tests.harness import Case
+    from workloads import WORKLOADS
+    errors = []
+    for seed in range(8):
+        wl = replace(WORKLOADS["gpt2_smoke"], shape=BlockShape(256, 4, 1, 64, True, 500.0), seed=seed)
+        c = Case(wl, 2, 65, 64)
+        ws = c.workspace()
+        A, _, _ = c.gpu_teacher(ws)
+        loss, sq = (torch.empty(1, dtype=torch.float64, device="cuda") for _ in range(2))
+        dw = torch.empty((c.D, 256), dtype=torch.float32, device="cuda")
+        J().jab_loss_backward_weights(c.desc, 2, 65, c.X, c.W, A, 2, c.gpu_scales(2), loss, grad_w=dw, grad_sqnorm=sq,
+                                      ws=ws)
+        exact = math.fsum((np64(dw).ravel() ** 2).tolist())
+        errors.append(sq.item() / exact - 1)
+    assert J().jab_get_device_status() == 0
+    assert abs(np.mean(errors)) <= 2.0 ** -52, errors
