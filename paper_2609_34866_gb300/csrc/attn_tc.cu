@@ -13,6 +13,7 @@
 
 #include "kernels.h"
 #include "tc.cuh"
+#include "two_boxes.h"
 
 namespace jab {
 namespace {
@@ -504,7 +505,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const int y_off = (quarter * 32) & (RPH - 1);  // this warp's rows lie in one head
     const int h_off = quarter * 32 / RPH;
     int tc_ = 0;
-    int cc = 0;               // chunks done: buffer cc & 1, phase (cc >> 1) & 1
+    int cc = 0;               // chunks done: buffer cc & 1
     uint32_t range_bits = 0;  // mode 2: an fp16 dO value out of range (inf) or NaN
     const int64_t ext_p = (int64_t)p.C * p.B * p.Hq * p.nP;       // loss partials
     // This row's A_ref (DH fp32) of tile k into L2, one line at a time.
@@ -518,17 +519,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       for (int l = 0; l < NCH; ++l) tc::prefetch_line_l2(src + 32 * l);
     };
     // The loads of A_ref run two chunks ahead: the next one is chunk lch of tile lt, which is round lit's.
-    int lit = 0, lk = sched_tile(0, gridDim.x, blockIdx.x), lch = 0, issued = 0;
+    int lit = 0, lk = sched_tile(0, gridDim.x, blockIdx.x), lch = 0;
+    TwoBoxes loads;
     StackTile lt = stack_tile(p, lk < ntiles ? lk : 0, RPH);
     auto load_next = [&] {  // the whole warp
       if (lk >= ntiles) return;
-      const int i = issued & 1;
+      const int i = loads.next();
       if (tc::elect_one()) {
         tc::mbar_expect_tx(&a_full[i], 4096);
         tc::tma_load_3d(buf + 4096 * i, &tm_a, &a_full[i], (HPT * lt.hu + h_off) * DH + lch * 32,
                         lt.qb * RPH + y_off, lt.bc - p.by_b.quot(lt.bc) * p.B);
       }
-      ++issued;
+      ++loads.issued;
       if (++lch == NCH) {
         lch = 0;
         lk = sched_tile(++lit, gridDim.x, blockIdx.x);
@@ -569,7 +571,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         auto process = [&](int ch, const uint32_t (&r)[32]) {
           const int i = cc & 1;
           uint8_t* bf = buf + 4096 * i;
-          if (MODE != 0 && !tc::mbar_wait(&a_full[i], (cc >> 1) & 1, abort, p.status)) have = false;
+          // (as many loads have landed as chunks are done; what follows a wait given up is not used)
+          if (MODE != 0 && have)
+            have = loads.take([&](int u, uint32_t ph) { return tc::mbar_wait(&a_full[u], ph, abort, p.status); });
           if (MODE == 0) {  // this buffer's last store (issued by the same elected lane) has been read
             if (tc::elect_one()) tc::bulk_wait_group_read<1>();
             __syncwarp();
@@ -662,7 +666,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
     if (MODE != 1 && tc::elect_one()) tc::bulk_wait_group<0>();
     if (MODE != 0)  // loads that nobody waited for land before shared memory goes
-      for (int i = cc; i < issued; ++i) drain_wait(&a_full[i & 1], (i >> 1) & 1);
+      loads.drain([&](int u, uint32_t ph) { drain_wait(&a_full[u], ph); });
     if (MODE == 2 && either_at_least(range_bits, kHalfInf)) report(p.status, JAB_ERR_RANGE);
   }
   tc::fence_before_sync();
