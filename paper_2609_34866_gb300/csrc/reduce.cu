@@ -25,8 +25,9 @@ __device__ __forceinline__ double loss_slice(const double* __restrict__ part, in
   return warp_sum(acc);
 }
 
-// Counts a warp's published partial (of `total`); true, in all its lanes, in the one that comes last, with
-// every partial visible. The counter (0 before the launch) is left at 0.
+// Counts a warp's partial, published by its lane 0 (of `total`); true, in all its lanes, in the one that comes
+// last, with every partial visible: lane 0's fences order its count against the partials, and __syncwarp the
+// other lanes' reads behind it (a shuffle orders no memory). The counter (0 before the launch) is left at 0.
 __device__ __forceinline__ bool last_warp(int* counter, int total) {
   int last = 0;
   if ((threadIdx.x & 31) == 0) {
@@ -37,6 +38,7 @@ __device__ __forceinline__ bool last_warp(int* counter, int total) {
       __threadfence();
     }
   }
+  __syncwarp();
   return __shfl_sync(0xffffffffu, last, 0) != 0;
 }
 
