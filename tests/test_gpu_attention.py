@@ -96,3 +96,27 @@ def test_kl_rows_vanish_with_the_softmax_scale(scale, T):
     v = qkv[..., -c.dh:].double()  # (one KV head) the uniform map's output: the mean of the visible values
     mean = (v.cumsum(1) / torch.arange(1, T + 1, device="cuda")[:, None]).repeat(1, 1, c.Hq)
     assert (A.double() - mean).abs().max() <= 2e-3 * mean.abs().max()
+
+
+@pytest.mark.parametrize("shape,B,T,bits", [(BlockShape(768, 6, 2, 128, True, 1e4), 2, 171, 3),
+                                            (BlockShape(384, 6, 2, 64, False), 1, 300, 2)])
+def test_three_query_heads_per_kv_head(shape, B, T, bits):
+    """An odd head ratio above 1 at both head sizes (tiles of 128 rows of one head): the teacher's output,
+    the candidates' losses, the KL maps, the Hessian products and the gradients with and without the KL term
+    against the oracle, with the bars of the other head ratios."""
+    from dataclasses import replace
+    from tests import test_gpu_parity as P
+    from tests.harness import Case
+    name = f"ratio3_dh{shape.head_dim}_T{T}"
+    P._cases[name] = Case(replace(WORKLOADS["gpt2_smoke"], shape=shape), B, T, 64)
+    try:
+        P.test_teacher_output_parity(name)
+        P.test_loss_forward_parity(name)
+        P.test_kl_forward_parity(name)
+        P.test_hutchinson_trace_parity(name)
+        P.test_backward_parity(name, bits)
+        P.test_weight_gradient_and_fisher_coupling_score(name, bits)
+        for regime in ("default", "balanced"):
+            P.test_backward_kl_parity(name, bits, regime)
+    finally:
+        del P._cases[name]

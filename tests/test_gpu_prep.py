@@ -176,6 +176,8 @@ def test_weight_gradient_norm_and_loss_parts_of_odd_batches(B, T):
                                        (BlockShape(768, 12, 12, 64, False), 1, 1337),
                                        (BlockShape(512, 4, 2, 128, True, 1e4), 3, 43),
                                        (BlockShape(512, 20, 2, 128, True, 1e4), 4, 301),
+                                       (BlockShape(256, 3, 1, 128, True, 1e4), 2, 65),
+                                       (BlockShape(256, 3, 1, 128, True, 1e4), 16, 395),
                                        (BlockShape(256, 4, 1, 64, True, 500.0), 2, 65)])
 def test_projection_with_narrow_and_wide_tiles(shape, B, T):
     """[Q | K | V] with RoPE from 128- and 256-column tiles (few tiles, or most of a round of CTA pairs),
@@ -204,16 +206,21 @@ def test_projection_with_narrow_and_wide_tiles(shape, B, T):
     assert (err <= bound).all(), (err / bound).max()
 
 
-@pytest.mark.parametrize("shape", [BlockShape(256, 4, 1, 64, True, 500.0), BlockShape(512, 4, 2, 128, True, 1e4)])
-@pytest.mark.parametrize("T", [128, 333])
-def test_persistent_maps_equal_single_sequences(shape, T):
-    """KL maps and Hessian products of a batch with several tiles per persistent CTA (and, in the longer
-    one, of several lengths): every KL row has the bits of a call with that sequence alone, and the
+@pytest.mark.parametrize("shape,B,T", [(BlockShape(256, 4, 1, 64, True, 500.0), 96, 128),
+                                       (BlockShape(256, 4, 1, 64, True, 500.0), 96, 333),
+                                       (BlockShape(512, 4, 2, 128, True, 1e4), 96, 128),
+                                       (BlockShape(512, 4, 2, 128, True, 1e4), 96, 333),
+                                       (BlockShape(256, 4, 1, 64, True, 500.0), 320, 333),
+                                       (BlockShape(256, 6, 2, 128, True, 1e4), 216, 333)])
+def test_persistent_maps_equal_single_sequences(shape, B, T):
+    """KL maps and Hessian products of a batch with several tiles per persistent CTA (of several lengths
+    where T > 128; in the last two cases with more than 24 tiles per SM, so that tiles go by KV head and not
+    by length, the last with three query heads per KV head): every KL row has the bits of a call with that sequence alone, and the
     probes' v^T H v, sums of per-sequence values over n, agree to the fp64 sums' 2^-52 a term."""
     from dataclasses import replace
     from tests.harness import Case
     from workloads import WORKLOADS
-    B, bits = 96, [2, 4]
+    bits = [2, 4]
     c = Case(replace(WORKLOADS["gpt2_smoke"], shape=shape), B, T, 64)
 
     def run(X):
