@@ -219,7 +219,7 @@ struct DkdvBars {
 // each thread loads its 16 words while dP^T is on its way, adds b_kl (P - P^T) to a_mse P (dP - D), and the
 // dS^T tile is stored over them. (Through shared memory, where it had to share the dS^T staging tile, a
 // block's P^T could be loaded only when the previous dS^T had been stored, a round trip per block: a whole
-// fitting step of 8 x 2048 tokens took 2605 us against 2469 us.)
+// fitting step of 8 x 2048 tokens took 2694 us against 2600 us.)
 
 // First of the four 16-byte words, 512 bytes apart, that a lane of elementwise warp w (0 .. 15) holds of a
 // P^T tile of 32 KB: its packed words 4 q .. 4 q + 3 in word q, so that a warp moves 512 bytes at a time.

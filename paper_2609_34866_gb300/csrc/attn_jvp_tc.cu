@@ -496,11 +496,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       } else {
         ok = false;
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float hi = __shfl_xor_sync(0xffffffffu, sq, o), lo = __shfl_xor_sync(0xffffffffu, sq_lo, o);
-        pair_add(sq, sq_lo, hi, lo);
-      }
+      warp_pair_sum(sq, sq_lo);
       float2* red = bars->red[it & 1];
       if (lane == 0) red[warp - 2] = make_float2(sq, sq_lo);
       // All elementwise warps leave after the same tile: one that stayed would wait on the next tile's barriers.

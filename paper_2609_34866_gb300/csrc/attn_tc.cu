@@ -64,8 +64,8 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
 //   warp 1       TMEM owner, tcgen05.cp of Q, UMMA issuer of S (one thread);   warp 15  of P V
 //   warps 2..9   softmax: warp (quarter q, half h) owns the 16 rows at lanes 32 q + 16 h; with the
 //                16x256b TMEM shape four threads share a row (32 of its 128 scores each, two rows per
-//                thread), so row maxima and sums need only warp shuffles. Lazy rescaling as in the
-//                single-head kernel. At the end of a tile the row statistics go to shared memory.
+//                thread), so row maxima and sums need only warp shuffles. Lazy rescaling
+//                (kRescaleLog2). At the end of a tile the row statistics go to shared memory.
 //   warp 10      TMA: V ring (2 stages), so that K loads never queue behind a V stage that is busy
 //   warps 11..14 epilogue, one TMEM lane quarter each (32x32b shape, one row per thread, 32 columns at a
 //                time): A_ref arrives in shared memory by TMA (32 x 32 boxes, two per warp in flight,

@@ -38,12 +38,6 @@ __device__ __forceinline__ bool in_bounds(int64_t last, int64_t extent, int* sta
   return true;
 }
 
-// Non-zero when either half of a packed fp16 pair has every exponent bit set: an infinity (the
-// rounded value was outside the fp16 range) or a NaN. Integer SIMD compare, no FP instructions.
-__device__ __forceinline__ uint32_t half2_exp_all_ones(uint32_t h2) {
-  return __vcmpeq2(h2 & 0x7C007C00u, 0x7C007C00u);
-}
-
 __host__ __device__ __forceinline__ int qmax_of(int bits) { return (1 << (bits - 1)) - 1; }
 
 // Eq. 2 with reading R1: v = fl32(w / s) (IEEE round-to-nearest division), q = clip(rint(v)).
@@ -65,8 +59,8 @@ __device__ __forceinline__ float lsq_factor(float w, float s, int qmax) {
 // fl32(w / s) of several bf16 weights with one scale: with r = fl32(1 / s) and v0 = fl32(w r), the
 // remainder w - v0 s is exact in one fused operation and v0 + r (w - v0 s) rounds to the IEEE quotient
 // (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990).
-// Equal to w / s for every pair of a bf16 and an fp32 mantissa (2^7 x 2^23, checked one by one), and
-// so wherever no intermediate leaves the normal range: s within 2^-60 .. 2^60, |w| within 2^-90 ..
+// Equal to w / s for every pair of a bf16 and an fp32 mantissa (2^7 x 2^23, one by one in
+// tests/test_quotient_cpu.py), and so wherever no intermediate leaves the normal range: s within 2^-60 .. 2^60, |w| within 2^-90 ..
 // 2^60 or 0 (below 2^-90 the quotient is less than 2^-30 and its code 0 either way). Other values take
 // the division. Three operations a weight, in packed pairs, where the division takes about ten.
 __device__ __forceinline__ bool quot_window(float s) { return s >= 8.6736174e-19f && s <= 1.1529215e18f; }
@@ -161,7 +155,7 @@ struct FastDiv {
 // visible, and whatever it read may be overwritten; only then is the successor let in, so that at most one
 // kernel waits behind the running one and, with all of a grid's tensor memory allocated before, none can take
 // what a block still to be set up needs. The seven kernels of a small fitting step (GPT-2 block, 4 x 128 tokens)
-// take 45.3 us this way; one after the other, each with its launch and its set-up in the open, 61.5 us.
+// take 40.9 us this way; one after the other, each with its launch and its set-up in the open, 56.5 us.
 __device__ __forceinline__ void stream_order() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

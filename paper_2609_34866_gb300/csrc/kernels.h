@@ -57,9 +57,9 @@ cudaError_t launch_init_scales(const void* w, int D, int d, int G, int bits, int
 cudaError_t launch_proj_gemm_tc(const void* A, const void* Bw, void* C, int64_t M, int Nn, int K,
                                 int D, int n_rot, int dh, int T, const float* cos_t,
                                 const float* sin_t, int* status, cudaStream_t st);
-// x: bf16 [N, d] as the caller stores it (no transposed copy)
 // Tiles of 256 columns that a group of G may touch: 1 where whole groups fit a tile.
 int lsq_group_parts(int G);
+// x: bf16 [N, d] as the caller stores it (no transposed copy)
 // dspart: fp32, the scale gradient's partials [*splits, D, d/G]: of every K range (at most kMaxSplits) and,
 // with lsq_group_parts(G) > 1, of every tile of a group
 cudaError_t launch_wgrad_lsq_tc(const void* dqkvt, int64_t ldt, const void* x, const void* w,

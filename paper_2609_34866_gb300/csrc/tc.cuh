@@ -25,11 +25,9 @@ __device__ __forceinline__ uint64_t globaltimer() {
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
 // True in one lane of the (converged) warp. The roles of a single thread branch on this rather than
-// on a lane number: the compiler then knows that one thread runs and issues a tcgen05 or TMA
-// instruction, whose operands are uniform registers, as it stands. After `lane == 0` it cannot know, and
-// each such instruction waits for its operands to be made uniform: four K = 16 UMMAs took 400 clocks to
-// issue that way and 120 this way (GB300; the pipe needs 256 for them), more than any attention
-// kernel's products left room for.
+// on a lane number: four K = 16 UMMAs took 400 clocks to issue behind `lane == 0` and 120 behind this
+// (clock stamps around the issue, GB300; the pipe needs 256 for them), and the attention kernels' products
+// left no room for the former.
 __device__ __forceinline__ bool elect_one() {
   uint32_t ok;
   asm volatile(

@@ -21,7 +21,7 @@ struct Workspace {
   size_t part;     // fp64 [C, B, Hq, nP]    per-tile partial sums (SSE or ||A||^2)
   size_t status;   // int32 [16]             [0]: blocks done of the reduction in flight, else 0
   size_t scal;     // fp64 [2, C]            per-candidate scalars (MSE and KL terms)
-  size_t red;      // fp64 [C, kRedBlocks]   per-block partial sums of the quantisation error
+  size_t red;      // fp64 [C, kRedBlocks]   per-block partial sums: quantisation error, loss, KL value, ||dW||^2
   // backward only
   size_t d_o;      // fp16 [N, Hq*d_h]       e = A_hat - A_ref (dL/dA_hat up to 2/n)
   size_t lse;      // fp32 [B, Hq, Tp]       student log-sum-exp in log2 units (Tp = T rounded to 128)
