@@ -688,8 +688,8 @@ __global__ void __launch_bounds__(DKDV_THREADS, 1)
 // (the next block's products run while the elementwise warps read this one), P^T = exp2(s_t^T sl2 -
 // lse2_t) with the causal mask, the CTA's partial sum of P (s_t - s_s) (and, in the key-block-0 CTAs
 // that see every query row once, of lse^S - lse^T). It writes 32 KB a block, 1.14 GB for 8 x 32 heads of 2048,
-// which take 168 us at the copy rate; the kernel takes some 310 us (363 with P^T staged in shared memory, one
-// tile at a time, and with stages that the elementwise warps held for their log-sum-exp rows). Next to the
+// which take 168 us at the copy rate; the kernel takes 335 us (16 x 2048: 652, and 787 with P^T staged in shared
+// memory, one tile at a time, and with stages that the elementwise warps held for their log-sum-exp rows). Next to the
 // stores, its SS products and the loads of 64 KB a block keep shared memory busy for 1600 of 2500 clocks.
 //   warp 0      TMA: K_t, K_s once; per block Q_t, Q_s and the two rows of lse (log2 units)
 //   warp 1      TMEM owner, UMMA issuer
