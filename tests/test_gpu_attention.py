@@ -120,3 +120,41 @@ def test_three_query_heads_per_kv_head(shape, B, T, bits):
             P.test_backward_kl_parity(name, bits, regime)
     finally:
         del P._cases[name]
+
+
+@pytest.mark.parametrize("shape", [BlockShape(256, 4, 1, 64, True, 500.0), BlockShape(256, 3, 1, 128, False)])
+def test_row_sum_of_do_and_o_is_a_tree(shape):
+    """D = rowsum(dO * O) of the backward, as the call leaves it in its workspace slot: every fp32 rounding in
+    its place (column groups of four, the chunks of 32 columns in order, then a tree over the eight groups).
+    The student's weights are multiples of 2^-6, which bf16 holds, so that a teacher pass on them returns O
+    itself. (The products' sums are rounded by way of float64 here: equal but for double roundings.)"""
+    from dataclasses import replace
+    from tests.harness import Case
+    B, T, dh = 2, 333, shape.head_dim
+    c = Case(replace(WORKLOADS["gpt2_smoke"], shape=shape), B, T, 64)
+    ws = c.workspace()
+    A, _, _ = c.gpu_teacher(ws)
+    s = torch.full((c.D, shape.d_model // 64), 2.0 ** -6, device="cuda")
+    w_hat = (torch.clamp(torch.round(c.W.float() * 64), -3, 3) / 64).to(torch.bfloat16)
+    O = torch.empty_like(A)
+    J().jab_reference_forward(c.desc, B, T, c.X, w_hat, O, ws)
+    loss = torch.empty(1, dtype=torch.float64, device="cuda")
+    J().jab_loss_backward_scales(c.desc, B, T, c.X, c.W, A, 3, s, 1.0, loss, torch.empty_like(s), ws)
+    assert J().jab_get_device_status() == 0
+    N, tp, at = B * T, (T + 127) // 128 * 128, 0  # the slots before D's, in the order of csrc/workspace.h
+    for n in (64, N * shape.d_model * 2, c.D * shape.d_model * 2, N * c.D * 2, T * dh * 4, B * c.Hq * ((T + 63) // 64) * 8,
+              16, 1024 * 8, N * c.Hq * dh * 2, B * c.Hq * tp * 4):
+        at += (n + 255) // 256 * 256
+    d = ws.buf[at:at + B * c.Hq * tp * 4].view(torch.float32).view(B, c.Hq, tp)[..., :T]
+    o = O.view(B, T, c.Hq, dh // 32, 8, 4).cpu()
+    f = (O - A).half().float().view(o.shape).cpu()
+    low = f[..., :2] * o[..., :2]
+    pairs = (f[..., 2:].double() * o[..., 2:].double() + low.double()).float()
+    groups = pairs[..., 0] + pairs[..., 1]
+    t = groups[..., 0, :]
+    for ch in range(1, dh // 32):
+        t = t + groups[..., ch, :]
+    while t.shape[-1] > 1:
+        t = t[..., 0::2] + t[..., 1::2]
+    same = t[..., 0].permute(0, 2, 1) == d.cpu()
+    assert same.float().mean() >= 0.999, same.float().mean()
