@@ -109,23 +109,25 @@ __global__ void check_finite_kernel(const float* __restrict__ x, int64_t n, int*
 
 // Sum of squares: block b sums its contiguous chunk (fixed per-thread order, fixed tree), one block then
 // adds the kRedBlocks partials. The chip runs about two FP64 operations per clock and SM, and a
-// conversion and a multiply-add per value bounded the kernel (101 us for 25M values, now 43): eight squares
-// are added in floats with every rounding error carried along, and only that goes to the fp64 accumulator.
+// conversion and a multiply-add per value bounded the kernel (101 us for 25M values, now 27; 43 with eight
+// values at a time): up to sixteen squares are added in floats with every rounding error carried along, and only
+// that goes to the fp64 accumulator. (Eight blocks to an SM: all kRedBlocks are resident at once.)
 // The products' low parts are a pair of their own: their last bits do not round evenly (an odd
 // square is 1 modulo 8), and with all errors in one float the sum came out 1.1e-15 small. Values whose
 // largest is outside 2^-40 .. 2^60 are squared in fp64. With `status` a non-finite value is reported.
-__device__ __forceinline__ double sumsq8(const float (&v)[8]) {
+template <int N>
+__device__ __forceinline__ double sum_squares(const float (&v)[N]) {
   float big = 0.f;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) big = fmaxf(big, fabsf(v[k]));
+  for (int k = 0; k < N; ++k) big = fmaxf(big, fabsf(v[k]));
   if (!(big >= 9.0949470e-13f && big <= 1.1529215e18f)) {
     double acc = 0.0;
-    for (int k = 0; k < 8; ++k) acc += (double)v[k] * (double)v[k];
+    for (int k = 0; k < N; ++k) acc += (double)v[k] * (double)v[k];
     return acc;
   }
   float sh = 0.f, se = 0.f, sl = 0.f, s3 = 0.f;  // products and their sums' errors, low parts and theirs
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
+  for (int k = 0; k < N; ++k) {
     const float h = __fmul_rn(v[k], v[k]), l = __fmaf_rn(v[k], v[k], -h);
     float t, e;
     two_sum(sh, h, t, e);
@@ -140,7 +142,7 @@ __device__ __forceinline__ double sumsq8(const float (&v)[8]) {
   return (double)sh + ((double)a + (double)__fadd_rn(b, s3));
 }
 
-__global__ void __launch_bounds__(256) sumsq_partial_kernel(const float* __restrict__ x, int64_t n,
+__global__ void __launch_bounds__(256, 8) sumsq_partial_kernel(const float* __restrict__ x, int64_t n,
                                                             double* __restrict__ part, int* status) {
   __shared__ double red[8];
   const int64_t n8 = n / 8;  // n is a multiple of 64 (rows of a weight)
@@ -148,10 +150,17 @@ __global__ void __launch_bounds__(256) sumsq_partial_kernel(const float* __restr
   const int64_t lo = blockIdx.x * chunk, hi = lo + chunk < n8 ? lo + chunk : n8;
   const float4* x4 = reinterpret_cast<const float4*>(x);
   double acc = 0.0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+  int64_t i = lo + threadIdx.x;
+  for (; i + blockDim.x < hi; i += 2 * blockDim.x) {
+    const float4 a = x4[2 * i], b = x4[2 * i + 1];
+    const float4 c = x4[2 * (i + blockDim.x)], d = x4[2 * (i + blockDim.x) + 1];
+    const float v[16] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, d.x, d.y, d.z, d.w};
+    acc += sum_squares(v);
+  }
+  if (i < hi) {
     const float4 a = x4[2 * i], b = x4[2 * i + 1];
     const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    acc += sumsq8(v);
+    acc += sum_squares(v);
   }
   const double t = block_sum<256>(acc, red);
   if (threadIdx.x == 0) {
